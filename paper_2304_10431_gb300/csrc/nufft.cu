@@ -1,59 +1,18 @@
-// Non-uniform FFT steps (Sect. 3 "NUFFT": type 2 for the forward operator,
-// type 1 for the adjoint) on the oversampled torus grid.
-//
-// Kernel: exponential of semicircle, psi(z) = exp(beta (sqrt(1 - (2z/W)^2) - 1))
-// for |z| < W/2 (grid units), zero outside.  A point at grid coordinates
-// (u, v) = (theta N1 / 2pi, phi N2 / 2pi) touches the W x W cells
-// i0 + a, j0 + b with i0 = ceil(u - W/2), j0 = ceil(v - W/2), a, b < W:
-//   type 2:  f = sum_ab psi(u - i0 - a) psi(v - j0 - b) g[i0 + a, j0 + b]
-//   type 1:  g[i0 + a, j0 + b] += psi(u - i0 - a) psi(v - j0 - b) f
-// The two use the same weights, so they are exact transposes.
-//
-// Points are prepared once per plan (Sect. 4: the geometry is reused): cell
-// offset into the row-padded grid, fractional offsets (u - i0, v - j0) from
-// FP64 coordinates, the spin phase e^{i s chi}, a permutation that sorts
-// points by 32 x 32 grid tiles (of the first tap) so that neighbouring
-// threads share grid rows, and the first sorted point of every tile.
-// Interpolation runs one thread per sorted point and reads its W x W taps
-// through L1: sorted neighbours share rows, so the tile stays cached (staging
-// the tile and its halo in shared memory first measured 1.36x slower for
-// spin 0 at lmax 4096).  Spreading in FP32 runs one CTA per tile: its points
-// add their W x W taps into the tile and its halo, (32 + W - 1) x (32 + W - 1)
-// cells held in shared memory, and the CTA then adds the non-zero cells into
-// the grid with one global atomic each.  FP64
-// plans spread with one global atomic per tap instead: the L2 adds doubles
-// natively, while double additions into shared memory measured 1.9x (spin s)
-// to 2.4x (spin 0) slower at lmax 4096.
-//
-// Deterministic plans (LENS_DETERMINISTIC) spread in 64-bit fixed point: every
-// tap value is scaled by a power of two 2^k and rounded to an integer, and the
-// shared-memory and global atomics add integers, exactly and so in any order.
-// k is chosen per call so that no cell can exceed 2^62: a cell receives at
-// most Kmax points (the largest point count of a tile and its left, upper and
-// upper-left neighbours, whose taps are the only ones that reach it), each
-// contributing |x| psi psi <= max |x|.  A conversion pass then writes the
-// grid in the plan's precision.
+// Point preparation of the non-uniform FFT steps, the fixed-point scalars of a call and the entry points of
+// interpolation and spreading; the kernels themselves are in nufft.cuh, compiled per precision in
+// nufft_f32.cu, nufft_interp64.cu and nufft_spread64.cu.
 #include <cuda_runtime.h>
 #include <math.h>
 
-#include <type_traits>
-
 #include <cub/cub.cuh>
 
-#include "common.cuh"
-#include "internal.h"
+#include "nufft.cuh"
 
 namespace gsl {
 namespace {
 
 constexpr double kTwoPi = 6.283185307179586476925286766559;
 constexpr double kPi = 3.141592653589793238462643383280;
-constexpr int kSpreadThreads = 64;
-// FP64 tiles hold 64-bit cells (31 KB at W = 13, seven CTAs per SM): 256 threads keep
-// more warps in flight per tile
-constexpr int kSpreadThreads64 = 256;
-// FP64 double-float spreading tiles stage this many points at a time (offset + value pair)
-constexpr int kDDBatch = 512;
 
 // Grid coordinate u = t c with c = N / (2 pi) held as a double-double (c.x +
 // c.y): the product's rounding error, ~1e-16 of u (up to N/2 ~ 10^4 cells),
@@ -141,32 +100,6 @@ __global__ void k_tile_bounds(const uint32_t *__restrict__ skey, int64_t n, int 
     for (int64_t t = lo + 1; t <= hi; ++t) start[t] = (uint32_t)p;
 }
 
-// the ES kernel of tap offset z (FP64 plans)
-template <typename T> __device__ __forceinline__ T es_kernel(T z, T twoW, T beta)
-{
-    const T t = z * twoW;
-    const T q = T(1) - t * t;
-    return q > T(0) ? exp(beta * (sqrt(q) - T(1))) : T(0);
-}
-
-// FP32 plans: the kernel weight of tap a by Horner's rule in t = 2 frac - (W - 1) from the plan's
-// polynomial coefficients (W + 1 fused multiply-adds; interpolation and spreading read the same
-// coefficients, so the pair stay exact transposes of each other)
-template <int W> __device__ __forceinline__ float ker_poly(const KerPoly &kp, int a, float t)
-{
-    float acc = kp.c[a * (W + 2) + W + 1];
-#pragma unroll
-    for (int k = W; k >= 0; --k) acc = fmaf(acc, t, kp.c[a * (W + 2) + k]);
-    return acc;
-}
-
-// fixed-point term: v 2^k (exact, 2^k a power of two) rounded to an integer
-__device__ __forceinline__ unsigned long long to_fx(float v, float sc) { return (unsigned long long)__float2ll_rn(v * sc); }
-__device__ __forceinline__ unsigned long long to_fx(double v, double sc)
-{
-    return (unsigned long long)__double2ll_rn(v * sc);
-}
-
 // FP64 plans' 2W kernel weights of every (sorted) point, computed once, evaluated in FP64 and kept as
 // doubles or (dd, plans with epsilon >= 5e-11) as double-float pairs (8 bytes
 // each either way): the latter plans compute the interpolation and spreading
@@ -190,419 +123,6 @@ __global__ void k_weights(const double2 *__restrict__ frac, int64_t n, int W, do
         } else {
             wd[a] = x;
             wd[W + a] = y;
-        }
-    }
-}
-
-__device__ __forceinline__ df32 ld_df(const float2 *p)
-{
-    const float2 v = __ldg(p);
-    return {v.x, v.y};
-}
-
-// PRE: 0 evaluate the kernel, 1 read the double weights, 2 the double-float pairs
-template <typename T, int W, int PRE>
-__device__ __forceinline__ void tap_weights(T (&wa)[W], T (&wb)[W], const cplx<T> &f, const double *wts, int64_t p,
-                                            T beta, const KerPoly &kp)
-{
-    if (PRE == 1) {
-        const double *w = wts + p * 2 * W;
-#pragma unroll
-        for (int a = 0; a < W; ++a) {
-            wa[a] = (T)__ldg(w + a);
-            wb[a] = (T)__ldg(w + W + a);
-        }
-    } else if (PRE == 2) {
-        const float2 *w = reinterpret_cast<const float2 *>(wts) + p * 2 * W;
-#pragma unroll
-        for (int a = 0; a < W; ++a) {
-            wa[a] = (T)df_value(ld_df(w + a));
-            wb[a] = (T)df_value(ld_df(w + W + a));
-        }
-    } else if constexpr (std::is_same<T, float>::value) {
-        const float tx = fmaf(2.f, f.x, -(float)(W - 1)), ty = fmaf(2.f, f.y, -(float)(W - 1));
-#pragma unroll
-        for (int a = 0; a < W; ++a) {
-            wa[a] = ker_poly<W>(kp, a, tx);
-            wb[a] = ker_poly<W>(kp, a, ty);
-        }
-    } else {
-        const T twoW = T(2) / T(W);
-#pragma unroll
-        for (int a = 0; a < W; ++a) {
-            wa[a] = es_kernel<T>(f.x - T(a), twoW, beta);
-            wb[a] = es_kernel<T>(f.y - T(a), twoW, beta);
-        }
-    }
-}
-
-template <typename T, int W, bool SPIN, int PRE>
-__global__ void __launch_bounds__(256) k_interp(const void *__restrict__ grid, const uint32_t *__restrict__ cell,
-                                                const cplx<T> *__restrict__ frac, const int32_t *__restrict__ perm,
-                                                const cplx<T> *__restrict__ phase, const double *__restrict__ wts,
-                                                T *__restrict__ map, int64_t n, int pitch, T beta,
-                                                const __grid_constant__ KerPoly kp)
-{
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const uint32_t c0 = cell[p];
-    T wa[W], wb[W];
-    tap_weights<T, W, PRE>(wa, wb, PRE ? cplx<T>{} : frac[p], wts, p, beta, kp);
-    const int32_t dst = perm[p];
-    if (!SPIN) {
-        const T *g = (const T *)grid + c0;
-        T acc = T(0);
-#pragma unroll
-        for (int a = 0; a < W; ++a) {
-            T r = T(0);
-#pragma unroll
-            for (int b = 0; b < W; ++b) r += wb[b] * __ldg(g + (int64_t)a * pitch + b);
-            acc += wa[a] * r;
-        }
-        map[dst] = acc;
-    } else {
-        const cplx<T> *g = (const cplx<T> *)grid + c0;
-        T ax = T(0), ay = T(0);
-#pragma unroll
-        for (int a = 0; a < W; ++a) {
-            T rx = T(0), ry = T(0);
-#pragma unroll
-            for (int b = 0; b < W; ++b) {
-                const cplx<T> v = __ldg(g + (int64_t)a * pitch + b);
-                rx += wb[b] * v.x;
-                ry += wb[b] * v.y;
-            }
-            ax += wa[a] * rx;
-            ay += wa[a] * ry;
-        }
-        const cplx<T> ph = phase[p];
-        map[dst] = ax * ph.x - ay * ph.y;
-        map[n + dst] = ax * ph.y + ay * ph.x;
-    }
-}
-
-// FP64 plans with point weights: the same sums in double-float arithmetic on
-// the FP32 pipe.  The grid holds double-float pairs (k_phi_fwd writes them
-// for these plans: float2 per real, spin s float4 (re h, re l, im h, im l));
-// each row sum adds the exact products of the high words with two-sum and
-// the products' error terms and cross terms in the low word, then the rows
-// are combined the same way; ~2^-46 relative per term.
-template <int W, bool SPIN>
-__global__ void __launch_bounds__(256) k_interp_dd(const void *__restrict__ grid, const uint32_t *__restrict__ cell,
-                                                   const int32_t *__restrict__ perm, const double2 *__restrict__ phase,
-                                                   const double *__restrict__ wts, double *__restrict__ map,
-                                                   int64_t n, int pitch)
-{
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const uint32_t c0 = cell[p];
-    const float2 *w = reinterpret_cast<const float2 *>(wts) + p * 2 * W;
-    df32 wb[W];
-#pragma unroll
-    for (int b = 0; b < W; ++b) wb[b] = ld_df(w + W + b);
-    const int32_t dst = perm[p];
-    if (!SPIN) {
-        const float2 *g = reinterpret_cast<const float2 *>(grid) + c0;
-        df32 acc = {0.f, 0.f};
-#pragma unroll
-        for (int a = 0; a < W; ++a) {
-            df32 r = {0.f, 0.f};
-#pragma unroll
-            for (int b = 0; b < W; ++b) df_acc(r, df_mul(wb[b], ld_df(g + (int64_t)a * pitch + b)));
-            df_acc(acc, df_mul(ld_df(w + a), df_renorm(r)));
-        }
-        map[dst] = df_value(acc);
-    } else {
-        const float4 *g = reinterpret_cast<const float4 *>(grid) + c0;
-        df32 ax = {0.f, 0.f}, ay = {0.f, 0.f};
-#pragma unroll
-        for (int a = 0; a < W; ++a) {
-            df32 rx = {0.f, 0.f}, ry = {0.f, 0.f};
-#pragma unroll
-            for (int b = 0; b < W; ++b) {
-                const float4 v = __ldg(g + (int64_t)a * pitch + b);
-                df_acc(rx, df_mul(wb[b], df32{v.x, v.y}));
-                df_acc(ry, df_mul(wb[b], df32{v.z, v.w}));
-            }
-            const df32 wa = ld_df(w + a);
-            df_acc(ax, df_mul(wa, df_renorm(rx)));
-            df_acc(ay, df_mul(wa, df_renorm(ry)));
-        }
-        const double2 ph = phase[p];
-        const double x = df_value(ax), y = df_value(ay);
-        map[dst] = x * ph.x - y * ph.y;
-        map[n + dst] = x * ph.y + y * ph.x;
-    }
-}
-
-// one thread per sorted point, one global atomic per tap (FP64 plans); FX:
-// fixed-point integers into the same grid memory (scale *fxs)
-template <typename T, bool FX> struct Acc {
-    using type = T;
-};
-template <typename T> struct Acc<T, true> {
-    using type = unsigned long long;
-};
-template <typename T, bool FX>
-__device__ __forceinline__ void acc_add(typename Acc<T, FX>::type *dst, T v, T sc)
-{
-    if constexpr (FX) atomicAdd(dst, to_fx(v, sc));
-    else atomicAdd(dst, v);
-}
-
-template <typename T, int W, bool SPIN, int PRE, bool FX>
-__global__ void __launch_bounds__(256) k_spread_direct(void *__restrict__ grid, const uint32_t *__restrict__ cell,
-                                                       const cplx<T> *__restrict__ frac,
-                                                       const int32_t *__restrict__ perm,
-                                                       const cplx<T> *__restrict__ phase,
-                                                       const double *__restrict__ wts, const T *__restrict__ map,
-                                                       int64_t n, int pitch, T beta, const double *__restrict__ fxs,
-                                                       const __grid_constant__ KerPoly kp)
-{
-    using G = typename Acc<T, FX>::type;
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const T sc = FX ? (T)fxs[0] : T(1);
-    const uint32_t c0 = cell[p];
-    T wa[W], wb[W];
-    tap_weights<T, W, PRE>(wa, wb, PRE ? cplx<T>{} : frac[p], wts, p, beta, kp);
-    const int32_t src = perm[p];
-    if (!SPIN) {
-        const T x = map[src];
-        G *g = (G *)grid + c0;
-#pragma unroll
-        for (int a = 0; a < W; ++a) {
-            const T xa = wa[a] * x;
-#pragma unroll
-            for (int b = 0; b < W; ++b) acc_add<T, FX>(g + (int64_t)a * pitch + b, xa * wb[b], sc);
-        }
-    } else {
-        // e^{-i s chi} (Q + i U)
-        const cplx<T> ph = phase[p];
-        const T q = map[src], u = map[n + src];
-        const T zx = ph.x * q + ph.y * u, zy = ph.x * u - ph.y * q;
-        G *g = (G *)grid + 2 * (int64_t)c0;
-#pragma unroll
-        for (int a = 0; a < W; ++a) {
-            const T xa = wa[a] * zx, ya = wa[a] * zy;
-#pragma unroll
-            for (int b = 0; b < W; ++b) {
-                G *q2 = g + 2 * ((int64_t)a * pitch + b);
-                acc_add<T, FX>(q2, xa * wb[b], sc);
-                acc_add<T, FX>(q2 + 1, ya * wb[b], sc);
-            }
-        }
-    }
-}
-
-// FX: fixed-point integers in shared memory and in the grid (scale *fxs).
-// IT (integer tiles; FP32 plans at epsilon >= 1e-5 and FP64 plans, not FX):
-// the tile accumulates in fixed point in shared memory, 32-bit integers for
-// FP32 plans (integer atomics there run ~3x the rate of float atomics) and
-// 64-bit for FP64 plans (no FP64 atomics in the inner loop), in units of 1/u
-// with u = 2^k per tile, k the largest integer with kmax_t max|x| u <= 2^30
-// (FP64: 2^62): kmax_t (plan time) is the most of the tile's points whose
-// W x W windows cover one cell and max|x| (per call) the map's largest |value|
-// (|Q| + |U| for spin s), taps |psi| <= 1, so no cell sum can overflow.  Every
-// term is rounded once (to 2^-k; FP64: relative 2^-62 of the tile's bound);
-// the flush converts back for one global atomic per non-zero cell.  A map
-// with a non-finite value makes the whole tile NaN.
-template <typename T, bool FX, bool IT> struct SAcc { using type = typename Acc<T, FX>::type; };
-template <> struct SAcc<float, false, true> { using type = int; };
-template <> struct SAcc<double, false, true> { using type = long long; };
-__device__ __forceinline__ int tile_int(float v) { return __float2int_rn(v); }
-// A double-float term (p, e) with |p| < 2^53 as a 64-bit integer (nearest) without
-// 64-bit conversions (those run at GB300's FP64 rate): p = p1 + p2 with p1 a multiple
-// of 2^31 (|p1| / 2^31 < 2^22, read off the bits of p1 / 2^31 + 1.5 * 2^23) and
-// |p2| <= 2^30 exact, then p2 and e by 32-bit conversions
-__device__ __forceinline__ long long dd_tile_int(df32 t)
-{
-    const float big = 0x1.8p54f;  // 1.5 * 2^54: t.h + big rounds t.h to a multiple of 2^31
-    const float p1 = __fsub_rn(__fadd_rn(t.h, big), big);
-    const int i1 = __float_as_int(__fmaf_rn(p1, 0x1p-31f, 12582912.0f)) - 0x4B400000;
-    const float p2 = __fsub_rn(t.h, p1);
-    return ((long long)i1 << 31) + (long long)__float2int_rn(p2) + (long long)__float2int_rn(t.l);
-}
-__device__ __forceinline__ long long tile_int(double v) { return __double2ll_rn(v); }
-__device__ __forceinline__ void tile_add(int *dst, int v) { atomicAdd(dst, v); }
-__device__ __forceinline__ void tile_add(long long *dst, long long v)
-{
-    atomicAdd(reinterpret_cast<unsigned long long *>(dst), (unsigned long long)v);  // two's complement sum
-}
-
-template <typename T, int W, bool SPIN, int PRE, bool FX, bool IT = false>
-__global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThreads) k_spread(void *__restrict__ grid, const uint32_t *__restrict__ cell,
-                                                           const cplx<T> *__restrict__ frac,
-                                                           const int32_t *__restrict__ perm,
-                                                           const cplx<T> *__restrict__ phase,
-                                                           const double *__restrict__ wts, const T *__restrict__ map,
-                                                           int64_t n, int pitch, int R, int ntc,
-                                                           const uint32_t *__restrict__ tile_start, T beta,
-                                                           const double *__restrict__ fxs,
-                                                           int tile_r, const unsigned short *__restrict__ tile_kmax,
-                                                           const unsigned long long *__restrict__ maxbits,
-                                                           const __grid_constant__ KerPoly kp)
-{
-    static_assert(!(IT && FX), "fixed-point tiles or fixed-point grid");
-    using G = typename SAcc<T, FX, IT>::type;
-    constexpr bool DD = std::is_same<T, double>::value && IT && PRE == 2;  // double-float taps
-    constexpr int TC = kTileC + W - 1, NC = SPIN ? 2 : 1;
-    const int TR = tile_r + W - 1;  // tile rows (16, 32 or 64) plus the kernel halo
-    extern __shared__ __align__(16) unsigned char spread_smem[];
-    G *buf = reinterpret_cast<G *>(spread_smem);  // TR x TC cells x NC planes
-    const int t = blockIdx.x;
-    const uint32_t p0 = tile_start[t], p1 = tile_start[t + 1];
-    if (p0 == p1) return;
-    T sc = FX ? (T)fxs[0] : T(1);
-    bool bad = false;  // IT: non-finite map value
-    if constexpr (IT) {
-        constexpr int kBits = sizeof(T) == 4 ? 30 : DD ? 53 : 62;  // tile sums of |terms| below 2^kBits
-        const double bound = (double)tile_kmax[t] * __longlong_as_double((long long)*maxbits);
-        if (!(bound < 1e300)) bad = true;  // infinity or NaN in the map
-        else if (bound > 0.0) sc = (T)ldexp(1.0, kBits - (ilogb(bound) + 1));  // bound < 2^(ilogb+1)
-    }
-    for (int i = threadIdx.x; i < TR * TC * NC; i += blockDim.x) buf[i] = G(0);
-    __syncthreads();
-    const int r0 = (t / ntc) * tile_r, c0 = (t % ntc) * kTileC;
-    if constexpr (DD && SPIN) {
-        // FP64 plans with point weights, spin s: work items (point, kernel row) instead of points, so
-        // that the threads of a tile finish together (a tile holds 2-3 points per thread, and
-        // one point per thread more meant a wait at the barrier) and the unrolled body is one
-        // row of W taps.  Per batch of points: each point's value times the unit (exact) as a
-        // double-float pair and its cell offset in shared memory; then the items.  Each tap is
-        // the double-float product of the row value and the weight pair (~2^-46 relative),
-        // rounded to an integer by dd_tile_int (tile sums of |terms| below 2^53).
-        int *soff = reinterpret_cast<int *>(buf + ((TR * TC * NC + 1) & ~1));  // 16-byte aligned
-        float4 *sval = reinterpret_cast<float4 *>(soff + kDDBatch);
-        for (uint32_t pb = p0; pb < (bad ? p0 : p1); pb += kDDBatch) {
-            const int nb = (int)min((uint32_t)kDDBatch, p1 - pb);
-            for (int q = threadIdx.x; q < nb; q += blockDim.x) {
-                const uint32_t p = pb + q;
-                const uint32_t c = cell[p];
-                const int lr = (int)(c / (uint32_t)pitch) - r0, lc = (int)(c % (uint32_t)pitch) - c0;
-                const bool mine = (unsigned)lr < (unsigned)tile_r && (unsigned)lc < (unsigned)kTileC;
-                soff[q] = mine ? lr * TC + lc : -1;
-                if (!mine) continue;
-                const int32_t src = perm[p];
-                const cplx<T> ph = phase[p];
-                const T qv = map[src], u = map[n + src];
-                const df32 zx = df_split((ph.x * qv + ph.y * u) * sc), zy = df_split((ph.x * u - ph.y * qv) * sc);
-                sval[q] = make_float4(zx.h, zx.l, zy.h, zy.l);
-            }
-            __syncthreads();
-            for (int it = threadIdx.x; it < nb * W; it += blockDim.x) {
-                const int q = it / W, a = it - q * W;
-                const int off = soff[q];
-                if (off < 0) continue;
-                const float2 *w = reinterpret_cast<const float2 *>(wts) + (int64_t)(pb + q) * 2 * W;
-                const df32 wa = ld_df(w + a);
-                const float4 v = sval[q];
-                G *row = buf + off + a * TC;
-                const df32 xa = df_renorm(df_mul(wa, df32{v.x, v.y})), ya = df_renorm(df_mul(wa, df32{v.z, v.w}));
-#pragma unroll
-                for (int b = 0; b < W; ++b) {
-                    const df32 wb = ld_df(w + W + b);
-                    tile_add(row + b, dd_tile_int(df_mul(xa, wb)));
-                    tile_add(row + b + TR * TC, dd_tile_int(df_mul(ya, wb)));
-                }
-            }
-            __syncthreads();  // the batch's staging is rewritten next
-        }
-    }
-    for (uint32_t p = p0 + threadIdx.x; p < ((bad || (DD && SPIN)) ? p0 : p1); p += blockDim.x) {
-        const uint32_t c = cell[p];
-        const int lr = (int)(c / (uint32_t)pitch) - r0, lc = (int)(c % (uint32_t)pitch) - c0;
-        if ((unsigned)lr >= (unsigned)tile_r || (unsigned)lc >= (unsigned)kTileC) continue;  // not this tile's
-        const int32_t src = perm[p];
-        // spin s: two planes (real parts, then imaginary parts), so that the lanes'
-        // atomics of one plane spread over all 32 banks
-        G *b0 = buf + (lr * TC + lc);
-        if constexpr (DD && !SPIN) {
-            // FP64 plans with point weights, spin 0: the value (times the unit, exact) as a
-            // double-float pair, each tap the double-float product with the pair of weights
-            // (~2^-46 relative), rounded to an integer by dd_tile_int (tile sums of |terms|
-            // below 2^53)
-            const float2 *w = reinterpret_cast<const float2 *>(wts) + (int64_t)p * 2 * W;
-            df32 wb[W];
-#pragma unroll
-            for (int b = 0; b < W; ++b) wb[b] = ld_df(w + W + b);
-            const df32 x = df_split(map[src] * sc);
-#pragma unroll
-            for (int a = 0; a < W; ++a) {
-                const df32 xa = df_renorm(df_mul(ld_df(w + a), x));
-#pragma unroll
-                for (int b = 0; b < W; ++b) tile_add(b0 + a * TC + b, dd_tile_int(df_mul(xa, wb[b])));
-            }
-            continue;
-        }
-        T wa[W], wb[W];
-        tap_weights<T, W, PRE>(wa, wb, PRE ? cplx<T>{} : frac[p], wts, p, beta, kp);
-        // IT: the power-of-two unit sc is applied to the point's value first (exact)
-        if (!SPIN) {
-            const T x = IT ? map[src] * sc : map[src];
-#pragma unroll
-            for (int a = 0; a < W; ++a) {
-                const T xa = wa[a] * x;
-#pragma unroll
-                for (int b = 0; b < W; ++b) {
-                    if constexpr (IT) tile_add(b0 + a * TC + b, tile_int(xa * wb[b]));
-                    else acc_add<T, FX>(b0 + a * TC + b, xa * wb[b], sc);
-                }
-            }
-        } else {
-            // e^{-i s chi} (Q + i U)
-            const cplx<T> ph = phase[p];
-            const T q = map[src], u = map[n + src];
-            T zx = ph.x * q + ph.y * u, zy = ph.x * u - ph.y * q;
-            if constexpr (IT) { zx *= sc; zy *= sc; }
-#pragma unroll
-            for (int a = 0; a < W; ++a) {
-                const T xa = wa[a] * zx, ya = wa[a] * zy;
-#pragma unroll
-                for (int b = 0; b < W; ++b) {
-                    G *q2 = b0 + (a * TC + b);
-                    if constexpr (IT) {
-                        tile_add(q2, tile_int(xa * wb[b]));
-                        tile_add(q2 + TR * TC, tile_int(ya * wb[b]));
-                    } else {
-                        acc_add<T, FX>(q2, xa * wb[b], sc);
-                        acc_add<T, FX>(q2 + TR * TC, ya * wb[b], sc);
-                    }
-                }
-            }
-        }
-    }
-    __syncthreads();
-    if constexpr (IT) {
-        T *g = (T *)grid;
-        const T inv = bad ? T(NAN) : T(1) / sc;
-        for (int i = threadIdx.x; i < TR * TC; i += blockDim.x) {
-            const int gr = r0 + i / TC, gc = c0 + i % TC;
-            if (gr >= R || gc >= pitch) continue;
-            const int64_t o = (int64_t)gr * pitch + gc;
-            if (!SPIN) {
-                const G v = buf[i];
-                if (v != 0 || bad) atomicAdd(g + o, (T)v * inv);
-            } else {
-                const G vx = buf[i], vy = buf[TR * TC + i];
-                if (vx != 0 || bad) atomicAdd(g + 2 * o, (T)vx * inv);
-                if (vy != 0 || bad) atomicAdd(g + 2 * o + 1, (T)vy * inv);
-            }
-        }
-    } else {
-        G *g = (G *)grid;
-        for (int i = threadIdx.x; i < TR * TC; i += blockDim.x) {
-            const int gr = r0 + i / TC, gc = c0 + i % TC;
-            if (gr >= R || gc >= pitch) continue;
-            const int64_t o = (int64_t)gr * pitch + gc;
-            if (!SPIN) {
-                const G v = buf[i];
-                if (v != G(0)) atomicAdd(g + o, v);
-            } else {
-                const G vx = buf[i], vy = buf[TR * TC + i];
-                if (vx != G(0)) atomicAdd(g + 2 * o, vx);
-                if (vy != G(0)) atomicAdd(g + 2 * o + 1, vy);
-            }
         }
     }
 }
@@ -707,133 +227,17 @@ __global__ void k_tile_kmax(const uint32_t *__restrict__ start, int ntr, int ntc
     atomicMax(kmax, cnt(tr, tc) + cnt(tr, tc - 1) + cnt(tr - 1, tc) + cnt(tr - 1, tc - 1));
 }
 
-template <typename T, bool SPIN, int W>
-cudaError_t interp_w(const Plan &p, const void *grid, void *map, cudaStream_t st)
-{
-    const int thr = 256;
-    const int64_t blocks = (p.npts + thr - 1) / thr;
-    if (blocks == 0) return cudaSuccess;
-    const auto run = [&](auto kern) {
-        kern<<<(unsigned)blocks, thr, 0, st>>>(grid, p.cell, (const cplx<T> *)p.frac, p.perm, (const cplx<T> *)p.phase,
-                                               p.wts, (T *)map, p.npts, p.pitch, (T)p.beta, p.kpoly);
-        return cudaGetLastError();
-    };
-    if constexpr (std::is_same<T, double>::value) {
-        if (p.wts && p.wts_dd) {  // double-float taps on the double-float grid k_phi_fwd wrote
-            k_interp_dd<W, SPIN><<<(unsigned)blocks, thr, 0, st>>>(grid, p.cell, p.perm, (const double2 *)p.phase,
-                                                                   p.wts, (double *)map, p.npts, p.pitch);
-            return cudaGetLastError();
-        }
-        if (p.wts) return run(k_interp<T, W, SPIN, 1>);
-    }
-    return run(k_interp<T, W, SPIN, 0>);
-}
-
-template <typename T, bool SPIN, int W>
-cudaError_t spread_w(const Plan &p, const void *map, void *grid, cudaStream_t st)
-{
-    if (p.npts == 0) return cudaSuccess;
-    const double *fxs = p.fx_scale;
-    const size_t cells = (size_t)(p.tile_r + W - 1) * (kTileC + W - 1) * (SPIN ? 2 : 1);
-    const auto run = [&](auto kern, size_t esz) {
-        const size_t sm = cells * esz;
-        cudaError_t e2 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e2 != cudaSuccess) return e2;
-        kern<<<(unsigned)p.ntiles, sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThreads, sm, st>>>(
-            grid, p.cell, (const cplx<T> *)p.frac, p.perm, (const cplx<T> *)p.phase, p.wts, (const T *)map, p.npts,
-            p.pitch, p.R, p.ntile_c, p.tile_start, (T)p.beta, fxs, p.tile_r, p.tile_kmax, p.maxbits, p.kpoly);
-        return cudaGetLastError();
-    };
-    if constexpr (std::is_same<T, double>::value) {
-        if (!p.det && p.tile_kmax) {  // 64-bit integer tiles (double-float taps with double-float weights)
-            if (p.wts && p.wts_dd && SPIN) {  // plus the staged points: int offset and float4 value each
-                const size_t extra = (size_t)kDDBatch * (sizeof(int) + sizeof(float4));
-                const auto kern = k_spread<T, W, SPIN, 2, false, true>;
-                const size_t sm = ((cells + 1) & ~(size_t)1) * 8 + extra;
-                cudaError_t e2 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-                if (e2 != cudaSuccess) return e2;
-                kern<<<(unsigned)p.ntiles, kSpreadThreads64, sm, st>>>(
-                    grid, p.cell, (const cplx<T> *)p.frac, p.perm, (const cplx<T> *)p.phase, p.wts, (const T *)map,
-                    p.npts, p.pitch, p.R, p.ntile_c, p.tile_start, (T)p.beta, fxs, p.tile_r, p.tile_kmax, p.maxbits,
-                    p.kpoly);
-                return cudaGetLastError();
-            }
-            if (p.wts && p.wts_dd) return run(k_spread<T, W, SPIN, 2, false, true>, 8);
-            if (p.wts) return run(k_spread<T, W, SPIN, 1, false, true>, 8);
-            return run(k_spread<T, W, SPIN, 0, false, true>, 8);
-        }
-        const unsigned blocks = (unsigned)((p.npts + 255) / 256);
-        const cplx<T> *fr = (const cplx<T> *)p.frac, *ph = (const cplx<T> *)p.phase;
-        const auto direct = [&](auto kern) {
-            kern<<<blocks, 256, 0, st>>>(grid, p.cell, fr, p.perm, ph, p.wts, (const T *)map, p.npts, p.pitch,
-                                         (T)p.beta, fxs, p.kpoly);
-            return cudaGetLastError();
-        };
-        if (p.det) {
-            if (p.wts) return p.wts_dd ? direct(k_spread_direct<T, W, SPIN, 2, true>)
-                                       : direct(k_spread_direct<T, W, SPIN, 1, true>);
-            return direct(k_spread_direct<T, W, SPIN, 0, true>);
-        }
-        if (p.wts) return p.wts_dd ? direct(k_spread_direct<T, W, SPIN, 2, false>)
-                                   : direct(k_spread_direct<T, W, SPIN, 1, false>);
-        return direct(k_spread_direct<T, W, SPIN, 0, false>);
-    } else {
-        if (p.det) return run(k_spread<T, W, SPIN, 0, true>, 8);
-        if (p.tile_kmax) return run(k_spread<T, W, SPIN, 0, false, true>, 4);
-        return run(k_spread<T, W, SPIN, 0, false>, sizeof(T));
-    }
-    return cudaGetLastError();
-}
-
-template <typename T, bool SPIN>
-cudaError_t interp_dispatch(const Plan &p, const void *grid, void *map, cudaStream_t st)
-{
-    switch (p.W) {
-    case 4: return interp_w<T, SPIN, 4>(p, grid, map, st);
-    case 5: return interp_w<T, SPIN, 5>(p, grid, map, st);
-    case 6: return interp_w<T, SPIN, 6>(p, grid, map, st);
-    case 7: return interp_w<T, SPIN, 7>(p, grid, map, st);
-    case 8: return interp_w<T, SPIN, 8>(p, grid, map, st);
-    case 9: return interp_w<T, SPIN, 9>(p, grid, map, st);
-    case 10: return interp_w<T, SPIN, 10>(p, grid, map, st);
-    case 11: return interp_w<T, SPIN, 11>(p, grid, map, st);
-    case 12: return interp_w<T, SPIN, 12>(p, grid, map, st);
-    case 13: return interp_w<T, SPIN, 13>(p, grid, map, st);
-    case 14: return interp_w<T, SPIN, 14>(p, grid, map, st);
-    case 15: return interp_w<T, SPIN, 15>(p, grid, map, st);
-    case 16: return interp_w<T, SPIN, 16>(p, grid, map, st);
-    default: return cudaErrorInvalidValue;
-    }
-}
-
-template <typename T, bool SPIN>
-cudaError_t spread_dispatch(const Plan &p, const void *map, void *grid, cudaStream_t st)
-{
-    switch (p.W) {
-    case 4: return spread_w<T, SPIN, 4>(p, map, grid, st);
-    case 5: return spread_w<T, SPIN, 5>(p, map, grid, st);
-    case 6: return spread_w<T, SPIN, 6>(p, map, grid, st);
-    case 7: return spread_w<T, SPIN, 7>(p, map, grid, st);
-    case 8: return spread_w<T, SPIN, 8>(p, map, grid, st);
-    case 9: return spread_w<T, SPIN, 9>(p, map, grid, st);
-    case 10: return spread_w<T, SPIN, 10>(p, map, grid, st);
-    case 11: return spread_w<T, SPIN, 11>(p, map, grid, st);
-    case 12: return spread_w<T, SPIN, 12>(p, map, grid, st);
-    case 13: return spread_w<T, SPIN, 13>(p, map, grid, st);
-    case 14: return spread_w<T, SPIN, 14>(p, map, grid, st);
-    case 15: return spread_w<T, SPIN, 15>(p, map, grid, st);
-    case 16: return spread_w<T, SPIN, 16>(p, map, grid, st);
-    default: return cudaErrorInvalidValue;
-    }
-}
-
 }  // namespace
+
+// per precision (nufft_f32.cu, nufft_interp64.cu, nufft_spread64.cu)
+cudaError_t interp_f32(const Plan &p, const void *grid, void *map, cudaStream_t st);
+cudaError_t interp_f64(const Plan &p, const void *grid, void *map, cudaStream_t st);
+cudaError_t spread_f32(const Plan &p, const void *map, void *grid, cudaStream_t st);
+cudaError_t spread_f64(const Plan &p, const void *map, void *grid, cudaStream_t st);
 
 cudaError_t launch_interp(const Plan &p, const void *grid, void *map, cudaStream_t st)
 {
-    if (p.prec == LENS_FP32)
-        return p.spin ? interp_dispatch<float, true>(p, grid, map, st) : interp_dispatch<float, false>(p, grid, map, st);
-    return p.spin ? interp_dispatch<double, true>(p, grid, map, st) : interp_dispatch<double, false>(p, grid, map, st);
+    return p.prec == LENS_FP32 ? interp_f32(p, grid, map, st) : interp_f64(p, grid, map, st);
 }
 
 cudaError_t launch_spread(const Plan &p, const void *map, void *grid, cudaStream_t st)
@@ -858,11 +262,7 @@ cudaError_t launch_spread(const Plan &p, const void *map, void *grid, cudaStream
                 if ((e = cudaGetLastError()) != cudaSuccess) return e;
             }
         }
-        if (f32)
-            return p.spin ? spread_dispatch<float, true>(p, map, grid, st)
-                          : spread_dispatch<float, false>(p, map, grid, st);
-        return p.spin ? spread_dispatch<double, true>(p, map, grid, st)
-                      : spread_dispatch<double, false>(p, map, grid, st);
+        return f32 ? spread_f32(p, map, grid, st) : spread_f64(p, map, grid, st);
     }
     // fixed point: FP32 plans accumulate in their own int64 grid, FP64 plans in place
     void *fxg = f32 ? p.fx_grid : grid;
@@ -880,10 +280,7 @@ cudaError_t launch_spread(const Plan &p, const void *map, void *grid, cudaStream
     }
     k_fx_grid_unit<<<1, 1, 0, st>>>(p.fx_maxbits, p.fx_kmax, p.fx_scale);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (f32)
-        e = p.spin ? spread_dispatch<float, true>(p, map, fxg, st) : spread_dispatch<float, false>(p, map, fxg, st);
-    else
-        e = p.spin ? spread_dispatch<double, true>(p, map, fxg, st) : spread_dispatch<double, false>(p, map, fxg, st);
+    e = f32 ? spread_f32(p, map, fxg, st) : spread_f64(p, map, fxg, st);
     if (e != cudaSuccess) return e;
     const unsigned cb = (unsigned)std::min<size_t>((ncell + 255) / 256, 152 * 16);
     if (f32) k_fx_to_grid<float><<<cb, 256, 0, st>>>((const unsigned long long *)fxg, (float *)grid, ncell, p.fx_scale);
