@@ -45,22 +45,22 @@ struct RingTab {
 
 // Restart values of the FP32 Legendre recursion (FP32 plans, see legendre.cu):
 // entry base[m] + (k - 1) nnorth + ring holds the recursion state before the
-// k-th restart of order m (every K degrees) as the pair v (float2, spin s:
+// k-th restart of order m (every K degrees; k = 0: the start values) as the pair v (float2, spin s:
 // float4 for +s then -s) scaled by 2^(-60 E) and its exponent E (e: short,
-// spin s short2; kCkZero marks a state that is identically zero).  Rings
+// spin s short2; 0 for states above 2^-100 and for zeros).  Rings
 // below jb (a multiple of 128: no warp straddles it) run Reinsch's form of the
 // recursion.
 // kstart[m][g]: the restart at which the 32 rings g*32 .. g*32+31 of order m
 // begin (every degree before it is below 2^-40 on all of them; 0 = from the
 // start value).
-constexpr int kCkZero = -30000;
+constexpr int kCkMin = -30000;     // smallest stored exponent
 struct CkTab {
     const void *v = nullptr;
     const void *e = nullptr;
     const int64_t *base = nullptr;
     const short *kstart = nullptr;
     const unsigned char *klog = nullptr;  // per-order log2 of the restart interval (nullptr: K for all)
-    const float2 *cs = nullptr;           // FP32 plans: (c_l, 1/c_l) per alm index (monic scale, PolSM)
+    const float2 *cs = nullptr;           // FP32 plans: c_l as a df32 pair per alm index (monic scale)
     int ngrp = 0;
     int K = 0, jb = 0;
 };
@@ -117,7 +117,7 @@ struct Plan {
     // FP32 plans: restarted FP32 recursion (rst) with its step table rec_s
     // (float4 per alm index) and restart values ck (ck_bytes); otherwise the
     // df32 recursion of rec_a.  FP64 plans: rst selects the restarted df32
-    // recursion (PolDDR), with a restart interval per order (ck_klog, on the
+    // recursion (PkD of legendre_pk.cuh), with a restart interval per order (ck_klog, on the
     // host; ck.klog on the device).
     bool rst = false;
     void *rec_s = nullptr;
@@ -140,9 +140,8 @@ struct Plan {
     void *rec_a = nullptr, *rec_t = nullptr;
     void *rec_a_df = nullptr, *rec_t_df = nullptr;
     double *scale = nullptr;
-    void *coef = nullptr;     // workspace: forward coefficients c_l a_lm of one call
-    void *coef_m = nullptr;   // workspace, restarted FP32 plans: c_l a_lm for the monic plain-form warps
-                              // ([ncomp][nalm], float2 / double2 / df32 float4)
+    void *coef = nullptr;     // workspace: forward coefficients c_l a_lm of one call ([ncomp][nalm], float2 /
+                              // double2 / df32 float4; restarted FP32 plans form them in the kernel)
     // FP32 plans, several maps per call: ring coefficients and prepared
     // coefficients of up to 4 maps, allocated on the first such call
     void *ring_batch = nullptr, *coef_batch = nullptr;
@@ -223,6 +222,10 @@ cudaError_t launch_tab_fill(const Plan &p);
 // gradient entry points use 1/2 forward and 2 adjoint)
 cudaError_t launch_legendre_fwd(const Plan &p, const void *alm, void *ring, cudaStream_t st, double wpos = 1.0);
 cudaError_t launch_legendre_adj(const Plan &p, const void *ring, void *alm, cudaStream_t st, double wpos = 1.0);
+// packed kernels of the plans with restart values (legendre_pk.cuh): rpt rings per thread; src the a_lm of
+// nm maps (FP32 plans) or the prepared df32 coefficients (FP64 plans, nm = 1)
+cudaError_t launch_leg_fwd_pk(const Plan &p, int rpt, const void *src, void *ring, int nm, double wpos, cudaStream_t st);
+cudaError_t launch_leg_adj_pk(const Plan &p, int rpt, const void *ring, void *alm, double wpos, void *fx, cudaStream_t st);
 // FP32 plans: Legendre synthesis of nm = 2 or 4 maps (a_lm consecutive) sharing
 // one recursion; ring and coef hold nm maps' ring / prepared coefficients
 cudaError_t launch_legendre_fwd_batch(const Plan &p, const void *alm, void *ring, void *coef, int nm, cudaStream_t st,

@@ -27,7 +27,8 @@
 //
 // Arithmetic (policies below): FP32 plans run the recursion in df32 (pairs of
 // FP32 words) and accumulate in FP32; FP64 plans run either native FP64, or
-// (orders m >= m_df) the df32 recursion with df32 accumulation.
+// (orders m >= m_df) the df32 recursion with df32 accumulation.  Plans with
+// restart values run the kernels of legendre_pk.cuh instead.
 //
 // Mapping: one CTA per (m, ring chunk); each thread owns RPT adjacent north
 // rings (theta <= pi/2) and obtains the mirrored south ring from
@@ -206,52 +207,15 @@ __device__ __forceinline__ void fwd_block(Rings<P, RPT, SPIN> &st, FwdAcc<P, RPT
     }
 }
 
-// Restarted FP32 recursion, one spin-0 map: the block's step-table entries and
-// prepared coefficients are loaded together before its 8 steps, so their
-// latency is paid once per block instead of once per degree (spin s: the
-// 16 more coefficient registers cost as much as the latency saves).
-template <class P, int RPT, bool SPIN, int REG, class TabE>
-__device__ __forceinline__ void fwd_block_pf(Rings<P, RPT, SPIN> &st, FwdAcc<P, RPT, SPIN, 1, false> &acc,
-                                             const TabE *reca, const float2 *ca, const float2 *cb, int lb)
-{
-    TabE tb[kBlk];
-    float2 a[kBlk], b[kBlk];
-#pragma unroll
-    for (int j = 0; j < kBlk; ++j) {
-        tb[j] = __ldg(reca + lb + j);
-        if (REG != 1) {
-            a[j] = __ldg(ca + lb + j);
-            if (SPIN) b[j] = __ldg(cb + lb + j);
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < kBlk; ++j) {
-        typename P::V vp[RPT], vm[RPT];
-        if (j & 1) st.template advance_c<1, REG != 0>(tb[j]);
-        else st.template advance_c<0, REG != 0>(tb[j]);
-        if (REG == 1) continue;
-#pragma unroll
-        for (int k = 0; k < RPT; ++k) {
-            vp[k] = (j & 1) ? st.template vplus<1, REG == 2>(k) : st.template vplus<0, REG == 2>(k);
-            if (SPIN) vm[k] = (j & 1) ? st.template vminus<1, REG == 2>(k) : st.template vminus<0, REG == 2>(k);
-        }
-        const float2 bb = SPIN ? b[j] : make_float2(0.f, 0.f);
-        if (j & 1) acc.template add_vals_c<true>(vp, vm, a[j].x, a[j].y, bb.x, bb.y);
-        else acc.template add_vals_c<false>(vp, vm, a[j].x, a[j].y, bb.x, bb.y);
-    }
-}
-
 // NM maps share each recursion (prepared coefficients of map b at coef + b *
 // ncomp nalm entries, its ring coefficients at ring + b * ring_stride).
 // GRAD: gradient-only spin s (prepared coefficients of G alone, see FwdAcc).
-// Restarted FP32 recursions (P::kRestart) reset their state from ck at every
-// K-th degree of the block loop.
 template <class P, int RPT, bool SPIN, int NM, bool GRAD>
 __device__ __forceinline__ void leg_fwd_body(const void *__restrict__ coef, const void *__restrict__ rec_a,
                                              const void *__restrict__ rec_t, const double *__restrict__ lognorm,
                                              const RingTab &rt, typename P::C *__restrict__ ring, int lmax, int mmax,
                                              int spin, int ntheta, int nnorth, int64_t nalm, int m_begin,
-                                             int64_t ring_stride, const CkTab &ck)
+                                             int64_t ring_stride)
 {
     using Sg = decltype(P::fac(0));
     using Cx = typename P::C;
@@ -274,47 +238,14 @@ __device__ __forceinline__ void leg_fwd_body(const void *__restrict__ coef, cons
     acc.init(coef, nalm, base);
     const Sg s0 = ((lf - m) & 1) ? Sg(-1) : Sg(1);  // (-1)^(lf - m)
     int l = lf;
-    bool jumped = false;
-    const int Km = P::kRestart ? ck_interval(ck, m) : 0;
-    if constexpr (P::kRestart) {  // start at the warp's first restart: every earlier degree is negligible
-        const int kj = first_restart<RPT>(ck, m);
-        if (kj > 0) {
-            st.init_geom(rt, rp0, nnorth);
-            l = lf + kj * Km;  // the restart at l sets the state
-            jumped = true;
-        }
-    }
-    if (!jumped) {
-        st.init(rt, rp0, nnorth, m, s, lognorm[m]);
-        acc.add_rt(st, l0, true);  // l0 = lf - 1
-    }
-    const int64_t ckrow = P::kRestart ? __ldg(ck.base + m) : 0;
+    st.init(rt, rp0, nnorth, m, s, lognorm[m]);
+    acc.add_rt(st, l0, true);  // l0 = lf - 1
     for (; l + kBlk <= lmax + 1; l += kBlk) {
-        if constexpr (P::kRestart) {
-            const int dl = l - lf;
-            if (dl != 0 && (dl & (Km - 1)) == 0) {
-                const int64_t row = ckrow + (int64_t)(dl / Km - 1) * nnorth;
-                if constexpr (P::kScaleF) st.restart_scaled(ck, row, rp0, nnorth, ck.cs + base, l);
-                else st.restart(ck, row, rp0, nnorth);
-            }
-        }
-        int reg = st.regime();
-        // restarted recursions start at the warp's first significant restart, so a block of
-        // negligible states is rare there: it runs the scaled path (its terms are exact zeros)
-        // and the recursion-only variant is not compiled
-        if constexpr (P::kRestart) reg = reg == 1 ? 2 : reg;
+        const int reg = st.regime();
         acc.renorm();
-        if constexpr (P::kRestart && !P::kMonic && NM == 1 && !GRAD && !SPIN) {  // lmax 4096: 4.52 -> 4.40 ms;
-                                                                                // spin s gains nothing
-            const float2 *ca = (const float2 *)coef + base;
-            const float2 *cb = (const float2 *)coef + nalm + base;
-            if (reg == 0) fwd_block_pf<P, RPT, SPIN, 0>(st, acc, reca, ca, cb, l);
-            else fwd_block_pf<P, RPT, SPIN, 2>(st, acc, reca, ca, cb, l);
-        } else {
-            if (reg == 0) fwd_block<P, RPT, SPIN, 0, NM, GRAD>(st, acc, reca, rect, l);
-            else if (!P::kRestart && reg == 1) fwd_block<P, RPT, SPIN, 1, NM, GRAD>(st, acc, reca, rect, l);
-            else fwd_block<P, RPT, SPIN, 2, NM, GRAD>(st, acc, reca, rect, l);
-        }
+        if (reg == 0) fwd_block<P, RPT, SPIN, 0, NM, GRAD>(st, acc, reca, rect, l);
+        else if (reg == 1) fwd_block<P, RPT, SPIN, 1, NM, GRAD>(st, acc, reca, rect, l);
+        else fwd_block<P, RPT, SPIN, 2, NM, GRAD>(st, acc, reca, rect, l);
     }
     for (; l <= lmax; ++l) {  // tail: general path
         st.advance_moved(reca, rect, l);
@@ -370,35 +301,10 @@ __global__ void __launch_bounds__(512) k_leg_fwd(const void *__restrict__ coef, 
                                                  const void *__restrict__ rec_t, const double *__restrict__ lognorm,
                                                  RingTab rt, typename P::C *__restrict__ ring, int lmax, int mmax,
                                                  int spin, int ntheta, int nnorth, int64_t nalm, int m_begin,
-                                                 int64_t ring_stride, CkTab ck)
+                                                 int64_t ring_stride)
 {
     leg_fwd_body<P, RPT, SPIN, NM, GRAD>(coef, rec_a, rec_t, lognorm, rt, ring, lmax, mmax, spin, ntheta, nnorth,
-                                         nalm, m_begin, ring_stride, ck);
-}
-
-// Restarted FP32 recursion: warps whose rings lie below ck.jb run Reinsch's
-// form, the others the plain form (the choice is uniform per warp).
-// One map: the plain-form warps run the monic step (PolSM) on the df32 table
-// rec_a with the coefficients coef_m (times c_l): spin 2 at lmax 4096 12.09 ->
-// 11.46 ms (spin 0 unchanged); several maps keep PolS.
-template <int RPT, bool SPIN, int NM = 1, bool GRAD = false>
-__global__ void __launch_bounds__(512) k_leg_fwd32(const void *__restrict__ coef, const void *__restrict__ rec_s,
-                                                   const double *__restrict__ lognorm, RingTab rt,
-                                                   float2 *__restrict__ ring, int lmax, int mmax, int spin, int ntheta,
-                                                   int nnorth, int64_t nalm, int m_begin, int64_t ring_stride,
-                                                   CkTab ck, const void *__restrict__ coef_m,
-                                                   const void *__restrict__ rec_a)
-{
-    const int wr0 = ((blockIdx.x * blockDim.x + threadIdx.x) & ~31) * RPT;  // first ring of the warp
-    if (wr0 < ck.jb)
-        leg_fwd_body<PolR, RPT, SPIN, NM, GRAD>(coef, rec_s, nullptr, lognorm, rt, ring, lmax, mmax, spin, ntheta,
-                                                nnorth, nalm, m_begin, ring_stride, ck);
-    else if constexpr (NM == 1)
-        leg_fwd_body<PolSM, RPT, SPIN, NM, GRAD>(coef_m, rec_a, nullptr, lognorm, rt, ring, lmax, mmax, spin, ntheta,
-                                                 nnorth, nalm, m_begin, ring_stride, ck);
-    else
-        leg_fwd_body<PolS, RPT, SPIN, NM, GRAD>(coef, rec_s, nullptr, lognorm, rt, ring, lmax, mmax, spin, ntheta,
-                                                nnorth, nalm, m_begin, ring_stride, ck);
+                                         nalm, m_begin, ring_stride);
 }
 
 // ---------------------------------------------------------------- adjoint
@@ -542,11 +448,9 @@ template <class P, int RPT, bool SPIN, bool GRAD = false> struct AdjIn {
 // times the monic scale c_l and the order weight wm, into a_lm (spin 0) or
 // G, C (spin s); with fx (deterministic plans) into the fixed-point sums fx
 // (same layout, units of 1 / fxu) instead.
-// wmf: (float) wm, formed once by the caller, so that FP32 plans without a scale table
-// add their sums with no FP64 arithmetic here.
 template <class P, bool SPIN, int NV>
 __device__ __forceinline__ void flush(typename P::A (&part)[NV], typename P::R *out, const double *__restrict__ sc,
-                                      double wm, float wmf, int64_t base, int64_t nalm, int m, int lb, int lmax,
+                                      double wm, int64_t base, int64_t nalm, int m, int lb, int lmax,
                                       decltype(P::fac(0)) sgs, unsigned long long *fx, double fxu)
 {
     using A = typename P::A;
@@ -561,13 +465,7 @@ __device__ __forceinline__ void flush(typename P::A (&part)[NV], typename P::R *
     if (!SPIN) {
         if ((lane & ((1 << SH) - 1)) == 0 && l <= lmax && !(m == 0 && c == 1)) {
             const int64_t dst = 2 * (base + l) + c;
-            if constexpr (std::is_same<typename P::A, float>::value) {
-                if (!sc && !fx) {
-                    atomicAdd(out + dst, tot * wmf);
-                    return;
-                }
-            }
-            const double cl = sc ? __ldg(sc + l) : 1.0;
+            const double cl = __ldg(sc + l);
             if (fx) P::atomic_add_fx(fx + dst, tot, cl * wm, fxu);
             else P::atomic_add(out + dst, tot, cl * wm);
         }
@@ -586,13 +484,7 @@ __device__ __forceinline__ void flush(typename P::A (&part)[NV], typename P::R *
             else if (c == 2) { val = P::ascale(P::aadd(other, P::ascale(tot, -sgs)), h); dst = 2 * (nalm + base + l) + 1; }
             else { val = P::ascale(P::aadd(other, P::ascale(tot, sgs)), -h); dst = 2 * (nalm + base + l); }
             if (!(m == 0 && (c == 1 || c == 2))) {
-                if constexpr (std::is_same<typename P::A, float>::value) {
-                    if (!sc && !fx) {
-                        atomicAdd(out + dst, val * wmf);
-                        return;
-                    }
-                }
-                const double cl = sc ? __ldg(sc + l) : 1.0;
+                const double cl = __ldg(sc + l);
                 if (fx) P::atomic_add_fx(fx + dst, val, cl * wm, fxu);
                 else P::atomic_add(out + dst, val, cl * wm);
             }
@@ -611,7 +503,7 @@ template <int NV> constexpr int kRowStride = NV + 4;
 
 template <bool SPIN, int NV>
 __device__ __forceinline__ void flush_smem(float (&part)[NV], float *wbuf, float *out, const double *__restrict__ sc,
-                                           double wm, float wmf, int64_t base, int64_t nalm, int m, int lb, int lmax,
+                                           double wm, int64_t base, int64_t nalm, int m, int lb, int lmax,
                                            float sgs, unsigned long long *fx, double fxu)
 {
     static_assert(NV == 16 || NV == 32, "NV must be 16 or 32");
@@ -643,8 +535,8 @@ __device__ __forceinline__ void flush_smem(float (&part)[NV], float *wbuf, float
     if (!SPIN) {
         if (lane < NV && l <= lmax && !(m == 0 && c == 1)) {
             const int64_t dst = 2 * (base + l) + c;
-            if (fx) PolDF::atomic_add_fx(fx + dst, tot, (sc ? __ldg(sc + l) : 1.0) * wm, fxu);
-            else atomicAdd(out + dst, tot * (sc ? (float)(__ldg(sc + l) * wm) : wmf));
+            if (fx) PolDF::atomic_add_fx(fx + dst, tot, __ldg(sc + l) * wm, fxu);
+            else atomicAdd(out + dst, tot * (float)(__ldg(sc + l) * wm));
         }
     } else {
         const float other = __shfl_xor_sync(0xffffffffu, tot, 2);  // U <-> V of the same l
@@ -656,8 +548,8 @@ __device__ __forceinline__ void flush_smem(float (&part)[NV], float *wbuf, float
             else if (c == 2) { val = 0.5f * (other - sgs * tot); dst = 2 * (nalm + base + l) + 1; }
             else { val = -0.5f * (other + sgs * tot); dst = 2 * (nalm + base + l); }
             if (!(m == 0 && (c == 1 || c == 2))) {
-                if (fx) PolDF::atomic_add_fx(fx + dst, val, (sc ? __ldg(sc + l) : 1.0) * wm, fxu);
-                else atomicAdd(out + dst, val * (sc ? (float)(__ldg(sc + l) * wm) : wmf));
+                if (fx) PolDF::atomic_add_fx(fx + dst, val, __ldg(sc + l) * wm, fxu);
+                else atomicAdd(out + dst, val * (float)(__ldg(sc + l) * wm));
             }
         }
     }
@@ -693,7 +585,7 @@ __device__ __forceinline__ void leg_adj_body(const typename P::C *__restrict__ r
                                              const double *__restrict__ scale, const RingTab &rt,
                                              typename P::C *__restrict__ alm, int lmax, int mmax, int spin,
                                              int ntheta, int nnorth, int64_t nalm, int m_begin, double wpos,
-                                             unsigned long long *fx, const double *__restrict__ fxs, const CkTab &ck)
+                                             unsigned long long *fx, const double *__restrict__ fxs)
 {
     using A = typename P::A;
     using R = typename P::R;
@@ -711,37 +603,25 @@ __device__ __forceinline__ void leg_adj_body(const typename P::C *__restrict__ r
         SPIN ? reinterpret_cast<const typename P::Tab *>((const typename P::TabAT *)rec_a + base)
              : (const typename P::Tab *)rec_a + base;
     const typename P::TTab *rect = SPIN ? (const typename P::TTab *)rec_t + base : nullptr;
-    const double *sc = P::kMonic ? scale + base : nullptr;  // restarted FP32 recursions carry lambda itself
+    const double *sc = scale + base;
     const int rp0 = (blockIdx.x * blockDim.x + threadIdx.x) * RPT;
     const Sg sgs = (s & 1) ? Sg(-1) : Sg(1);
     R *out = reinterpret_cast<R *>(alm);
     const int lf = l0 + 1;
     const double wm = (m > 0 ? wpos : 1.0) * (GRAD ? -0.5 : 1.0);
-    const float wmf = (float)wm;
     const double fxu = fx ? fxs[1 + m] : 0.0;  // deterministic plans: fixed-point unit of order m
 
     Rings<P, RPT, SPIN> st;
     AdjIn<P, RPT, SPIN, GRAD> in;
     in.init(ring, rp0, nnorth, ntheta, m, mmax, ((lf - m) & 1) != 0, (s & 1) != 0);
     int l = lf;
-    bool jumped = false;
-    const int Km = P::kRestart ? ck_interval(ck, m) : 0;
-    if constexpr (P::kRestart) {  // start at the warp's first restart: every earlier degree is negligible
-        const int kj = first_restart<RPT>(ck, m);
-        if (kj > 0) {
-            st.init_geom(rt, rp0, nnorth);
-            l = lf + kj * Km;  // the restart at l sets the state
-            jumped = true;
-        }
-    }
-    if (!jumped) {
-        st.init(rt, rp0, nnorth, m, s, lognorm[m]);
-        // degree l0 (the start value): one reduction of NCOMP values
+    st.init(rt, rp0, nnorth, m, s, lognorm[m]);
+    {  // degree l0 (the start value): one reduction of NCOMP values
         A p0[NCOMP];
 #pragma unroll
         for (int c = 0; c < NCOMP; ++c) p0[c] = P::azero();
         in.add_rt(st, true, p0);  // l0 = lf - 1
-        flush<P, FSPIN, NCOMP>(p0, out, sc, wm, wmf, base, nalm, m, l0, lmax, sgs, fx, fxu);
+        flush<P, FSPIN, NCOMP>(p0, out, sc, wm, base, nalm, m, l0, lmax, sgs, fx, fxu);
     }
     A part[NV];
     // measured at lmax 4096: spin s 42.8 -> 41.6 ms; spin 0 (16 values per lane)
@@ -749,30 +629,21 @@ __device__ __forceinline__ void leg_adj_body(const typename P::C *__restrict__ r
     constexpr bool kSmemFlush = std::is_same<typename P::A, float>::value && FSPIN;
     extern __shared__ __align__(16) float adj_smem[];
     float *wbuf = adj_smem + (threadIdx.x >> 5) * (adj_smem_per_warp<FSPIN>() / sizeof(float));
-    const int64_t ckrow = P::kRestart ? __ldg(ck.base + m) : 0;
     for (; l + kBlk <= lmax + 1; l += kBlk) {
-        if constexpr (P::kRestart) {
-            const int dl = l - lf;
-            if (dl != 0 && (dl & (Km - 1)) == 0) {
-                const int64_t row = ckrow + (int64_t)(dl / Km - 1) * nnorth;
-                if constexpr (P::kScaleF) st.restart_scaled(ck, row, rp0, nnorth, ck.cs + base, l);
-                else st.restart(ck, row, rp0, nnorth);
-            }
-        }
         const int reg = st.regime();
-        if (!P::kRestart && reg == 1) {  // every contribution of this block is below 2^-180: recursion only
+        if (reg == 1) {  // every contribution of this block is below 2^-180: recursion only
             adj_block<P, RPT, SPIN, 1, GRAD>(st, in, part, reca, rect, l);
             continue;
-        }  // restarted recursions: such blocks are rare (see leg_fwd_body) and take the scaled path
+        }
 #pragma unroll
         for (int i = 0; i < NV; ++i) part[i] = P::azero();
         if (reg == 0) adj_block<P, RPT, SPIN, 0, GRAD>(st, in, part, reca, rect, l);
         else adj_block<P, RPT, SPIN, 2, GRAD>(st, in, part, reca, rect, l);
         if constexpr (kSmemFlush)
-            flush_smem<FSPIN, NV>(part, wbuf, reinterpret_cast<float *>(alm), sc, wm, wmf, base, nalm, m, l, lmax, sgs, fx,
+            flush_smem<FSPIN, NV>(part, wbuf, reinterpret_cast<float *>(alm), sc, wm, base, nalm, m, l, lmax, sgs, fx,
                                   fxu);
         else
-            flush<P, FSPIN, NV>(part, out, sc, wm, wmf, base, nalm, m, l, lmax, sgs, fx, fxu);
+            flush<P, FSPIN, NV>(part, out, sc, wm, base, nalm, m, l, lmax, sgs, fx, fxu);
     }
     if (l <= lmax) {  // tail: fewer than kBlk degrees, general path
 #pragma unroll
@@ -784,7 +655,7 @@ __device__ __forceinline__ void leg_adj_body(const typename P::C *__restrict__ r
                 in.add_rt(st, (j & 1) != 0, part + j * NCOMP);
             }
         }
-        flush<P, FSPIN, NV>(part, out, sc, wm, wmf, base, nalm, m, l, lmax, sgs, fx, fxu);
+        flush<P, FSPIN, NV>(part, out, sc, wm, base, nalm, m, l, lmax, sgs, fx, fxu);
     }
 }
 
@@ -794,30 +665,10 @@ __global__ void __launch_bounds__(512) k_leg_adj(const typename P::C *__restrict
                                                  const double *__restrict__ scale, RingTab rt,
                                                  typename P::C *__restrict__ alm, int lmax, int mmax, int spin,
                                                  int ntheta, int nnorth, int64_t nalm, int m_begin, double wpos,
-                                                 unsigned long long *fx, const double *__restrict__ fxs, CkTab ck)
+                                                 unsigned long long *fx, const double *__restrict__ fxs)
 {
     leg_adj_body<P, RPT, SPIN, GRAD>(ring, rec_a, rec_t, lognorm, scale, rt, alm, lmax, mmax, spin, ntheta, nnorth,
-                                     nalm, m_begin, wpos, fx, fxs, ck);
-}
-
-// Restarted FP32 recursion (see k_leg_fwd32).
-// At most 80 registers: the spin-s kernel (97 registers unconstrained) then keeps 24
-// instead of 16 warps per SM (lmax 4096: spin 2 14.39 -> 13.68 ms, spin 0 5.38 -> 5.26 ms;
-// 96 registers: 13.64 / 5.35 ms).
-template <int RPT, bool SPIN, bool GRAD = false>
-__global__ void __maxnreg__(80) k_leg_adj32(const float2 *__restrict__ ring, const void *__restrict__ rec_s,
-                                                   const double *__restrict__ lognorm, RingTab rt,
-                                                   float2 *__restrict__ alm, int lmax, int mmax, int spin, int ntheta,
-                                                   int nnorth, int64_t nalm, int m_begin, double wpos,
-                                                   unsigned long long *fx, const double *__restrict__ fxs, CkTab ck)
-{
-    const int wr0 = ((blockIdx.x * blockDim.x + threadIdx.x) & ~31) * RPT;  // first ring of the warp
-    if (wr0 < ck.jb)
-        leg_adj_body<PolR, RPT, SPIN, GRAD>(ring, rec_s, nullptr, lognorm, nullptr, rt, alm, lmax, mmax, spin, ntheta,
-                                            nnorth, nalm, m_begin, wpos, fx, fxs, ck);
-    else  // (the monic PolSM measured 8% slower here for spin 2: 16.0 -> 17.3 ms at lmax 4096)
-        leg_adj_body<PolS, RPT, SPIN, GRAD>(ring, rec_s, nullptr, lognorm, nullptr, rt, alm, lmax, mmax, spin, ntheta,
-                                            nnorth, nalm, m_begin, wpos, fx, fxs, ck);
+                                     nalm, m_begin, wpos, fx, fxs);
 }
 
 // ---------------------------------------------- fixed point (deterministic plans)
@@ -923,10 +774,10 @@ __global__ void k_rec_tables(int lmax, int spin, double *__restrict__ scale, flo
             if (t64) t64[base + l] = tau;
         }
     }
-    if (cs) {  // (c_l, 1/c_l) in FP32 for the monic plain-form rings of the restarted FP32 recursion
+    if (cs) {  // c_l as a df32 pair for the monic plain-form rings of the restarted FP32 recursion
         for (int l = m + threadIdx.x; l <= lmax; l += blockDim.x) {
-            const double c = scale[base + l];
-            cs[base + l] = l >= l0 ? make_float2((float)c, (float)(1.0 / c)) : make_float2(0.f, 0.f);
+            const df32 c = df_split(scale[base + l]);
+            cs[base + l] = make_float2(c.h, c.l);
         }
     }
 }
@@ -961,10 +812,11 @@ __global__ void k_rec_tables_s(int lmax, int spin, float4 *__restrict__ out)
 // lb = lf + K k (k = 1 .. ck_count) the FP32 kernels hold (lambda_{lb-2},
 // lambda_{lb-1}) in the plain form and (D_{lb-1}, lambda_{lb-1}) in Reinsch's
 // form (rings below jb); those pairs are written scaled by 2^(-60 E) in FP32
-// with E (kCkZero for a state that is identically zero).  lt[m][j]: the first
+// with E (0 from 2^-100 up and for a state that is identically zero); the row before the first restart's
+// holds the start values, the state before lf (w0 = 0, Reinsch D = lambda_{l0}).  lt[m][j]: the first
 // degree at which |lambda| (either sign of the spin) reaches 2^-40, lmax + 1
 // if none does before the last restart.
-// DD (FP64 plans, PolDDR): the monic state itself split into df32 words,
+// DD (FP64 plans, PkD of legendre_pk.cuh): the monic state itself split into df32 words,
 // float4 (w0.h, w0.l, w1.h, w1.l) per sign of the spin, no Reinsch form, and
 // lt the first degree reaching 2^-64.
 template <bool SPIN, bool DD = false>
@@ -985,30 +837,83 @@ __global__ void k_ck_build(const double *__restrict__ a64, const double *__restr
     if (l0 > lmax) return;
     const int lf = l0 + 1;
     const int nck = ck_count(lmax, lf, K);
-    if (nck == 0) return;
     const int64_t base = alm_base(lmax, m);
     const double x = rt.x[j];
     PolF64::St sp, sm;
     start_value<PolF64>(sp, m, s, s, lognorm[m], rt.lsin2[j], rt.lcos2[j]);
     if (SPIN) start_value<PolF64>(sm, m, s, -s, lognorm[m], rt.lsin2[j], rt.lcos2[j]);
     const bool rein = !DD && j < jb;
+    // A state above 2^-100 (DD: 2^-75, for its low words) is written at scale 0, where FP32 still holds it as a
+    // normal number, so that few evanescent states take the kernels' scaled path; an identically zero
+    // state too.
+    auto scaled_down = [&](const PolF64::St &st, short &e) {
+        const double w = fmax(fabs(st.w[0]), fabs(st.w[1]));
+        const bool up = w == 0.0 || ilogb(w) + kScaleBits * st.E >= (DD ? -75 : -100);
+        e = up ? (short)0 : (short)max(st.E, kCkMin);
+        return up ? ldexp(1.0, kScaleBits * max(st.E, -3)) : 1.0;
+    };
     auto quad = [&](const PolF64::St &st, float4 &v, short &e) {
-        if (st.w[0] == 0.0 && st.w[1] == 0.0) { v = make_float4(0.f, 0.f, 0.f, 0.f); e = (short)kCkZero; return; }
-        const df32 a = df_split(st.w[0]), b = df_split(st.w[1]);
+        const double f = scaled_down(st, e);
+        const df32 a = df_split(st.w[0] * f), b = df_split(st.w[1] * f);
         v = make_float4(a.h, a.l, b.h, b.l);
-        e = (short)max(st.E, kCkZero + 1);
     };
     auto pair = [&](const PolF64::St &st, int l, float &w0, float &w1, short &e) {
-        if (st.w[0] == 0.0 && st.w[1] == 0.0) { w0 = 0.f; w1 = 0.f; e = (short)kCkZero; return; }
-        const double v1 = st.w[1] * scale[base + l];
-        const double v0 = st.w[0] * scale[base + l - 1];
+        const double f = scaled_down(st, e);
+        const double v1 = st.w[1] * f * scale[base + l];
+        const double v0 = l > l0 ? st.w[0] * f * scale[base + l - 1] : 0.0;
         w1 = (float)v1;
         w0 = (float)(rein ? v1 - v0 : v0);
-        e = (short)max(st.E, kCkZero + 1);
     };
     auto big = [&](const PolF64::St &st, int l) {  // |lambda_l| >= 2^-40 (DD: 2^-64)
         return st.E >= -2 && ldexp(fabs(st.w[1]) * scale[base + l], kScaleBits * st.E) >= (DD ? 0x1p-64 : 0x1p-40);
     };
+    // start values of the FP32 recursion: mantissas formed in FP32, as its own start does
+    auto start32 = [&](int sigma, float &w0, float &w1, short &e) {
+        PolS::St f;
+        start_value<PolS>(f, m, s, sigma, lognorm[m], rt.lsin2[j], rt.lcos2[j]);
+        const bool up = f.w[1] == 0.f || ilogbf(f.w[1]) + kScaleBits * f.E >= -100;
+        e = up ? (short)0 : (short)max(f.E, kCkMin);
+        w1 = up ? ldexpf(f.w[1], kScaleBits * max(f.E, -3)) : f.w[1];
+        w0 = rein ? w1 : 0.f;
+    };
+    auto store = [&](int k, int l) {  // the state before restart k (k = 0: before lf), l its last degree
+        const int64_t idx = ckbase[m] + (int64_t)(k - 1) * nnorth + j;
+        if (DD) {
+            float4 a, b;
+            short ea, eb;
+            quad(sp, a, ea);
+            if (!SPIN) {
+                reinterpret_cast<float4 *>(vout)[idx] = a;
+                reinterpret_cast<short *>(eout)[idx] = ea;
+            } else {
+                quad(sm, b, eb);
+                reinterpret_cast<float4 *>(vout)[2 * idx] = a;
+                reinterpret_cast<float4 *>(vout)[2 * idx + 1] = b;
+                reinterpret_cast<short2 *>(eout)[idx] = make_short2(ea, eb);
+            }
+        } else if (!SPIN) {
+            float2 v;
+            short e;
+            if (k == 0) start32(s, v.x, v.y, e);
+            else pair(sp, l, v.x, v.y, e);
+            reinterpret_cast<float2 *>(vout)[idx] = v;
+            reinterpret_cast<short *>(eout)[idx] = e;
+        } else {
+            float4 v;
+            short2 e;
+            if (k == 0) {
+                start32(s, v.x, v.y, e.x);
+                start32(-s, v.z, v.w, e.y);
+            } else {
+                pair(sp, l, v.x, v.y, e.x);
+                pair(sm, l, v.z, v.w, e.y);
+            }
+            reinterpret_cast<float4 *>(vout)[idx] = v;
+            reinterpret_cast<short2 *>(eout)[idx] = e;
+        }
+    };
+    store(0, l0);
+    if (nck == 0) return;
     int lfirst = lmax + 1;
     if (big(sp, l0) || (SPIN && big(sm, l0))) lfirst = l0;
     int k = 1;
@@ -1030,39 +935,35 @@ __global__ void k_ck_build(const double *__restrict__ a64, const double *__restr
         }
         if (lfirst > lmax && (big(sp, l) || (SPIN && big(sm, l)))) lfirst = l;
         if (l == lck) {
-            const int64_t idx = ckbase[m] + (int64_t)(k - 1) * nnorth + j;
-            if (DD) {
-                float4 a, b;
-                short ea, eb;
-                quad(sp, a, ea);
-                if (!SPIN) {
-                    reinterpret_cast<float4 *>(vout)[idx] = a;
-                    reinterpret_cast<short *>(eout)[idx] = ea;
-                } else {
-                    quad(sm, b, eb);
-                    reinterpret_cast<float4 *>(vout)[2 * idx] = a;
-                    reinterpret_cast<float4 *>(vout)[2 * idx + 1] = b;
-                    reinterpret_cast<short2 *>(eout)[idx] = make_short2(ea, eb);
-                }
-            } else if (!SPIN) {
-                float2 v;
-                short e;
-                pair(sp, l, v.x, v.y, e);
-                reinterpret_cast<float2 *>(vout)[idx] = v;
-                reinterpret_cast<short *>(eout)[idx] = e;
-            } else {
-                float4 v;
-                short2 e;
-                pair(sp, l, v.x, v.y, e.x);
-                pair(sm, l, v.z, v.w, e.y);
-                reinterpret_cast<float4 *>(vout)[idx] = v;
-                reinterpret_cast<short2 *>(eout)[idx] = e;
-            }
+            store(k, l);
             ++k;
             lck += K;
         }
     }
     *ltp = lfirst;
+}
+
+// Clears the restart states that never reach lt's threshold before the next restart (identically zero at
+// scale 0: they contribute nothing, as the degrees before a warp's first restart do), so that the rings of a
+// warp that are still evanescent keep it out of the scaled path.  The degrees after an order's last restart
+// are not tracked by lt: that row stays.
+__global__ void k_ck_clear(const int *__restrict__ lt, int lmax, int spin, int nnorth, int Kall,
+                           const int64_t *__restrict__ ckbase, void *__restrict__ v, void *__restrict__ e, int vsz,
+                           const unsigned char *__restrict__ klog)
+{
+    const int m = blockIdx.y;
+    const int K = klog ? 1 << klog[m] : Kall;
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    const int l0 = m > spin ? m : spin;
+    if (j >= nnorth || l0 > lmax) return;
+    const int lf = l0 + 1, nck = ck_count(lmax, lf, K);
+    const int first = lt[(int64_t)m * nnorth + j];
+    for (int k = 1; k < nck && lf + K * (k + 1) <= first; ++k) {
+        const int64_t idx = ckbase[m] + (int64_t)(k - 1) * nnorth + j;
+        for (int i = 0; i < vsz / 8; ++i) reinterpret_cast<float2 *>(v)[idx * (vsz / 8) + i] = make_float2(0.f, 0.f);
+        if (spin) reinterpret_cast<short2 *>(e)[idx] = make_short2(0, 0);
+        else reinterpret_cast<short *>(e)[idx] = 0;
+    }
 }
 
 // First restart of every 32-ring group and order: the largest k <= ck_count
@@ -1117,8 +1018,7 @@ __global__ void k_coef_prep(const Tin *__restrict__ alm, const double *__restric
     const bool hi = m >= m_split;
     for (int l = m + blockIdx.x * blockDim.x + threadIdx.x; l <= lmax; l += gridDim.x * blockDim.x) {
         const int64_t i = base + l;
-        // plans with restarted FP32 recursions carry lambda itself (no monic scale)
-        const double c = (scale ? scale[i] : (l >= (m > spin ? m : spin) ? 1.0 : 0.0)) * wm;
+        const double c = scale[i] * wm;
         const Tin gv = alm[i];
         const double gr = gv.x, gi = m == 0 ? 0.0 : (double)gv.y;
         if (!spin) {
@@ -1147,7 +1047,7 @@ cudaError_t fwd_launch(const Plan &p, const Plan::LegShape &sh, const void *coef
     dim3 block(sh.warps * 32);
     k_leg_fwd<P, RPT, SPIN, NM, GRAD><<<grid, block, 0, st>>>(coef, ta, tt, p.lognorm, p.rings, (typename P::C *)ring,
                                                         p.lmax, p.mmax, p.spin, p.ntheta, p.nnorth, p.nalm, m_begin,
-                                                        (int64_t)p.ncol * p.ntheta, P::kRestart ? p.ck : CkTab{});
+                                                        (int64_t)p.ncol * p.ntheta);
     return cudaGetLastError();
 }
 
@@ -1166,8 +1066,7 @@ cudaError_t adj_launch(const Plan &p, const Plan::LegShape &sh, const void *ring
     k_leg_adj<P, RPT, SPIN, GRAD><<<grid, block, adj_smem_bytes<P, SPIN, GRAD>(sh.warps), st>>>(
                                                     (const typename P::C *)ring, ta, tt, p.lognorm, p.scale, p.rings,
                                                     (typename P::C *)alm, p.lmax, p.mmax, p.spin, p.ntheta, p.nnorth,
-                                                    p.nalm, m_begin, wpos, (unsigned long long *)fx,
-                                                    p.fx_scale, P::kRestart ? p.ck : CkTab{});
+                                                    p.nalm, m_begin, wpos, (unsigned long long *)fx, p.fx_scale);
     return cudaGetLastError();
 }
 
@@ -1185,90 +1084,6 @@ cudaError_t adj_rpt(const Plan &p, const Plan::LegShape &sh, const void *ring, c
 {
     if (sh.rpt == 1) return adj_launch<P, 1, SPIN, GRAD>(p, sh, ring, ta, tt, alm, m_begin, m_end, st, wpos, fx);
     return adj_launch<P, 2, SPIN, GRAD>(p, sh, ring, ta, tt, alm, m_begin, m_end, st, wpos, fx);
-}
-
-// Restarted FP32 recursion (plans with p.rst): one launch per direction
-template <int RPT, bool SPIN, int NM = 1, bool GRAD = false>
-cudaError_t fwd32_launch(const Plan &p, const Plan::LegShape &sh, const void *coef, void *ring, int m_begin,
-                         int m_end, cudaStream_t st)
-{
-    if (m_end <= m_begin) return cudaSuccess;
-    dim3 grid(sh.chunks, m_end - m_begin);
-    dim3 block(sh.warps * 32);
-    k_leg_fwd32<RPT, SPIN, NM, GRAD><<<grid, block, 0, st>>>(coef, p.rec_s, p.lognorm, p.rings, (float2 *)ring, p.lmax,
-                                                           p.mmax, p.spin, p.ntheta, p.nnorth, p.nalm, m_begin,
-                                                           (int64_t)p.ncol * p.ntheta, p.ck, p.coef_m, p.rec_a);
-    return cudaGetLastError();
-}
-
-template <int RPT, bool SPIN, bool GRAD = false>
-cudaError_t adj32_launch(const Plan &p, const Plan::LegShape &sh, const void *ring, void *alm, int m_begin, int m_end,
-                         cudaStream_t st, double wpos, void *fx)
-{
-    if (m_end <= m_begin) return cudaSuccess;
-    dim3 grid(sh.chunks, m_end - m_begin);
-    dim3 block(sh.warps * 32);
-    k_leg_adj32<RPT, SPIN, GRAD><<<grid, block, adj_smem_bytes<PolDF, SPIN, GRAD>(sh.warps), st>>>(
-        (const float2 *)ring, p.rec_s, p.lognorm, p.rings, (float2 *)alm, p.lmax, p.mmax, p.spin, p.ntheta, p.nnorth,
-        p.nalm, m_begin, wpos, (unsigned long long *)fx, p.fx_scale, p.ck);
-    return cudaGetLastError();
-}
-
-// rings per thread 1, 2 or 4 (the warp-uniform table loads are shared by the rings of a thread)
-template <bool SPIN, int NM = 1, bool GRAD = false>
-cudaError_t fwd32_rpt(const Plan &p, const Plan::LegShape &sh, const void *coef, void *ring, int m_begin, int m_end,
-                      cudaStream_t st)
-{
-    if (sh.rpt == 1) return fwd32_launch<1, SPIN, NM, GRAD>(p, sh, coef, ring, m_begin, m_end, st);
-    if (sh.rpt == 2) return fwd32_launch<2, SPIN, NM, GRAD>(p, sh, coef, ring, m_begin, m_end, st);
-    return fwd32_launch<4, SPIN, NM, GRAD>(p, sh, coef, ring, m_begin, m_end, st);
-}
-
-cudaError_t fwd32_spin(const Plan &p, const Plan::LegShape &sh, const void *coef, void *ring, int m_begin, int m_end,
-                       cudaStream_t st)
-{
-    if (!p.spin) return fwd32_rpt<false>(p, sh, coef, ring, m_begin, m_end, st);
-    if (p.grad) return fwd32_rpt<true, 1, true>(p, sh, coef, ring, m_begin, m_end, st);
-    return fwd32_rpt<true>(p, sh, coef, ring, m_begin, m_end, st);
-}
-
-template <bool SPIN, bool GRAD = false>
-cudaError_t adj32_rpt(const Plan &p, const Plan::LegShape &sh, const void *ring, void *alm, int m_begin, int m_end,
-                      cudaStream_t st, double wpos, void *fx)
-{
-    if (sh.rpt == 1) return adj32_launch<1, SPIN, GRAD>(p, sh, ring, alm, m_begin, m_end, st, wpos, fx);
-    if (sh.rpt == 2) return adj32_launch<2, SPIN, GRAD>(p, sh, ring, alm, m_begin, m_end, st, wpos, fx);
-    return adj32_launch<4, SPIN, GRAD>(p, sh, ring, alm, m_begin, m_end, st, wpos, fx);
-}
-
-cudaError_t adj32_spin(const Plan &p, const Plan::LegShape &sh, const void *ring, void *alm, int m_begin, int m_end,
-                       cudaStream_t st, double wpos, void *fx)
-{
-    if (!p.spin) return adj32_rpt<false>(p, sh, ring, alm, m_begin, m_end, st, wpos, fx);
-    if (p.grad) return adj32_rpt<true, true>(p, sh, ring, alm, m_begin, m_end, st, wpos, fx);
-    return adj32_rpt<true>(p, sh, ring, alm, m_begin, m_end, st, wpos, fx);
-}
-
-template <int RPT> const void *kernel_of32_r(bool spin, bool grad, bool adjoint, int nm)
-{
-    if (adjoint) {
-        if (spin && grad) return (const void *)k_leg_adj32<RPT, true, true>;
-        if (spin) return (const void *)k_leg_adj32<RPT, true>;
-        return (const void *)k_leg_adj32<RPT, false>;
-    }
-    if (nm == 2) return spin ? (const void *)k_leg_fwd32<RPT, true, 2> : (const void *)k_leg_fwd32<RPT, false, 2>;
-    if (nm == 4) return spin ? (const void *)k_leg_fwd32<RPT, true, 4> : (const void *)k_leg_fwd32<RPT, false, 4>;
-    if (spin && grad) return (const void *)k_leg_fwd32<RPT, true, 1, true>;
-    if (spin) return (const void *)k_leg_fwd32<RPT, true>;
-    return (const void *)k_leg_fwd32<RPT, false>;
-}
-
-// Kernel entry of a restarted-FP32 variant (nm > 1: forward sharing the recursion among nm maps)
-const void *kernel_of32(bool spin, bool grad, int rpt, bool adjoint, int nm)
-{
-    if (rpt == 4) return kernel_of32_r<4>(spin, grad, adjoint, nm);
-    if (rpt == 2) return kernel_of32_r<2>(spin, grad, adjoint, nm);
-    return kernel_of32_r<1>(spin, grad, adjoint, nm);
 }
 
 template <class P>
@@ -1660,7 +1475,6 @@ __global__ void __launch_bounds__(256) k_tab_adj(const float2 *__restrict__ ring
     const float sgs = (s & 1) ? -1.f : 1.f;
     const int lf = l0 + 1;
     const double wm = (m > 0 ? wpos : 1.0) * (GRAD ? -0.5 : 1.0);
-    const float wmf = (float)wm;
     const double fxu = fx ? fxs[1 + m] : 0.0;
     float *out = reinterpret_cast<float *>(alm);
     AdjIn<P, kTabG, SPIN, GRAD> in;
@@ -1715,9 +1529,9 @@ __global__ void __launch_bounds__(256) k_tab_adj(const float2 *__restrict__ ring
         if (unit == UPB - 1 || !more) {
             const int blk = lb - unit * kTabS;
             if constexpr (FSPIN)
-                flush_smem<FSPIN, NV>(part, wbuf, out, sc, wm, wmf, base, nalm, m, blk, lmax, sgs, fx, fxu);
+                flush_smem<FSPIN, NV>(part, wbuf, out, sc, wm, base, nalm, m, blk, lmax, sgs, fx, fxu);
             else
-                flush<P, FSPIN, NV>(part, out, sc, wm, wmf, base, nalm, m, blk, lmax, sgs, fx, fxu);
+                flush<P, FSPIN, NV>(part, out, sc, wm, base, nalm, m, blk, lmax, sgs, fx, fxu);
         }
     }
 }
@@ -1754,14 +1568,16 @@ const void *kernel_of_batch(bool spin, int rpt, int nm)
 // the fewest idle ring slots.  nm > 1: the FP32 forward kernel for nm maps.
 Plan::LegShape legendre_shape(const Plan &p, bool adjoint, bool dd, int rpt, int nm)
 {
-    const void *fn = (p.rst && p.prec == LENS_FP32) ? kernel_of32(p.spin != 0, p.grad, rpt, adjoint, nm)
-                     : (nm > 1)            ? kernel_of_batch(p.spin != 0, rpt, nm)
+    const void *fn = (nm > 1)              ? kernel_of_batch(p.spin != 0, rpt, nm)
                      : p.prec == LENS_FP32 ? kernel_of<PolDF>(p.spin != 0, p.grad, rpt, adjoint)
-                     : (dd && p.rst)       ? kernel_of<PolDDR>(p.spin != 0, p.grad, rpt, adjoint)
                      : dd                  ? kernel_of<PolDD>(p.spin != 0, p.grad, rpt, adjoint)
                                            : kernel_of<PolF64>(p.spin != 0, p.grad, rpt, adjoint);
     const int nw = (p.nnorth + 32 * rpt - 1) / (32 * rpt);
     Plan::LegShape best;
+    if (p.rst && (p.prec == LENS_FP32 || dd)) {  // legendre_pk.cu packs its own CTAs
+        best.rpt = rpt;
+        return best;
+    }
     long best_active = -1, best_slots = 0;
     for (int w = 4; w <= 16; ++w) {
         const int chunks = (nw + w - 1) / w;
@@ -1803,12 +1619,15 @@ cudaError_t launch_ck_build(Plan &p, double *a64, double *t64, void *v_out, void
         k_ck_build<false><<<g, 128, 0, p.stream>>>(a64, nullptr, p.scale, p.lognorm, p.rings, p.lmax, p.spin, p.nnorth,
                                                    p.ck.K, p.ck.jb, p.ck.base, v_out, e_out, lt, nullptr);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_ck_clear<<<g, 128, 0, p.stream>>>(lt, p.lmax, p.spin, p.nnorth, p.ck.K, p.ck.base, v_out, e_out, p.spin ? 16 : 8,
+                                        p.ck.klog);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_ck_start<<<p.mmax + 1, 128, 0, p.stream>>>(lt, p.lmax, p.mmax, p.spin, p.nnorth, p.ck.K, p.ck.ngrp, kstart,
                                                  p.ck.klog);
     return cudaGetLastError();
 }
 
-// FP64 plans: restart values of PolDDR from the plan's FP64 recursion tables
+// FP64 plans: restart values (double-float) from the plan's FP64 recursion tables
 cudaError_t launch_ck_build64(Plan &p, void *v_out, void *e_out, int *lt, short *kstart)
 {
     const dim3 g((p.nnorth + 127) / 128, p.mmax + 1);
@@ -1822,6 +1641,9 @@ cudaError_t launch_ck_build64(Plan &p, void *v_out, void *e_out, int *lt, short 
                                                          v_out, e_out, lt, p.ck.klog);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    k_ck_clear<<<g, 128, 0, p.stream>>>(lt, p.lmax, p.spin, p.nnorth, p.ck.K, p.ck.base, v_out, e_out, p.spin ? 32 : 16,
+                                        p.ck.klog);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_ck_start<<<p.mmax + 1, 128, 0, p.stream>>>(lt, p.lmax, p.mmax, p.spin, p.nnorth, p.ck.K, p.ck.ngrp, kstart,
                                                  p.ck.klog);
     return cudaGetLastError();
@@ -1844,20 +1666,36 @@ cudaError_t launch_rec_tables(Plan &p)
 //   FP32 spin 2: fwd 47.4 / 73.4 / 158 and adj 52.4 / 75.6 / 193
 //   FP64 spin 0: fwd 246 / 252 / 295 and adj 258 / 236 / 262
 //   FP64 spin 2: fwd 760 / 700 / 790 and adj 851 / 801 / 916
-// Restarted FP32 recursion (FP32 state, rst), lmax 4096 (ms per launch, fwd / adj):
-//   spin 0: 6.9 / 8.7, 4.8 / 5.9, 4.5 / 5.7 for RPT 1 / 2 / 4
-//   spin 2: 12.3 / 17.1, 14.0 / 15.9, 15.8 / 20.5
-int legendre_rpt(int prec, int spin, bool adjoint, bool rst)
+int legendre_rpt(int prec, int spin, bool adjoint)
 {
-    if (prec == LENS_FP32 && rst) return spin ? (adjoint ? 2 : 1) : 4;
     if (prec == LENS_FP32) return spin ? 1 : 2;
     return spin ? 2 : (adjoint ? 2 : 1);
 }
 
-// df32 part of FP64 plans: twice the accumulator words of the FP32 plans.  Restarted
-// double-float recursion at lmax 4096 (ms, RPT 1 / 2): spin 0 synthesis 20.4 / 19.2,
-// adjoint 29.9 / 27.0; spin 2 synthesis 63.6 / 100.0, adjoint 100.9 / 124.1
-int legendre_rpt_dd(int spin, bool) { return spin ? 1 : 2; }
+// df32 part of FP64 plans without restart values: twice the accumulator words of the FP32 plans
+// (lmax 4096, ms, RPT 1 / 2: spin 0 synthesis 20.4 / 19.2, adjoint 29.9 / 27.0; spin 2 63.6 / 100.0, 100.9 / 124.1)
+int legendre_rpt_dd(int spin) { return spin ? 1 : 2; }
+
+// Plans with restart values (legendre_pk.cuh).  More rings per thread share the staged operands and the flush; fewer
+// leave less of a warp's ring range evanescent and more warps at small lmax.  us per launch, RPT 1 / 2 / 4 (spin 0
+// pairs rings: 2 / 4):
+//   FP32 spin 0 synthesis  lmax 1024 91 / 109, 2048 493 / 465, 4096 3277 / 2994
+//               adjoint    lmax 512 53 / 55, 1024 138 / 133, 2048 889 / 712, 4096 5935 / 4820
+//   FP32 spin 2 synthesis  lmax 512 43 / 51 / 59, 1024 208 / 192 / 215, 2048 1309 / 1147 / 1103, 4096 9368 / 7762 / 7529
+//               adjoint    lmax 256 33 / 35 / 39, 512 76 / 66 / 77, 1024 317 / 240 / 274, 2048 2052 / 1588 / 1393
+//   (gradient-only plans order the same way)
+//   FP64 spin 0 synthesis  lmax 2048 2433 / 2595; adjoint lmax 1024 538 / 577, 2048 3409 / 3110, 4096 23217 / 22097
+//   FP64 spin 2 synthesis  lmax 2048 7219 / 7793, 4096 51343 / 52223; adjoint lmax 2048 10804 / 11049, 4096 77126 / 70401
+int legendre_rpt_pk(int prec, int spin, bool adjoint, int nnorth)
+{
+    if (prec == LENS_FP32) {
+        if (!spin) return nnorth >= (adjoint ? 448 : 768) ? 4 : 2;
+        if (adjoint) return nnorth >= 800 ? 4 : nnorth >= 200 ? 2 : 1;
+        return nnorth >= 800 ? 4 : nnorth >= 400 ? 2 : 1;
+    }
+    if (!spin) return adjoint && nnorth >= 800 ? 4 : 2;
+    return adjoint && nnorth >= 1500 ? 2 : 1;
+}
 
 bool legendre_rpt_supported(int prec, int, bool, int rpt, bool rst)
 {
@@ -1869,17 +1707,19 @@ cudaError_t launch_legendre_fwd(const Plan &p, const void *alm, void *ring, cuda
     // entries with l < spin / columns without rings are never written by the
     // kernel: start from zero
     const size_t eb = p.prec == LENS_FP32 ? 8 : 16;
-    cudaError_t e = cudaMemsetAsync(ring, 0, eb * (size_t)p.ncol * p.ntheta, st);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     const dim3 g(4, p.mmax + 1);
+    if (p.rst) {  // packed kernels: they write every ring of every column
+        if (p.prec == LENS_FP32) return launch_leg_fwd_pk(p, p.leg_f.rpt, alm, ring, 1, wpos, st);
+        k_coef_prep<double2, double2, float4><<<g, 256, 0, st>>>((const double2 *)alm, p.scale, p.coef, p.lmax, p.spin,
+                                                                 p.nalm, 0, wpos, p.grad);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        return launch_leg_fwd_pk(p, p.leg_fd.rpt, p.coef, ring, 1, wpos, st);
+    }
+    if ((e = cudaMemsetAsync(ring, 0, eb * (size_t)p.ncol * p.ntheta, st)) != cudaSuccess) return e;
     if (p.prec == LENS_FP32) {
-        k_coef_prep<float2, float2, float2><<<g, 256, 0, st>>>((const float2 *)alm, p.rst ? nullptr : p.scale, p.coef,
-                                                               p.lmax, p.spin, p.nalm, p.mmax + 1, wpos, p.grad);
-        if (p.rst && !p.tab) {  // the monic plain-form warps' coefficients carry c_l
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            k_coef_prep<float2, float2, float2><<<g, 256, 0, st>>>((const float2 *)alm, p.scale, p.coef_m, p.lmax,
-                                                                   p.spin, p.nalm, p.mmax + 1, wpos, p.grad);
-        }
+        k_coef_prep<float2, float2, float2><<<g, 256, 0, st>>>((const float2 *)alm, p.scale, p.coef, p.lmax, p.spin,
+                                                               p.nalm, p.mmax + 1, wpos, p.grad);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if (p.tab) {
             const dim3 tg(p.tab_fchunks, p.mmax + 1);
@@ -1895,14 +1735,12 @@ cudaError_t launch_legendre_fwd(const Plan &p, const void *alm, void *ring, cuda
             else args(k_tab_fwd<true, false>);
             return cudaGetLastError();
         }
-        if (p.rst) return fwd32_spin(p, p.leg_f, p.coef, ring, 0, p.mmax + 1, st);
         return fwd_spin<PolDF>(p, p.leg_f, p.coef, p.rec_a, p.rec_t, ring, 0, p.mmax + 1, st);
     }
     k_coef_prep<double2, double2, float4><<<g, 256, 0, st>>>((const double2 *)alm, p.scale, p.coef, p.lmax, p.spin,
                                                              p.nalm, p.m_df, wpos, p.grad);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = fwd_spin<PolF64>(p, p.leg_f, p.coef, p.rec_a, p.rec_t, ring, 0, p.m_df, st)) != cudaSuccess) return e;
-    if (p.rst) return fwd_spin<PolDDR>(p, p.leg_fd, p.coef, p.rec_a_df, p.rec_t_df, ring, p.m_df, p.mmax + 1, st);
     return fwd_spin<PolDD>(p, p.leg_fd, p.coef, p.rec_a_df, p.rec_t_df, ring, p.m_df, p.mmax + 1, st);
 }
 
@@ -1910,6 +1748,18 @@ cudaError_t launch_legendre_fwd_batch(const Plan &p, const void *alm, void *ring
                                       double wpos)
 {
     if (p.prec != LENS_FP32 || (nm != 2 && nm != 4)) return cudaErrorInvalidValue;
+    if (p.rst) {
+        // four spin-s maps as two pairs: their sums leave registers for one ring per thread only (lmax 2048: 1159 us
+        // per map against 929, and 1103 alone)
+        const int at = p.spin && nm == 4 ? 2 : nm;
+        for (int b = 0; b < nm; b += at) {
+            const cudaError_t e2 = launch_leg_fwd_pk(p, p.leg_fb[at == 2 ? 0 : 1].rpt,
+                                                     (const float2 *)alm + (size_t)b * p.alm_ncomp() * p.nalm,
+                                                     (float2 *)ring + (size_t)b * p.ncol * p.ntheta, at, wpos, st);
+            if (e2 != cudaSuccess) return e2;
+        }
+        return cudaSuccess;
+    }
     const size_t ring_elems = (size_t)p.ncol * p.ntheta;
     cudaError_t e = cudaMemsetAsync(ring, 0, 8 * ring_elems * nm, st);
     if (e != cudaSuccess) return e;
@@ -1917,8 +1767,7 @@ cudaError_t launch_legendre_fwd_batch(const Plan &p, const void *alm, void *ring
     const dim3 g(4, p.mmax + 1);
     for (int b = 0; b < nm; ++b) {
         k_coef_prep<float2, float2, float2><<<g, 256, 0, st>>>((const float2 *)alm + (size_t)b * ncomp * p.nalm,
-                                                               p.rst ? nullptr : p.scale,
-                                                               (float2 *)coef + (size_t)b * ncomp * p.nalm,
+                                                               p.scale, (float2 *)coef + (size_t)b * ncomp * p.nalm,
                                                                p.lmax, p.spin, p.nalm, p.mmax + 1, wpos, false);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -1943,13 +1792,6 @@ cudaError_t launch_legendre_fwd_batch(const Plan &p, const void *alm, void *ring
         return cudaGetLastError();
     }
     const Plan::LegShape &sh = p.leg_fb[nm == 2 ? 0 : 1];
-    if (p.rst) {
-        if (p.spin)
-            return nm == 2 ? fwd32_rpt<true, 2>(p, sh, coef, ring, 0, p.mmax + 1, st)
-                           : fwd32_rpt<true, 4>(p, sh, coef, ring, 0, p.mmax + 1, st);
-        return nm == 2 ? fwd32_rpt<false, 2>(p, sh, coef, ring, 0, p.mmax + 1, st)
-                       : fwd32_rpt<false, 4>(p, sh, coef, ring, 0, p.mmax + 1, st);
-    }
     if (p.spin) {
         if (sh.rpt == 1)
             return nm == 2 ? fwd_launch<PolDF, 1, true, 2>(p, sh, coef, p.rec_a, p.rec_t, ring, 0, p.mmax + 1, st)
@@ -1995,14 +1837,14 @@ cudaError_t launch_legendre_adj(const Plan &p, const void *ring, void *alm, cuda
         else if (p.grad) args(k_tab_adj<true, true>, warps * tab_smem_per_warp<true, false>());
         else args(k_tab_adj<true, false>, warps * tab_smem_per_warp<true, true>());
         e = cudaGetLastError();
+    } else if (p.rst) {
+        e = launch_leg_adj_pk(p, f32 ? p.leg_a.rpt : p.leg_ad.rpt, ring, alm, wpos, fx, st);
     } else if (f32) {
-        e = p.rst ? adj32_spin(p, p.leg_a, ring, alm, 0, p.mmax + 1, st, wpos, fx)
-                  : adj_spin<PolDF>(p, p.leg_a, ring, p.rec_a, p.rec_t, alm, 0, p.mmax + 1, st, wpos, fx);
+        e = adj_spin<PolDF>(p, p.leg_a, ring, p.rec_a, p.rec_t, alm, 0, p.mmax + 1, st, wpos, fx);
     } else {
         e = adj_spin<PolF64>(p, p.leg_a, ring, p.rec_a, p.rec_t, alm, 0, p.m_df, st, wpos, fx);
         if (e == cudaSuccess)
-            e = p.rst ? adj_spin<PolDDR>(p, p.leg_ad, ring, p.rec_a_df, p.rec_t_df, alm, p.m_df, p.mmax + 1, st, wpos, fx)
-                      : adj_spin<PolDD>(p, p.leg_ad, ring, p.rec_a_df, p.rec_t_df, alm, p.m_df, p.mmax + 1, st, wpos, fx);
+            e = adj_spin<PolDD>(p, p.leg_ad, ring, p.rec_a_df, p.rec_t_df, alm, p.m_df, p.mmax + 1, st, wpos, fx);
     }
     if (e != cudaSuccess || !p.det) return e;
     const dim3 g(4, p.mmax + 1);

@@ -17,8 +17,9 @@
 #include "internal.h"
 
 namespace gsl {
-int legendre_rpt(int prec, int spin, bool adjoint, bool rst);
-int legendre_rpt_dd(int spin, bool adjoint);
+int legendre_rpt(int prec, int spin, bool adjoint);
+int legendre_rpt_dd(int spin);
+int legendre_rpt_pk(int prec, int spin, bool adjoint, int nnorth);
 bool legendre_rpt_supported(int prec, int spin, bool adjoint, int rpt, bool rst);
 }
 
@@ -577,7 +578,7 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
             const double jr = acos(0.7) / kPi * (nt - 1);
             p->ck.jb = (int)std::ceil(jr / 128.0) * 128;
         }
-        // FP64 plans whose epsilon admits df32 orders: every order in df32 (PolDDR), restarted
+        // FP64 plans whose epsilon admits df32 orders: every order in df32 (PkD), restarted
         // every K = 128 degrees from the FP64 recursion, so that no order runs on the FP64 pipe
         // (1/60 of the FP32 rate on GB300); the FP64 orders of m_df are not needed then
         const bool mdf_set = prm && prm->legendre_df32_mmin != 0;  // explicit FP64 orders: no restarts
@@ -619,15 +620,16 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
         const int want = prm ? (adj ? prm->legendre_rpt_adj : prm->legendre_rpt_fwd) : 0;
         if (want && !legendre_rpt_supported(prec, spin, adj != 0, want, p->rst))
             return bail(LENS_ERR_INVALID, "unsupported Legendre rings-per-thread setting");
-        (adj ? p->leg_a : p->leg_f) =
-            legendre_shape(*p, adj != 0, false, want ? want : legendre_rpt(prec, spin, adj != 0, p->rst));
+        const int pk = p->rst ? legendre_rpt_pk(prec, spin, adj != 0, p->nnorth) : 0;
+        (adj ? p->leg_a : p->leg_f) = legendre_shape(
+            *p, adj != 0, false, want ? want : pk && prec == LENS_FP32 ? pk : legendre_rpt(prec, spin, adj != 0));
         if (prec == LENS_FP64)
             (adj ? p->leg_ad : p->leg_fd) =
-                legendre_shape(*p, adj != 0, true, (want && want <= 2) ? want : legendre_rpt_dd(spin, adj != 0));
+                legendre_shape(*p, adj != 0, true, (want && want <= 2) ? want : pk ? pk : legendre_rpt_dd(spin));
     }
     if (prec == LENS_FP32) {  // synthesis of 2 / 4 maps sharing one recursion
         p->leg_fb[0] = legendre_shape(*p, false, false, p->leg_f.rpt, 2);
-        p->leg_fb[1] = legendre_shape(*p, false, false, 1, 4);
+        p->leg_fb[1] = legendre_shape(*p, false, false, p->rst ? p->leg_f.rpt : 1, 4);
     }
 
     cudaError_t e;
@@ -646,9 +648,9 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
         std::vector<int64_t> cb(mmax + 1);
         int64_t off = 0;
         for (int m = 0; m <= mmax; ++m) {
-            cb[m] = off;
+            cb[m] = off + p->nnorth;  // the row before holds the start values
             const int Km = p->ck_klog.empty() ? p->ck.K : 1 << p->ck_klog[m];
-            off += (int64_t)ck_count(lmax, std::max(m, spin) + 1, Km) * p->nnorth;
+            off += (int64_t)(1 + ck_count(lmax, std::max(m, spin) + 1, Km)) * p->nnorth;
         }
         void *d = nullptr;
         if ((e = B.upload(&d, cb)) != cudaSuccess) return bailc(e, "upload restart offsets");
@@ -661,11 +663,14 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
         if ((e = B.alloc(&d, sizeof(short) * (size_t)(mmax + 1) * p->ck.ngrp, false)) != cudaSuccess)
             return bailc(e, "alloc restart starts");
         p->ck.kstart = (const short *)d;
-        if (p->ck_bytes > 0) {
-            // values (FP32 plans 8 / 16 bytes, FP64 plans 16 / 32) and exponents (2 / 4 bytes) per entry
+        {
+            // values (FP32 plans 8 / 16 bytes, FP64 plans 16 / 32) and exponents (2 / 4 bytes) per entry;
+            // ck_bytes counts the restarts' rows, without the start values' (one row per order)
+            const size_t vsz = (prec == LENS_FP32 ? 8 : 16) * (spin ? 2 : 1), vbytes = vsz * (size_t)off;
             const size_t ebytes = p->ck_bytes / (prec == LENS_FP32 ? 4 : 8);
             void *dv = nullptr, *de = nullptr;
-            if ((e = B.alloc(&dv, p->ck_bytes, false)) != cudaSuccess || (e = B.alloc(&de, ebytes, false)) != cudaSuccess) {
+            if ((e = B.alloc(&dv, vbytes, false)) != cudaSuccess ||
+                (e = B.alloc(&de, (spin ? 4 : 2) * (size_t)off, false)) != cudaSuccess) {
                 if (e == cudaErrorMemoryAllocation) {
                     cudaGetLastError();
                     return bail(LENS_ERR_NOMEM, "Legendre restart values: " + std::to_string((p->ck_bytes + ebytes) >> 20) +
@@ -682,12 +687,12 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
         if ((e = B.alloc(&p->rec_a_df, (size_t)p->nalm * (spin ? 16 : 8), false)) != cudaSuccess)
             return bailc(e, "alloc rec_a_df");
     }
-    if ((e = B.alloc(&p->coef, (size_t)p->nalm * esz * ncomp, true)) != cudaSuccess) return bailc(e, "alloc coef");
-    if (p->rst && prec == LENS_FP32) {  // monic plain-form rings: c_l a_lm and the (c_l, 1/c_l) table
+    if (!(p->rst && prec == LENS_FP32) && (e = B.alloc(&p->coef, (size_t)p->nalm * esz * ncomp, true)) != cudaSuccess)
+        return bailc(e, "alloc coef");
+    if (p->rst && prec == LENS_FP32) {  // monic plain-form rings: the c_l table
         void *d = nullptr;
-        if ((e = B.alloc(&p->coef_m, (size_t)p->nalm * esz * ncomp, true)) != cudaSuccess ||
-            (e = B.alloc(&d, (size_t)p->nalm * sizeof(float2), false)) != cudaSuccess)
-            return bailc(e, "alloc monic coefficients");
+        if ((e = B.alloc(&d, (size_t)p->nalm * sizeof(float2), false)) != cudaSuccess)
+            return bailc(e, "alloc monic scale");
         p->ck.cs = (const float2 *)d;
     }
     const ScratchSizes scr = plan_scratch_sizes(*p);
@@ -832,7 +837,7 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
     if ((e = launch_rec_tables(*p)) != cudaSuccess) return bailc(e, "recursion tables");
     if (p->rst) {  // (FP32: step table, then) restart values from the FP64 recursion
         if (prec == LENS_FP32 && (e = launch_rec_tables_s(*p)) != cudaSuccess) return bailc(e, "restart step table");
-        if (p->ck_bytes > 0) {
+        {
             // temporaries: FP64 alpha and tau [nalm] each (FP32 plans; FP64 plans have their own),
             // first significant degree [mmax + 1][nnorth]
             const size_t tb = (size_t)p->nalm * 16 + sizeof(int) * (size_t)(mmax + 1) * p->nnorth;
@@ -864,9 +869,6 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
             }
             cudaFree(tmp);
             if (e != cudaSuccess) return bailc(e, "restart values");
-        } else if ((e = cudaMemsetAsync(const_cast<short *>(p->ck.kstart), 0,
-                                        sizeof(short) * (size_t)(mmax + 1) * p->ck.ngrp, p->stream)) != cudaSuccess) {
-            return bailc(e, "restart starts");
         }
     }
     if (p->tab) {
