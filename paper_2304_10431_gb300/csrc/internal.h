@@ -16,6 +16,10 @@ constexpr int kScaleBits = 60;       // exponent step of the scaled Legendre rec
 constexpr int kLegBlock = 8;         // degrees per unrolled block of the Legendre kernels
 constexpr int kTileR = 32, kTileC = 32;  // default grid tile of the point sort (rows x columns)
 constexpr int kMaxW = 16;                 // largest kernel support
+// Double-float kernel weights of a point: the theta taps in pairs (h0, h1, l0, l1), one operand pair of a packed
+// instruction per 8 bytes, then the phi taps (h, l); both padded with zeros to an even count.
+__host__ __device__ constexpr int dd_pairs(int W) { return (W + 1) / 2; }
+__host__ __device__ constexpr int dd_words(int W) { return 8 * dd_pairs(W); }  // FP32 words of one point
 
 // FP32 plans: the weight of kernel tap a (0 <= a < W) as a polynomial of degree W + 1 in
 // t = 2 frac - (W - 1), t in [-1, 1] (frac = u - ceil(u - W/2) in (W/2 - 1, W/2]);
@@ -184,9 +188,11 @@ struct Plan {
     int ntile_c = 0, ntiles = 0;     // tiles per grid row band, total tiles
     int tile_r = kTileR;             // rows of a tile (16, 32 or 64; 32 columns)
     void *phase = nullptr;     // float2 / double2 e^{i s chi}, spin != 0 only
+    int tile_c = kTileC;             // columns of a tile: 32; FP64 plans that spread by strips 33 - W
+    bool strip = false;              // spreading by strips (nufft_strip.cuh): points sorted by tile, then by row
     double *wts = nullptr;     // FP64 plans: [npts][2W] kernel weights (theta taps, then phi taps)
-    bool wts_dd = false;       // weights as double-float pairs; double-float interpolation and
-                               // spreading taps (FP64 plans with epsilon >= 5e-11)
+    bool wts_dd = false;       // weights as double-float pairs (layout: dd_words, nufft.cuh); double-float
+                               // interpolation and spreading taps (FP64 plans with epsilon >= 5e-11)
 
     // per-call workspace
     void *ring = nullptr;      // [ncol][ntheta] complex

@@ -30,7 +30,7 @@ __device__ __forceinline__ int grid_coord(double t, double2 c, double hw, double
 
 __global__ void k_prep(const double *__restrict__ theta, const double *__restrict__ phi,
                        const double *__restrict__ chi, int64_t n, int N1, int N2, int W, int r_lo, int R, int pitch,
-                       int spin, double2 c1, double2 c2, int tile_r, uint32_t *__restrict__ key,
+                       int spin, double2 c1, double2 c2, int tile_r, int tile_c, int rows, uint32_t *__restrict__ key,
                        int32_t *__restrict__ idx, uint32_t *__restrict__ cell_u, double2 *__restrict__ frac_u,
                        double2 *__restrict__ phase_u, unsigned *__restrict__ flags)
 {
@@ -59,8 +59,9 @@ __global__ void k_prep(const double *__restrict__ theta, const double *__restric
     }
     cell_u[i] = (uint32_t)row * (uint32_t)pitch + (uint32_t)j0;
     frac_u[i] = make_double2(fu, fv);
-    const int ntc = (N2 + kTileC - 1) / kTileC;
-    key[i] = (uint32_t)(row / tile_r) * (uint32_t)ntc + (uint32_t)(j0 / kTileC);
+    const int ntc = (N2 + tile_c - 1) / tile_c;
+    const uint32_t tile = (uint32_t)(row / tile_r) * (uint32_t)ntc + (uint32_t)(j0 / tile_c);
+    key[i] = rows ? tile * (uint32_t)tile_r + (uint32_t)(row % tile_r) : tile;  // rows: by cell row within the tile
     idx[i] = (int32_t)i;
     if (spin) {
         const double c = chi ? chi[i] : 0.0;
@@ -89,14 +90,14 @@ __global__ void k_gather_points(const int32_t *__restrict__ perm, int64_t n, con
     }
 }
 
-// start[t] = first sorted point whose tile key is >= t, t = 0..ntiles (the
+// start[t] = first sorted point whose tile (key / per) is >= t, t = 0..ntiles (the
 // ranges (key[p-1], key[p]] partition 0..ntiles, so each entry is written once)
-__global__ void k_tile_bounds(const uint32_t *__restrict__ skey, int64_t n, int ntiles, uint32_t *__restrict__ start)
+__global__ void k_tile_bounds(const uint32_t *__restrict__ skey, int64_t n, int ntiles, int per, uint32_t *__restrict__ start)
 {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p > n) return;
-    const int64_t lo = p == 0 ? -1 : (int64_t)skey[p - 1];
-    const int64_t hi = p == n ? (int64_t)ntiles : (int64_t)skey[p];
+    const int64_t lo = p == 0 ? -1 : (int64_t)(skey[p - 1] / per);
+    const int64_t hi = p == n ? (int64_t)ntiles : (int64_t)(skey[p] / per);
     for (int64_t t = lo + 1; t <= hi; ++t) start[t] = (uint32_t)p;
 }
 
@@ -112,18 +113,25 @@ __global__ void k_weights(const double2 *__restrict__ frac, int64_t n, int W, do
     if (p >= n) return;
     const double2 f = frac[p];
     const double twoW = 2.0 / W;
-    double *wd = wts + p * 2 * W;
-    float2 *w = reinterpret_cast<float2 *>(wd);
-    for (int a = 0; a < W; ++a) {
-        const double x = es_kernel<double>(f.x - a, twoW, beta), y = es_kernel<double>(f.y - a, twoW, beta);
-        if (dd) {
-            const df32 xs = df_split(x), ys = df_split(y);
-            w[a] = make_float2(xs.h, xs.l);
-            w[W + a] = make_float2(ys.h, ys.l);
-        } else {
-            wd[a] = x;
-            wd[W + a] = y;
+    if (dd) {  // layout: dd_words
+        const int np = dd_pairs(W);
+        float4 *w = reinterpret_cast<float4 *>(reinterpret_cast<float *>(wts) + p * dd_words(W));
+        for (int i = 0; i < np; ++i) {
+            df32 x[2], y[2];
+            for (int k = 0; k < 2; ++k) {
+                const int a = 2 * i + k;
+                x[k] = df_split(a < W ? es_kernel<double>(f.x - a, twoW, beta) : 0.0);
+                y[k] = df_split(a < W ? es_kernel<double>(f.y - a, twoW, beta) : 0.0);
+            }
+            w[i] = make_float4(x[0].h, x[1].h, x[0].l, x[1].l);
+            w[np + i] = make_float4(y[0].h, y[0].l, y[1].h, y[1].l);
         }
+        return;
+    }
+    double *wd = wts + p * 2 * W;
+    for (int a = 0; a < W; ++a) {
+        wd[a] = es_kernel<double>(f.x - a, twoW, beta);
+        wd[W + a] = es_kernel<double>(f.y - a, twoW, beta);
     }
 }
 
@@ -133,7 +141,8 @@ __global__ void k_weights(const double2 *__restrict__ frac, int64_t n, int W, do
 // for every cell of the tile and its halo.
 template <int W>
 __global__ void __launch_bounds__(256) k_tile_window_kmax(const uint32_t *__restrict__ cell, int pitch, int ntc,
-                                                         int tile_r, const uint32_t *__restrict__ tile_start,
+                                                         int tile_r,
+                                                         const uint32_t *__restrict__ tile_start,
                                                          unsigned short *__restrict__ out)
 {
     constexpr int TC = kTileC + W - 1;
@@ -328,12 +337,14 @@ cudaError_t launch_prep_points(Plan &p, const double *theta, const double *phi, 
         return make_double2(hi, q2 - (hi - q1));
     };
     k_prep<<<blocks, thr, 0, st>>>(theta, phi, chi, n, p.N1, p.N2, p.W, p.r_lo, p.R, p.pitch, p.spin, scale_of(p.N1),
-                                   scale_of(p.N2), p.tile_r, key, idx, cell_u, frac_u, phase_u, p.flags);
+                                   scale_of(p.N2), p.tile_r, p.tile_c, p.strip ? 1 : 0, key, idx, cell_u, frac_u, phase_u, p.flags);
     GSL_TRY(cudaGetLastError());
-    const int ntc = (p.N2 + kTileC - 1) / kTileC;
+    const int ntc = p.ntile_c;
+    const int per = p.strip ? p.tile_r : 1;
     const uint64_t nkeys = (uint64_t)((p.R + p.tile_r - 1) / p.tile_r) * ntc;
+    if (nkeys * per > 0xffffffffull) { cleanup(); err = "internal: tile keys above 32 bits"; return cudaErrorInvalidValue; }
     int bits = 1;
-    while (bits < 32 && (1ull << bits) < nkeys) ++bits;
+    while (bits < 32 && (1ull << bits) < nkeys * per) ++bits;
     GSL_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tmp_bytes, key, key2, idx, p.perm, (int)n, 0, bits, st));
     GSL_TRY(cudaMalloc(&tmp, tmp_bytes));
     GSL_TRY(cub::DeviceRadixSort::SortPairs(tmp, tmp_bytes, key, key2, idx, p.perm, (int)n, 0, bits, st));
@@ -341,7 +352,7 @@ cudaError_t launch_prep_points(Plan &p, const double *theta, const double *phi, 
                                             p.phase);
     GSL_TRY(cudaGetLastError());
     if (nkeys != (uint64_t)p.ntiles) { cleanup(); err = "internal: tile count mismatch"; return cudaErrorInvalidValue; }
-    k_tile_bounds<<<(unsigned)((n + 1 + thr - 1) / thr), thr, 0, st>>>(key2, n, p.ntiles, p.tile_start);
+    k_tile_bounds<<<(unsigned)((n + 1 + thr - 1) / thr), thr, 0, st>>>(key2, n, p.ntiles, per, p.tile_start);
     GSL_TRY(cudaGetLastError());
     if (p.det) {
         GSL_TRY(cudaMemsetAsync(p.fx_kmax, 0, sizeof(uint32_t), st));

@@ -51,8 +51,6 @@ constexpr int kSpreadThreads = 64;
 // FP64 tiles hold 64-bit cells (31 KB at W = 13, seven CTAs per SM): 256 threads keep
 // more warps in flight per tile
 constexpr int kSpreadThreads64 = 256;
-// FP64 double-float spreading tiles stage this many points at a time (offset + value pair)
-constexpr int kDDBatch = 512;
 
 // the ES kernel of tap offset z (FP64 plans)
 template <typename T> __device__ __forceinline__ T es_kernel(T z, T twoW, T beta)
@@ -85,6 +83,20 @@ __device__ __forceinline__ df32 ld_df(const float2 *p)
     const float2 v = __ldg(p);
     return {v.x, v.y};
 }
+// double-float weights of sorted point p: theta tap a, phi tap b
+template <int W> __device__ __forceinline__ const float *dd_weights(const double *wts, int64_t p)
+{
+    return reinterpret_cast<const float *>(wts) + p * dd_words(W);
+}
+template <int W> __device__ __forceinline__ df32 dd_theta(const float *w, int a)
+{
+    const float *q = w + 4 * (a >> 1) + (a & 1);
+    return {__ldg(q), __ldg(q + 2)};
+}
+template <int W> __device__ __forceinline__ df32 dd_phi(const float *w, int b)
+{
+    return ld_df(reinterpret_cast<const float2 *>(w + 4 * dd_pairs(W)) + b);
+}
 
 // PRE: 0 evaluate the kernel, 1 read the double weights, 2 the double-float pairs
 template <typename T, int W, int PRE>
@@ -99,11 +111,11 @@ __device__ __forceinline__ void tap_weights(T (&wa)[W], T (&wb)[W], const cplx<T
             wb[a] = (T)__ldg(w + W + a);
         }
     } else if (PRE == 2) {
-        const float2 *w = reinterpret_cast<const float2 *>(wts) + p * 2 * W;
+        const float *w = dd_weights<W>(wts, p);
 #pragma unroll
         for (int a = 0; a < W; ++a) {
-            wa[a] = (T)df_value(ld_df(w + a));
-            wb[a] = (T)df_value(ld_df(w + W + a));
+            wa[a] = (T)df_value(dd_theta<W>(w, a));
+            wb[a] = (T)df_value(dd_phi<W>(w, a));
         }
     } else if constexpr (std::is_same<T, float>::value) {
         const float tx = fmaf(2.f, f.x, -(float)(W - 1)), ty = fmaf(2.f, f.y, -(float)(W - 1));
@@ -182,10 +194,10 @@ __global__ void __launch_bounds__(256) k_interp_dd(const void *__restrict__ grid
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const uint32_t c0 = cell[p];
-    const float2 *w = reinterpret_cast<const float2 *>(wts) + p * 2 * W;
+    const float *w = dd_weights<W>(wts, p);
     df32 wb[W];
 #pragma unroll
-    for (int b = 0; b < W; ++b) wb[b] = ld_df(w + W + b);
+    for (int b = 0; b < W; ++b) wb[b] = dd_phi<W>(w, b);
     const int32_t dst = perm[p];
     if (!SPIN) {
         const float2 *g = reinterpret_cast<const float2 *>(grid) + c0;
@@ -195,7 +207,7 @@ __global__ void __launch_bounds__(256) k_interp_dd(const void *__restrict__ grid
             df32 r = {0.f, 0.f};
 #pragma unroll
             for (int b = 0; b < W; ++b) df_acc(r, df_mul(wb[b], ld_df(g + (int64_t)a * pitch + b)));
-            df_acc(acc, df_mul(ld_df(w + a), df_renorm(r)));
+            df_acc(acc, df_mul(dd_theta<W>(w, a), df_renorm(r)));
         }
         map[dst] = df_value(acc);
     } else {
@@ -210,7 +222,7 @@ __global__ void __launch_bounds__(256) k_interp_dd(const void *__restrict__ grid
                 df_acc(rx, df_mul(wb[b], df32{v.x, v.y}));
                 df_acc(ry, df_mul(wb[b], df32{v.z, v.w}));
             }
-            const df32 wa = ld_df(w + a);
+            const df32 wa = dd_theta<W>(w, a);
             df_acc(ax, df_mul(wa, df_renorm(rx)));
             df_acc(ay, df_mul(wa, df_renorm(ry)));
         }
@@ -221,8 +233,8 @@ __global__ void __launch_bounds__(256) k_interp_dd(const void *__restrict__ grid
     }
 }
 
-// one thread per sorted point, one global atomic per tap (FP64 plans); FX:
-// fixed-point integers into the same grid memory (scale *fxs)
+// one thread per sorted point, one global atomic per tap (deterministic FP64 plans):
+// fixed-point integers into the grid memory (scale *fxs)
 template <typename T, bool FX> struct Acc {
     using type = T;
 };
@@ -236,7 +248,7 @@ __device__ __forceinline__ void acc_add(typename Acc<T, FX>::type *dst, T v, T s
     else atomicAdd(dst, v);
 }
 
-template <typename T, int W, bool SPIN, int PRE, bool FX>
+template <typename T, int W, bool SPIN, int PRE>
 __global__ void __launch_bounds__(256) k_spread_direct(void *__restrict__ grid, const uint32_t *__restrict__ cell,
                                                        const cplx<T> *__restrict__ frac,
                                                        const int32_t *__restrict__ perm,
@@ -245,10 +257,10 @@ __global__ void __launch_bounds__(256) k_spread_direct(void *__restrict__ grid, 
                                                        int64_t n, int pitch, T beta, const double *__restrict__ fxs,
                                                        const __grid_constant__ KerPoly kp)
 {
-    using G = typename Acc<T, FX>::type;
+    using G = typename Acc<T, true>::type;
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
-    const T sc = FX ? (T)fxs[0] : T(1);
+    const T sc = (T)fxs[0];
     const uint32_t c0 = cell[p];
     T wa[W], wb[W];
     tap_weights<T, W, PRE>(wa, wb, PRE ? cplx<T>{} : frac[p], wts, p, beta, kp);
@@ -260,7 +272,7 @@ __global__ void __launch_bounds__(256) k_spread_direct(void *__restrict__ grid, 
         for (int a = 0; a < W; ++a) {
             const T xa = wa[a] * x;
 #pragma unroll
-            for (int b = 0; b < W; ++b) acc_add<T, FX>(g + (int64_t)a * pitch + b, xa * wb[b], sc);
+            for (int b = 0; b < W; ++b) acc_add<T, true>(g + (int64_t)a * pitch + b, xa * wb[b], sc);
         }
     } else {
         // e^{-i s chi} (Q + i U)
@@ -274,8 +286,8 @@ __global__ void __launch_bounds__(256) k_spread_direct(void *__restrict__ grid, 
 #pragma unroll
             for (int b = 0; b < W; ++b) {
                 G *q2 = g + 2 * ((int64_t)a * pitch + b);
-                acc_add<T, FX>(q2, xa * wb[b], sc);
-                acc_add<T, FX>(q2 + 1, ya * wb[b], sc);
+                acc_add<T, true>(q2, xa * wb[b], sc);
+                acc_add<T, true>(q2 + 1, ya * wb[b], sc);
             }
         }
     }
@@ -297,18 +309,6 @@ template <typename T, bool FX, bool IT> struct SAcc { using type = typename Acc<
 template <> struct SAcc<float, false, true> { using type = int; };
 template <> struct SAcc<double, false, true> { using type = long long; };
 __device__ __forceinline__ int tile_int(float v) { return __float2int_rn(v); }
-// A double-float term (p, e) with |p| < 2^53 as a 64-bit integer (nearest) without
-// 64-bit conversions (those run at GB300's FP64 rate): p = p1 + p2 with p1 a multiple
-// of 2^31 (|p1| / 2^31 < 2^22, read off the bits of p1 / 2^31 + 1.5 * 2^23) and
-// |p2| <= 2^30 exact, then p2 and e by 32-bit conversions
-__device__ __forceinline__ long long dd_tile_int(df32 t)
-{
-    const float big = 0x1.8p54f;  // 1.5 * 2^54: t.h + big rounds t.h to a multiple of 2^31
-    const float p1 = __fsub_rn(__fadd_rn(t.h, big), big);
-    const int i1 = __float_as_int(__fmaf_rn(p1, 0x1p-31f, 12582912.0f)) - 0x4B400000;
-    const float p2 = __fsub_rn(t.h, p1);
-    return ((long long)i1 << 31) + (long long)__float2int_rn(p2) + (long long)__float2int_rn(t.l);
-}
 __device__ __forceinline__ long long tile_int(double v) { return __double2ll_rn(v); }
 __device__ __forceinline__ void tile_add(int *dst, int v) { atomicAdd(dst, v); }
 __device__ __forceinline__ void tile_add(long long *dst, long long v)
@@ -331,7 +331,6 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
 {
     static_assert(!(IT && FX), "fixed-point tiles or fixed-point grid");
     using G = typename SAcc<T, FX, IT>::type;
-    constexpr bool DD = std::is_same<T, double>::value && IT && PRE == 2;  // double-float taps
     constexpr int TC = kTileC + W - 1, NC = SPIN ? 2 : 1;
     const int TR = tile_r + W - 1;  // tile rows (16, 32 or 64) plus the kernel halo
     extern __shared__ __align__(16) unsigned char spread_smem[];
@@ -342,7 +341,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
     T sc = FX ? (T)fxs[0] : T(1);
     bool bad = false;  // IT: non-finite map value
     if constexpr (IT) {
-        constexpr int kBits = sizeof(T) == 4 ? 30 : DD ? 53 : 62;  // tile sums of |terms| below 2^kBits
+        constexpr int kBits = sizeof(T) == 4 ? 30 : 62;  // tile sums of |terms| below 2^kBits
         const double bound = (double)tile_kmax[t] * __longlong_as_double((long long)*maxbits);
         if (!(bound < 1e300)) bad = true;  // infinity or NaN in the map
         else if (bound > 0.0) sc = (T)ldexp(1.0, kBits - (ilogb(bound) + 1));  // bound < 2^(ilogb+1)
@@ -350,52 +349,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
     for (int i = threadIdx.x; i < TR * TC * NC; i += blockDim.x) buf[i] = G(0);
     __syncthreads();
     const int r0 = (t / ntc) * tile_r, c0 = (t % ntc) * kTileC;
-    if constexpr (DD && SPIN) {
-        // FP64 plans with point weights, spin s: work items (point, kernel row) instead of points, so
-        // that the threads of a tile finish together (a tile holds 2-3 points per thread, and
-        // one point per thread more meant a wait at the barrier) and the unrolled body is one
-        // row of W taps.  Per batch of points: each point's value times the unit (exact) as a
-        // double-float pair and its cell offset in shared memory; then the items.  Each tap is
-        // the double-float product of the row value and the weight pair (~2^-46 relative),
-        // rounded to an integer by dd_tile_int (tile sums of |terms| below 2^53).
-        int *soff = reinterpret_cast<int *>(buf + ((TR * TC * NC + 1) & ~1));  // 16-byte aligned
-        float4 *sval = reinterpret_cast<float4 *>(soff + kDDBatch);
-        for (uint32_t pb = p0; pb < (bad ? p0 : p1); pb += kDDBatch) {
-            const int nb = (int)min((uint32_t)kDDBatch, p1 - pb);
-            for (int q = threadIdx.x; q < nb; q += blockDim.x) {
-                const uint32_t p = pb + q;
-                const uint32_t c = cell[p];
-                const int lr = (int)(c / (uint32_t)pitch) - r0, lc = (int)(c % (uint32_t)pitch) - c0;
-                const bool mine = (unsigned)lr < (unsigned)tile_r && (unsigned)lc < (unsigned)kTileC;
-                soff[q] = mine ? lr * TC + lc : -1;
-                if (!mine) continue;
-                const int32_t src = perm[p];
-                const cplx<T> ph = phase[p];
-                const T qv = map[src], u = map[n + src];
-                const df32 zx = df_split((ph.x * qv + ph.y * u) * sc), zy = df_split((ph.x * u - ph.y * qv) * sc);
-                sval[q] = make_float4(zx.h, zx.l, zy.h, zy.l);
-            }
-            __syncthreads();
-            for (int it = threadIdx.x; it < nb * W; it += blockDim.x) {
-                const int q = it / W, a = it - q * W;
-                const int off = soff[q];
-                if (off < 0) continue;
-                const float2 *w = reinterpret_cast<const float2 *>(wts) + (int64_t)(pb + q) * 2 * W;
-                const df32 wa = ld_df(w + a);
-                const float4 v = sval[q];
-                G *row = buf + off + a * TC;
-                const df32 xa = df_renorm(df_mul(wa, df32{v.x, v.y})), ya = df_renorm(df_mul(wa, df32{v.z, v.w}));
-#pragma unroll
-                for (int b = 0; b < W; ++b) {
-                    const df32 wb = ld_df(w + W + b);
-                    tile_add(row + b, dd_tile_int(df_mul(xa, wb)));
-                    tile_add(row + b + TR * TC, dd_tile_int(df_mul(ya, wb)));
-                }
-            }
-            __syncthreads();  // the batch's staging is rewritten next
-        }
-    }
-    for (uint32_t p = p0 + threadIdx.x; p < ((bad || (DD && SPIN)) ? p0 : p1); p += blockDim.x) {
+    for (uint32_t p = p0 + threadIdx.x; p < (bad ? p0 : p1); p += blockDim.x) {
         const uint32_t c = cell[p];
         const int lr = (int)(c / (uint32_t)pitch) - r0, lc = (int)(c % (uint32_t)pitch) - c0;
         if ((unsigned)lr >= (unsigned)tile_r || (unsigned)lc >= (unsigned)kTileC) continue;  // not this tile's
@@ -403,24 +357,6 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
         // spin s: two planes (real parts, then imaginary parts), so that the lanes'
         // atomics of one plane spread over all 32 banks
         G *b0 = buf + (lr * TC + lc);
-        if constexpr (DD && !SPIN) {
-            // FP64 plans with point weights, spin 0: the value (times the unit, exact) as a
-            // double-float pair, each tap the double-float product with the pair of weights
-            // (~2^-46 relative), rounded to an integer by dd_tile_int (tile sums of |terms|
-            // below 2^53)
-            const float2 *w = reinterpret_cast<const float2 *>(wts) + (int64_t)p * 2 * W;
-            df32 wb[W];
-#pragma unroll
-            for (int b = 0; b < W; ++b) wb[b] = ld_df(w + W + b);
-            const df32 x = df_split(map[src] * sc);
-#pragma unroll
-            for (int a = 0; a < W; ++a) {
-                const df32 xa = df_renorm(df_mul(ld_df(w + a), x));
-#pragma unroll
-                for (int b = 0; b < W; ++b) tile_add(b0 + a * TC + b, dd_tile_int(df_mul(xa, wb[b])));
-            }
-            continue;
-        }
         T wa[W], wb[W];
         tap_weights<T, W, PRE>(wa, wb, PRE ? cplx<T>{} : frac[p], wts, p, beta, kp);
         // IT: the power-of-two unit sc is applied to the point's value first (exact)
@@ -493,6 +429,8 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
     }
 }
 
+template <int W, bool SPIN> cudaError_t spread_strip(const Plan &p, const void *map, void *grid, cudaStream_t st);
+
 template <typename T, bool SPIN, int W>
 cudaError_t interp_w(const Plan &p, const void *grid, void *map, cudaStream_t st)
 {
@@ -531,20 +469,9 @@ cudaError_t spread_w(const Plan &p, const void *map, void *grid, cudaStream_t st
         return cudaGetLastError();
     };
     if constexpr (std::is_same<T, double>::value) {
-        if (!p.det && p.tile_kmax) {  // 64-bit integer tiles (double-float taps with double-float weights)
-            if (p.wts && p.wts_dd && SPIN) {  // plus the staged points: int offset and float4 value each
-                const size_t extra = (size_t)kDDBatch * (sizeof(int) + sizeof(float4));
-                const auto kern = k_spread<T, W, SPIN, 2, false, true>;
-                const size_t sm = ((cells + 1) & ~(size_t)1) * 8 + extra;
-                cudaError_t e2 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-                if (e2 != cudaSuccess) return e2;
-                kern<<<(unsigned)p.ntiles, kSpreadThreads64, sm, st>>>(
-                    grid, p.cell, (const cplx<T> *)p.frac, p.perm, (const cplx<T> *)p.phase, p.wts, (const T *)map,
-                    p.npts, p.pitch, p.R, p.ntile_c, p.tile_start, (T)p.beta, fxs, p.tile_r, p.tile_kmax, p.maxbits,
-                    p.kpoly);
-                return cudaGetLastError();
-            }
-            if (p.wts && p.wts_dd) return run(k_spread<T, W, SPIN, 2, false, true>, 8);
+        if (!p.det) {
+            if (p.strip) return spread_strip<W, SPIN>(p, map, grid, st);
+            // 64-bit integer tiles
             if (p.wts) return run(k_spread<T, W, SPIN, 1, false, true>, 8);
             return run(k_spread<T, W, SPIN, 0, false, true>, 8);
         }
@@ -555,14 +482,8 @@ cudaError_t spread_w(const Plan &p, const void *map, void *grid, cudaStream_t st
                                          (T)p.beta, fxs, p.kpoly);
             return cudaGetLastError();
         };
-        if (p.det) {
-            if (p.wts) return p.wts_dd ? direct(k_spread_direct<T, W, SPIN, 2, true>)
-                                       : direct(k_spread_direct<T, W, SPIN, 1, true>);
-            return direct(k_spread_direct<T, W, SPIN, 0, true>);
-        }
-        if (p.wts) return p.wts_dd ? direct(k_spread_direct<T, W, SPIN, 2, false>)
-                                   : direct(k_spread_direct<T, W, SPIN, 1, false>);
-        return direct(k_spread_direct<T, W, SPIN, 0, false>);
+        if (p.wts) return p.wts_dd ? direct(k_spread_direct<T, W, SPIN, 2>) : direct(k_spread_direct<T, W, SPIN, 1>);
+        return direct(k_spread_direct<T, W, SPIN, 0>);
     } else {
         if (p.det) return run(k_spread<T, W, SPIN, 0, true>, 8);
         if (p.tile_kmax) return run(k_spread<T, W, SPIN, 0, false, true>, 4);

@@ -1,5 +1,6 @@
 // FP64 spreading (nufft.cuh).
 #include "nufft.cuh"
+#include "nufft_strip.cuh"
 
 namespace gsl {
 

@@ -719,19 +719,6 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
         if (tr != 0 && tr != 16 && tr != 32 && tr != 64)
             return bail(LENS_ERR_INVALID, "spread_tile_rows must be 0, 16, 32 or 64");
         p->tile_r = tr ? tr : kTileR;
-        p->ntile_c = (p->N2 + kTileC - 1) / kTileC;
-        p->ntiles = (p->R + p->tile_r - 1) / p->tile_r * p->ntile_c;
-        if ((e = B.alloc((void **)&p->tile_start, sizeof(uint32_t) * ((size_t)p->ntiles + 1), false)) != cudaSuccess)
-            return bailc(e, "alloc tile table");
-        if (spin && (e = B.alloc(&p->phase, esz * npoints, false)) != cudaSuccess) return bailc(e, "alloc phase");
-        // FP32 plans at epsilon >= 1e-5 accumulate the spreading tiles in 32-bit fixed point,
-        // FP64 plans in 64-bit fixed point (nufft.cu, k_spread); FP32 plans at smaller epsilon
-        // and deterministic plans keep their own paths
-        if (!p->det && (prec == LENS_FP64 || epsilon >= 1e-5)) {
-            if ((e = B.alloc((void **)&p->tile_kmax, sizeof(unsigned short) * (size_t)p->ntiles, false)) != cudaSuccess ||
-                (e = B.alloc((void **)&p->maxbits, sizeof(unsigned long long), true)) != cudaSuccess)
-                return bailc(e, "alloc spreading bounds");
-        }
         // FP64 plans keep the 2W kernel weights of every point (GB300's FP64 pipe makes
         // evaluating exp/sqrt per tap far dearer than reading 16 W bytes per point),
         // unless the table would exceed 48 GB (e.g. 805M points at W = 16: 206 GB);
@@ -739,18 +726,40 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
         const size_t wbytes = sizeof(double) * 2 * (size_t)p->W * npoints;
         const int pw = prm ? prm->point_weights : 0;
         if (pw < -1 || pw > 1) return bail(LENS_ERR_INVALID, "point_weights must be -1, 0 or 1");
-        if (prec == LENS_FP64 && (pw == 1 || (pw == 0 && wbytes <= (size_t)48 << 30)) &&
-            (e = B.alloc((void **)&p->wts, wbytes, false)) != cudaSuccess) {
+        const bool keep = prec == LENS_FP64 && (pw == 1 || (pw == 0 && wbytes <= (size_t)48 << 30));
+        // with the weights kept, FP64 plans at epsilon >= 5e-11 compute the interpolation and
+        // spreading taps in double-float on the FP32 pipe (~2^-46 relative per term; lmax 4096,
+        // 50M points, W = 13: interpolation 30.1 -> 13.4 ms for spin 2); smaller epsilon keeps FP64
+        const bool dd = keep && epsilon >= 5e-11;
+        if (dd && !p->det) {  // spreading by strips: fewer rows per tile where the tiles would not fill the chip
+            p->strip = true;
+            p->tile_c = 33 - p->W;
+            p->ntile_c = (p->N2 + p->tile_c - 1) / p->tile_c;
+            if (!tr)
+                for (p->tile_r = 64; p->tile_r > 8 && (p->R / p->tile_r) * p->ntile_c < 152 * 24; p->tile_r /= 2) {}
+        }
+        p->ntile_c = (p->N2 + p->tile_c - 1) / p->tile_c;
+        p->ntiles = (p->R + p->tile_r - 1) / p->tile_r * p->ntile_c;
+        if ((e = B.alloc((void **)&p->tile_start, sizeof(uint32_t) * ((size_t)p->ntiles + 1), false)) != cudaSuccess)
+            return bailc(e, "alloc tile table");
+        if (spin && (e = B.alloc(&p->phase, esz * npoints, false)) != cudaSuccess) return bailc(e, "alloc phase");
+        // FP32 plans at epsilon >= 1e-5 accumulate the spreading tiles in 32-bit fixed point,
+        // FP64 plans in 64-bit fixed point (nufft.cu, k_spread); FP32 plans at smaller epsilon
+        // and deterministic plans keep their own paths
+        if (!p->det && !p->strip && (prec == LENS_FP64 || epsilon >= 1e-5)) {
+            if ((e = B.alloc((void **)&p->tile_kmax, sizeof(unsigned short) * (size_t)p->ntiles, false)) != cudaSuccess ||
+                (e = B.alloc((void **)&p->maxbits, sizeof(unsigned long long), true)) != cudaSuccess)
+                return bailc(e, "alloc spreading bounds");
+        }
+        if (keep && (e = B.alloc((void **)&p->wts, dd ? sizeof(float) * (size_t)dd_words(p->W) * npoints : wbytes, false)) !=
+                        cudaSuccess) {
             if (e == cudaErrorMemoryAllocation) {
                 cudaGetLastError();
                 return bail(LENS_ERR_NOMEM, "point kernel weights: " + std::to_string(wbytes >> 20) + " MiB not available");
             }
             return bailc(e, "alloc weights");
         }
-        // with the weights kept, FP64 plans at epsilon >= 5e-11 compute the interpolation and
-        // spreading taps in double-float on the FP32 pipe (~2^-46 relative per term; lmax 4096,
-        // 50M points, W = 13: interpolation 30.1 -> 13.4 ms for spin 2); smaller epsilon keeps FP64
-        p->wts_dd = p->wts && epsilon >= 5e-11;
+        p->wts_dd = dd;
     }
 
     // ---- host tables: start-value norms, rings, deconvolution factors
