@@ -188,8 +188,10 @@ struct Plan {
     int ntile_c = 0, ntiles = 0;     // tiles per grid row band, total tiles
     int tile_r = kTileR;             // rows of a tile (16, 32 or 64; 32 columns)
     void *phase = nullptr;     // float2 / double2 e^{i s chi}, spin != 0 only
-    int tile_c = kTileC;             // columns of a tile: 32; FP64 plans that spread by strips 33 - W
-    bool strip = false;              // spreading by strips (nufft_strip.cuh): points sorted by tile, then by row
+    int tile_c = kTileC;             // columns of a tile: 32; plans that spread by strips 33 - W
+    bool strip = false;              // spreading by strips (nufft_strip.cuh)
+    uint32_t strip_part = 0;         // points of a tile that one warp sweeps, and the most such parts of a tile
+    int strip_parts = 1;
     double *wts = nullptr;     // FP64 plans: [npts][2W] kernel weights (theta taps, then phi taps)
     bool wts_dd = false;       // weights as double-float pairs (layout: dd_words, nufft.cuh); double-float
                                // interpolation and spreading taps (FP64 plans with epsilon >= 5e-11)

@@ -61,7 +61,10 @@ __global__ void k_prep(const double *__restrict__ theta, const double *__restric
     frac_u[i] = make_double2(fu, fv);
     const int ntc = (N2 + tile_c - 1) / tile_c;
     const uint32_t tile = (uint32_t)(row / tile_r) * (uint32_t)ntc + (uint32_t)(j0 / tile_c);
-    key[i] = rows ? tile * (uint32_t)tile_r + (uint32_t)(row % tile_r) : tile;  // rows: by cell row within the tile
+    uint32_t k = tile;  // rows: by cell row within the tile, 2: then by column
+    if (rows) k = k * (uint32_t)tile_r + (uint32_t)(row % tile_r);
+    if (rows == 2) k = k * (uint32_t)tile_c + (uint32_t)(j0 % tile_c);
+    key[i] = k;
     idx[i] = (int32_t)i;
     if (spin) {
         const double c = chi ? chi[i] : 0.0;
@@ -99,6 +102,14 @@ __global__ void k_tile_bounds(const uint32_t *__restrict__ skey, int64_t n, int 
     const int64_t lo = p == 0 ? -1 : (int64_t)(skey[p - 1] / per);
     const int64_t hi = p == n ? (int64_t)ntiles : (int64_t)(skey[p] / per);
     for (int64_t t = lo + 1; t <= hi; ++t) start[t] = (uint32_t)p;
+}
+
+__global__ void k_tile_most(const uint32_t *__restrict__ start, int ntiles, unsigned *__restrict__ most)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned c = t < ntiles ? start[t + 1] - start[t] : 0u;
+    c = __reduce_max_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31) == 0) atomicMax(most, c);
 }
 
 // FP64 plans' 2W kernel weights of every (sorted) point, computed once, evaluated in FP64 and kept as
@@ -336,13 +347,15 @@ cudaError_t launch_prep_points(Plan &p, const double *theta, const double *phi, 
         const double hi = q1 + q2;
         return make_double2(hi, q2 - (hi - q1));
     };
-    k_prep<<<blocks, thr, 0, st>>>(theta, phi, chi, n, p.N1, p.N2, p.W, p.r_lo, p.R, p.pitch, p.spin, scale_of(p.N1),
-                                   scale_of(p.N2), p.tile_r, p.tile_c, p.strip ? 1 : 0, key, idx, cell_u, frac_u, phase_u, p.flags);
-    GSL_TRY(cudaGetLastError());
     const int ntc = p.ntile_c;
-    const int per = p.strip ? p.tile_r : 1;
     const uint64_t nkeys = (uint64_t)((p.R + p.tile_r - 1) / p.tile_r) * ntc;
-    if (nkeys * per > 0xffffffffull) { cleanup(); err = "internal: tile keys above 32 bits"; return cudaErrorInvalidValue; }
+    // sorted by row (spreading by strips needs it) and by column (for the interpolation) within a tile where the keys
+    // fit 32 bits
+    const int rows = nkeys * p.tile_r * p.tile_c <= 0xffffffffull ? 2 : p.strip ? 1 : 0;
+    const int per = rows == 2 ? p.tile_r * p.tile_c : rows ? p.tile_r : 1;
+    k_prep<<<blocks, thr, 0, st>>>(theta, phi, chi, n, p.N1, p.N2, p.W, p.r_lo, p.R, p.pitch, p.spin, scale_of(p.N1),
+                                   scale_of(p.N2), p.tile_r, p.tile_c, rows, key, idx, cell_u, frac_u, phase_u, p.flags);
+    GSL_TRY(cudaGetLastError());
     int bits = 1;
     while (bits < 32 && (1ull << bits) < nkeys * per) ++bits;
     GSL_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tmp_bytes, key, key2, idx, p.perm, (int)n, 0, bits, st));
@@ -385,9 +398,22 @@ cudaError_t launch_prep_points(Plan &p, const double *theta, const double *phi, 
         k_weights<<<blocks, thr, 0, st>>>((const double2 *)p.frac, n, p.W, p.beta, p.wts, p.wts_dd ? 1 : 0);
         GSL_TRY(cudaGetLastError());
     }
-    unsigned hflags = 0;
-    GSL_TRY(cudaMemcpyAsync(&hflags, p.flags, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+    if (p.strip) {  // most points of a tile
+        GSL_TRY(cudaMemsetAsync(p.flags + 2, 0, sizeof(unsigned), st));
+        k_tile_most<<<(unsigned)((p.ntiles + thr - 1) / thr), thr, 0, st>>>(p.tile_start, p.ntiles, p.flags + 2);
+        GSL_TRY(cudaGetLastError());
+    }
+    unsigned hf[3] = {0, 0, 0};
+    GSL_TRY(cudaMemcpyAsync(hf, p.flags, sizeof(hf), cudaMemcpyDeviceToHost, st));
     GSL_TRY(cudaStreamSynchronize(st));
+    const unsigned hflags = hf[0];
+    if (p.strip) {
+        // A warp sweeps at most 4096 points (uniform skies have ~1000 per tile; a tile into which a survey patch
+        // piles its points is shared by up to 64 warps)
+        p.strip_part = 4096;
+        while ((uint64_t)p.strip_part * 64 < hf[2]) p.strip_part *= 2;
+        p.strip_parts = hf[2] ? (int)((hf[2] - 1) / p.strip_part + 1) : 1;
+    }
 #undef GSL_TRY
     cleanup();
     if (hflags & FLAG_DOMAIN) { err = "a coordinate is not finite or theta is outside [0, pi]"; return cudaErrorInvalidValue; }

@@ -12,18 +12,16 @@
 // Points are prepared once per plan (Sect. 4: the geometry is reused): cell
 // offset into the row-padded grid, fractional offsets (u - i0, v - j0) from
 // FP64 coordinates, the spin phase e^{i s chi}, a permutation that sorts
-// points by 32 x 32 grid tiles (of the first tap) so that neighbouring
-// threads share grid rows, and the first sorted point of every tile.
-// Interpolation runs one thread per sorted point and reads its W x W taps
+// points by grid tile (of the first tap), within a tile by cell row and column, so that neighbouring
+// threads share grid rows and cells, and the first sorted point of every tile.
+// Interpolation runs one thread per sorted point and reads its taps
 // through L1: sorted neighbours share rows, so the tile stays cached (staging
 // the tile and its halo in shared memory first measured 1.36x slower for
-// spin 0 at lmax 4096).  Spreading in FP32 runs one CTA per tile: its points
-// add their W x W taps into the tile and its halo, (32 + W - 1) x (32 + W - 1)
-// cells held in shared memory, and the CTA then adds the non-zero cells into
-// the grid with one global atomic each.  FP64
-// plans spread with one global atomic per tap instead: the L2 adds doubles
-// natively, while double additions into shared memory measured 1.9x (spin s)
-// to 2.4x (spin 0) slower at lmax 4096.
+// spin 0 at lmax 4096).  Sorted by row and column, and by aligned pairs (k_interp32): lmax 4096, 50M points, FP32, spin 0
+// 1.17 -> 0.77 ms, spin 2 2.08 -> 1.56 ms.
+// Spreading: FP64 plans with double-float weights and FP32 plans with W >= 8 by strips in registers (nufft_strip.cuh); the
+// others one CTA per 32 x 32 tile: its points add their W x W taps into the tile and its halo, (32 + W - 1) x (32 + W - 1)
+// integers held in shared memory, and the CTA then adds the non-zero cells into the grid with one global atomic each.
 //
 // Deterministic plans (LENS_DETERMINISTIC) spread in 64-bit fixed point: every
 // tap value is scaled by a power of two 2^k and rounded to an integer, and the
@@ -43,6 +41,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "pk.cuh"
 
 namespace gsl {
 namespace {
@@ -176,6 +175,68 @@ __global__ void __launch_bounds__(256) k_interp(const void *__restrict__ grid, c
         const cplx<T> ph = phase[p];
         map[dst] = ax * ph.x - ay * ph.y;
         map[n + dst] = ax * ph.y + ay * ph.x;
+    }
+}
+
+// FP32 plans: the W taps of a row by aligned pairs of cells (spin s 16-byte loads of two complex cells, spin 0 8-byte
+// loads of two real ones), the weights shifted by one cell where the first tap lies in the second half of its pair;
+// (W + 2) / 2 loads a row instead of W.  The sums were bound by the L1 data stage (92% of its wavefronts: lanes of
+// neighbouring points hit the same banks with 4- and 8-byte loads); with the points sorted by row and column the 8 lanes of a
+// 16-byte load's quarter lie within ~13 cells.  The extra cell of a pair may be one past the row's wrap columns: k_phi_fwd
+// writes zeros there.  Spin s sums in tap order, as before (its bits do not change).
+template <int W, bool SPIN>
+__global__ void __launch_bounds__(256) k_interp32(const float *__restrict__ grid, const uint32_t *__restrict__ cell,
+                                                  const float2 *__restrict__ frac, const int32_t *__restrict__ perm,
+                                                  const float2 *__restrict__ phase, float *__restrict__ map, int64_t n,
+                                                  int pitch, const __grid_constant__ KerPoly kp)
+{
+    constexpr int NPR = (W + 2) / 2;  // pairs that cover W cells from either half of a pair
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const uint32_t c0 = cell[p];  // row * pitch + column, pitch even: its parity is the column's
+    const bool odd = c0 & 1;
+    float wa[W], wb[W];
+    tap_weights<float, W, 0>(wa, wb, frac[p], nullptr, p, 0.f, kp);
+    float ws[2 * NPR];
+#pragma unroll
+    for (int k = 0; k < 2 * NPR; ++k) {
+        const float e = k < W ? wb[k < W ? k : 0] : 0.f, o = k > 0 && k - 1 < W ? wb[k > 0 && k - 1 < W ? k - 1 : 0] : 0.f;
+        ws[k] = odd ? o : e;
+    }
+    const int32_t dst = perm[p];
+    if constexpr (!SPIN) {
+        const float *g = grid + (c0 & ~1u);
+        pk w2[NPR];
+#pragma unroll
+        for (int k = 0; k < NPR; ++k) w2[k] = pk_make(ws[2 * k], ws[2 * k + 1]);
+        pk acc = 0ull;
+#pragma unroll
+        for (int a = 0; a < W; ++a) {
+            pk r = 0ull;
+#pragma unroll
+            for (int k = 0; k < NPR; ++k)
+                r = pk_fma(w2[k], __ldg(reinterpret_cast<const pk *>(g + (int64_t)a * pitch) + k), r);
+            acc = pk_fma(pk_make(wa[a], wa[a]), r, acc);
+        }
+        const float2 v = pk_get(acc);
+        map[dst] = v.x + v.y;
+    } else {
+        const float *g = grid + 2 * (int64_t)(c0 & ~1u);
+        pk acc = 0ull;
+#pragma unroll
+        for (int a = 0; a < W; ++a) {
+            pk r = 0ull;
+#pragma unroll
+            for (int k = 0; k < NPR; ++k) {
+                const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(g + 2 * (int64_t)a * pitch) + k);
+                r = pk_fma(pk_make(ws[2 * k], ws[2 * k]), v.x, r);
+                r = pk_fma(pk_make(ws[2 * k + 1], ws[2 * k + 1]), v.y, r);
+            }
+            acc = pk_fma(pk_make(wa[a], wa[a]), r, acc);
+        }
+        const float2 s = pk_get(acc), ph = phase[p];
+        map[dst] = s.x * ph.x - s.y * ph.y;
+        map[n + dst] = s.x * ph.y + s.y * ph.x;
     }
 }
 
@@ -349,6 +410,8 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
     for (int i = threadIdx.x; i < TR * TC * NC; i += blockDim.x) buf[i] = G(0);
     __syncthreads();
     const int r0 = (t / ntc) * tile_r, c0 = (t % ntc) * kTileC;
+    // (points in sorted order: spin 2, lmax 2048, W = 7: 0.69 ms; a run of points per thread, for fewer of a warp's taps in
+    // one bank, 0.77, runs per group of four threads 0.78: the loads then no longer coalesce)
     for (uint32_t p = p0 + threadIdx.x; p < (bad ? p0 : p1); p += blockDim.x) {
         const uint32_t c = cell[p];
         const int lr = (int)(c / (uint32_t)pitch) - r0, lc = (int)(c % (uint32_t)pitch) - c0;
@@ -430,6 +493,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
 }
 
 template <int W, bool SPIN> cudaError_t spread_strip(const Plan &p, const void *map, void *grid, cudaStream_t st);
+template <int W, bool SPIN> cudaError_t spread_strip32(const Plan &p, const void *map, void *grid, cudaStream_t st);
 
 template <typename T, bool SPIN, int W>
 cudaError_t interp_w(const Plan &p, const void *grid, void *map, cudaStream_t st)
@@ -449,8 +513,12 @@ cudaError_t interp_w(const Plan &p, const void *grid, void *map, cudaStream_t st
             return cudaGetLastError();
         }
         if (p.wts) return run(k_interp<T, W, SPIN, 1>);
+        return run(k_interp<T, W, SPIN, 0>);
+    } else {
+        k_interp32<W, SPIN><<<(unsigned)blocks, thr, 0, st>>>((const float *)grid, p.cell, (const float2 *)p.frac, p.perm,
+                                                              (const float2 *)p.phase, (float *)map, p.npts, p.pitch, p.kpoly);
+        return cudaGetLastError();
     }
-    return run(k_interp<T, W, SPIN, 0>);
 }
 
 template <typename T, bool SPIN, int W>
@@ -486,10 +554,9 @@ cudaError_t spread_w(const Plan &p, const void *map, void *grid, cudaStream_t st
         return direct(k_spread_direct<T, W, SPIN, 0>);
     } else {
         if (p.det) return run(k_spread<T, W, SPIN, 0, true>, 8);
-        if (p.tile_kmax) return run(k_spread<T, W, SPIN, 0, false, true>, 4);
-        return run(k_spread<T, W, SPIN, 0, false>, sizeof(T));
+        if (!p.strip) return run(k_spread<T, W, SPIN, 0, false, true>, 4);
+        return spread_strip32<W, SPIN>(p, map, grid, st);
     }
-    return cudaGetLastError();
 }
 
 template <typename T, bool SPIN>

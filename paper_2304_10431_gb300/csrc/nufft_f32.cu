@@ -1,5 +1,6 @@
 // FP32 interpolation and spreading (nufft.cuh).
 #include "nufft.cuh"
+#include "nufft_strip.cuh"
 
 namespace gsl {
 

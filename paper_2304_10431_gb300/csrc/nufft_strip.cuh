@@ -1,4 +1,5 @@
-// Spreading of FP64 plans with double-float weights (epsilon >= 5e-11): tiles swept row by row in registers.
+// Spreading of FP64 plans with double-float weights (epsilon >= 5e-11) and of FP32 plans with W >= 8 (or epsilon < 1e-5),
+// not deterministic: tiles swept row by row in registers.
 //
 // One warp owns a tile of tile_r rows x (33 - W) columns, so the W-wide windows of its points cover 32
 // columns: lane c holds column c of the W rows that the points of one cell row touch, as sums of row pairs
@@ -25,7 +26,7 @@ namespace gsl {
 namespace {
 
 constexpr int kStripWarps = 4;   // warps (tiles) per CTA
-constexpr int kStripBatch = 16;  // points per weight copy
+constexpr int kStripBatch = 16;  // points per weight copy (FP64)
 
 template <int W> __host__ __device__ constexpr size_t strip_warp_smem()
 {
@@ -33,20 +34,32 @@ template <int W> __host__ __device__ constexpr size_t strip_warp_smem()
     return 2 * kStripBatch * dd_words(W) * sizeof(float) + kStripBatch * (sizeof(float4) + sizeof(int)) + 16;
 }
 
+// Points of tile t for this CTA row: blockIdx.y-th part of `part` points (a tile with more points than that is shared
+// by several warps, each sweeping the rows of its part); false if there are none.
+__device__ __forceinline__ bool strip_points(const uint32_t *__restrict__ tile_start, int t, uint32_t part, uint32_t &p0,
+                                             uint32_t &p1)
+{
+    const uint32_t a = tile_start[t], b = tile_start[t + 1], off = blockIdx.y * part;
+    if (b - a <= off) return false;
+    p0 = a + off;
+    p1 = min(b, p0 + part);
+    return true;
+}
+
 template <int W, bool SPIN>
 __global__ void __launch_bounds__(32 * kStripWarps)
 k_spread_strip(double *__restrict__ grid, const uint32_t *__restrict__ cell, const int32_t *__restrict__ perm,
                const double2 *__restrict__ phase, const double *__restrict__ wts, const double *__restrict__ map,
                int64_t n, int pitch, int R, int ntc, int ntiles, const uint32_t *__restrict__ tile_start, int tile_r,
-               unsigned *__restrict__ status)
+               uint32_t part, unsigned *__restrict__ status)
 {
     constexpr int NP = dd_pairs(W), NC = SPIN ? 2 : 1, TC = 33 - W;
     constexpr uint32_t WBYTES = dd_words(W) * sizeof(float);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int t = blockIdx.x * kStripWarps + wid;
     if (t >= ntiles) return;
-    const uint32_t p0 = tile_start[t], p1 = tile_start[t + 1];
-    if (p0 == p1) return;
+    uint32_t p0, p1;
+    if (!strip_points(tile_start, t, part, p0, p1)) return;
     extern __shared__ __align__(16) unsigned char strip_smem[];
     unsigned char *mem = strip_smem + wid * strip_warp_smem<W>();
     float4 *sval = reinterpret_cast<float4 *>(mem + 2 * kStripBatch * WBYTES);
@@ -194,15 +207,162 @@ k_spread_strip(double *__restrict__ grid, const uint32_t *__restrict__ cell, con
     while (cur < last) next_row();
 }
 
+// FP32 plans with W >= 8 (or epsilon < 1e-5): the same sweep with FP32 sums.  Each lane evaluates the 2W polynomial weights
+// of one point of a batch of 32 into shared memory (the coefficients come from the constant bank); then the warp
+// takes the points in turn.  Bound by issue: ~50 instructions per point whatever W, where the tiles of 32-bit
+// integers in shared memory (nufft.cuh) cost W^2 atomics: spin 2, lmax 4096, 50M points, W = 8: 3.07 -> 2.66 ms; W = 7: lmax 2048 0.66
+// against 0.69 ms, lmax 1024 0.17 against 0.22, so W <= 7 keeps the tiles.  Two tiles of 17 - W columns per warp, one per half,
+// were tried for the lanes a point leaves idle: 2.83 ms, and the narrow tiles cost the interpolation 0.2-0.4 ms.
+template <int W> __host__ __device__ constexpr size_t strip32_warp_smem()
+{
+    // per point: value twice (float4), theta weights (padded to 16 bytes), tile row and column (int2), phi weights; one
+    // slot more than the 32 points, which the loop's look-ahead reads
+    return (33 * (4 + 4 * ((W + 3) / 4) + 2 + W) * sizeof(float) + 15) / 16 * 16;
+}
+
+template <int W, bool SPIN>
+__global__ void __launch_bounds__(32 * kStripWarps)
+k_spread_strip32(float *__restrict__ grid, const uint32_t *__restrict__ cell, const float2 *__restrict__ frac,
+                 const int32_t *__restrict__ perm, const float2 *__restrict__ phase, const float *__restrict__ map,
+                 int64_t n, int pitch, int R, int ntc, int ntiles, const uint32_t *__restrict__ tile_start, int tile_r,
+                 uint32_t part, const __grid_constant__ KerPoly kp)
+{
+    constexpr int NP = (W + 1) / 2, NC = SPIN ? 2 : 1, TC = 33 - W, WA = 4 * ((W + 3) / 4);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int t = blockIdx.x * kStripWarps + wid;
+    if (t >= ntiles) return;
+    uint32_t p0, p1;
+    if (!strip_points(tile_start, t, part, p0, p1)) return;
+    extern __shared__ __align__(16) unsigned char strip_smem[];
+    float4 *sval = reinterpret_cast<float4 *>(strip_smem + wid * strip32_warp_smem<W>());  // (x, x, y, y)
+    float *swa = reinterpret_cast<float *>(sval + 33);                                     // [33][WA]
+    int2 *soff = reinterpret_cast<int2 *>(swa + 33 * WA);                                  // (row, column)
+    float *swb = reinterpret_cast<float *>(soff + 33);                                     // [33][W]
+
+    const int r0 = (t / ntc) * tile_r, c0 = (t % ntc) * TC, gc = c0 + lane;
+    pk S[NC][NP];
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int i = 0; i < NP; ++i) S[c][i] = 0ull;
+    int cur = 0;
+    auto next_row = [&]() {
+        const int gr = r0 + cur;
+        float v[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) v[c] = pk_get(S[c][0]).x;
+        bool any = v[0] != 0.f;
+        if (SPIN) any = any || v[NC - 1] != 0.f;
+        if (any && gr < R && gc < pitch) {
+            const int64_t o = (int64_t)gr * pitch + gc;
+            if constexpr (SPIN) atomicAdd(reinterpret_cast<float2 *>(grid) + o, make_float2(v[0], v[NC - 1]));
+            else atomicAdd(grid + o, v[0]);
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+#pragma unroll
+            for (int i = 0; i < NP; ++i)
+                S[c][i] = pk_make(pk_get(S[c][i]).y, i + 1 < NP ? pk_get(S[c][i + 1 < NP ? i + 1 : i]).x : 0.f);
+        ++cur;
+    };
+    if (lane == 0) {  // the look-ahead slot: no column
+        sval[32] = make_float4(0.f, 0.f, 0.f, 0.f);
+        soff[32] = make_int2(0, 64);
+    }
+
+    for (uint32_t pb = p0; pb < p1; pb += 32) {
+        const int cnt = (int)min(32u, p1 - pb);
+        if (lane < cnt) {
+            const uint32_t p = pb + lane, c = cell[p];
+            const float2 f = frac[p];
+            const int lr = (int)(c / (uint32_t)pitch) - r0, lc = (int)(c % (uint32_t)pitch) - c0;
+            const bool mine = (unsigned)lr < (unsigned)tile_r && (unsigned)lc < (unsigned)TC;
+            const int32_t src = perm[p];
+            float2 z = make_float2(map[src], 0.f);
+            if constexpr (SPIN) {  // e^{-i s chi} (Q + i U)
+                const float2 ph = phase[p];
+                const float u = map[n + src];
+                z = make_float2(ph.x * z.x + ph.y * u, ph.x * u - ph.y * z.x);
+            }
+            soff[lane] = mine ? make_int2(lr, lc) : make_int2(0, 64);  // column 64: no lane's
+            const float tx = fmaf(2.f, f.x, -(float)(W - 1)), ty = fmaf(2.f, f.y, -(float)(W - 1));
+            float wa[WA];
+#pragma unroll
+            for (int a = 0; a < WA; ++a) wa[a] = a < W ? ker_poly<W>(kp, a < W ? a : 0, tx) : 0.f;
+#pragma unroll
+            for (int a = 0; a < WA; a += 4)
+                *reinterpret_cast<float4 *>(swa + lane * WA + a) = make_float4(wa[a], wa[a + 1], wa[a + 2], wa[a + 3]);
+            sval[lane] = make_float4(z.x, z.x, z.y, z.y);
+#pragma unroll
+            for (int b = 0; b < W; ++b) swb[lane * W + b] = ker_poly<W>(kp, b, ty) * (SPIN ? 1.f : z.x);
+        }
+        __syncwarp();
+        // each point's row and column are loaded two points ahead, its column weight and value one ahead
+        int2 so = soff[0], sn = soff[1];
+        float wb = (unsigned)(lane - so.y) < (unsigned)W ? swb[lane - so.y] : 0.f;
+        ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(sval);
+        const float *wap = swa, *wbp = swb + lane;
+#pragma unroll 1
+        for (int q = 0; q < cnt; ++q) {
+            const pk w2 = pk_make(wb, wb);
+            pk v[NC];
+            if constexpr (SPIN) {
+                v[0] = pk_mul(w2, z.x);
+                v[NC - 1] = pk_mul(w2, z.y);
+                z = *reinterpret_cast<const ulonglong2 *>(sval + q + 1);
+            } else {
+                v[0] = w2;
+            }
+            pk wa[2 * ((NP + 1) / 2)];
+#pragma unroll
+            for (int i = 0; i < NP; i += 2) {
+                const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(wap + 2 * i);
+                wa[i] = w.x;
+                wa[i + 1] = w.y;
+            }
+            wap += WA;
+            wbp += W;
+            wb = (unsigned)(lane - sn.y) < (unsigned)W ? wbp[-sn.y] : 0.f;
+            while (cur < so.x) next_row();
+            so = sn;
+            sn = soff[min(q + 2, 32)];
+#pragma unroll
+            for (int i = 0; i < NP; ++i)
+#pragma unroll
+                for (int c = 0; c < NC; ++c) S[c][i] = pk_fma(wa[i], v[c], S[c][i]);
+        }
+        __syncwarp();  // the staged points are rewritten by the next batch
+    }
+    const int last = min(tile_r + W - 1, cur + W);
+    while (cur < last) next_row();
+}
+
+inline dim3 strip_grid(const Plan &p)
+{
+    return dim3((unsigned)((p.ntiles + kStripWarps - 1) / kStripWarps), (unsigned)p.strip_parts);
+}
+
 template <int W, bool SPIN> cudaError_t spread_strip(const Plan &p, const void *map, void *grid, cudaStream_t st)
 {
     const auto kern = k_spread_strip<W, SPIN>;
     const size_t sm = kStripWarps * strip_warp_smem<W>();
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)((p.ntiles + kStripWarps - 1) / kStripWarps), 32 * kStripWarps, sm, st>>>(
+    kern<<<strip_grid(p), 32 * kStripWarps, sm, st>>>(
         (double *)grid, p.cell, p.perm, (const double2 *)p.phase, p.wts, (const double *)map, p.npts, p.pitch, p.R,
-        p.ntile_c, p.ntiles, p.tile_start, p.tile_r, p.flags + 1);
+        p.ntile_c, p.ntiles, p.tile_start, p.tile_r, p.strip_part, p.flags + 1);
+    return cudaGetLastError();
+}
+
+template <int W, bool SPIN> cudaError_t spread_strip32(const Plan &p, const void *map, void *grid, cudaStream_t st)
+{
+    const size_t sm = kStripWarps * strip32_warp_smem<W>();
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_spread_strip32<W, SPIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    k_spread_strip32<W, SPIN><<<strip_grid(p), 32 * kStripWarps, sm, st>>>(
+        (float *)grid, p.cell, (const float2 *)p.frac, p.perm, (const float2 *)p.phase, (const float *)map, p.npts,
+        p.pitch, p.R, p.ntile_c, p.ntiles, p.tile_start, p.tile_r, p.strip_part, p.kpoly);
     return cudaGetLastError();
 }
 

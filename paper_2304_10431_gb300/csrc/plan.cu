@@ -525,7 +525,7 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
     }
     p->r_lo = -p->W;
     p->R = p->N1 / 2 + 2 * p->W + 1;
-    p->pitch = ((p->N2 + p->W - 1) + 31) / 32 * 32;
+    p->pitch = ((p->N2 + p->W + 1) + 31) / 32 * 32;  // W - 1 wrap columns and two zeros (k_interp32)
 
     // ---- Legendre arithmetic: FP32 plans df32 for every m; FP64 plans native FP64
     // for m < m_df and df32 recursion + df32 accumulation for m >= m_df.  df32
@@ -731,7 +731,9 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
         // spreading taps in double-float on the FP32 pipe (~2^-46 relative per term; lmax 4096,
         // 50M points, W = 13: interpolation 30.1 -> 13.4 ms for spin 2); smaller epsilon keeps FP64
         const bool dd = keep && epsilon >= 5e-11;
-        if (dd && !p->det) {  // spreading by strips: fewer rows per tile where the tiles would not fill the chip
+        // spreading by strips (nufft_strip.cuh; FP32 plans by tiles of 32-bit integers where those are faster): fewer rows
+        // per tile where the tiles would not fill the chip
+        if ((dd || (prec == LENS_FP32 && (p->W >= 8 || epsilon < 1e-5))) && !p->det) {
             p->strip = true;
             p->tile_c = 33 - p->W;
             p->ntile_c = (p->N2 + p->tile_c - 1) / p->tile_c;
@@ -743,10 +745,9 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
         if ((e = B.alloc((void **)&p->tile_start, sizeof(uint32_t) * ((size_t)p->ntiles + 1), false)) != cudaSuccess)
             return bailc(e, "alloc tile table");
         if (spin && (e = B.alloc(&p->phase, esz * npoints, false)) != cudaSuccess) return bailc(e, "alloc phase");
-        // FP32 plans at epsilon >= 1e-5 accumulate the spreading tiles in 32-bit fixed point,
-        // FP64 plans in 64-bit fixed point (nufft.cu, k_spread); FP32 plans at smaller epsilon
-        // and deterministic plans keep their own paths
-        if (!p->det && !p->strip && (prec == LENS_FP64 || epsilon >= 1e-5)) {
+        // the other plans accumulate spreading tiles in fixed point, FP32 plans in 32 bits, FP64 plans in 64
+        // (nufft.cuh, k_spread); deterministic plans keep their own paths
+        if (!p->det && !p->strip) {
             if ((e = B.alloc((void **)&p->tile_kmax, sizeof(unsigned short) * (size_t)p->ntiles, false)) != cudaSuccess ||
                 (e = B.alloc((void **)&p->maxbits, sizeof(unsigned long long), true)) != cudaSuccess)
                 return bailc(e, "alloc spreading bounds");

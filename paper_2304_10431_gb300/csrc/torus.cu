@@ -349,8 +349,8 @@ __global__ void __launch_bounds__(512, OCC) k_phi_fwd(const cplx<T> *__restrict_
         } else {
             T *ga = (T *)grid + (int64_t)ra * pitch;
             T *gb = (T *)grid + (int64_t)rb * pitch;
-            for (int c = tid; c < N2 + W - 1; c += nthr) {
-                C v = buf[c < N2 ? c : c - N2];
+            for (int c = tid; c < N2 + W + 1; c += nthr) {  // two zeros past the wrap columns (k_interp32)
+                const C v = c < N2 + W - 1 ? buf[c < N2 ? c : c - N2] : mkc(T(0), T(0));
                 ga[c] = v.x;
                 if (hb) gb[c] = v.y;
             }
@@ -373,7 +373,8 @@ __global__ void __launch_bounds__(512, OCC) k_phi_fwd(const cplx<T> *__restrict_
             }
         } else {
             C *gr = (C *)grid + (int64_t)r * pitch;
-            for (int c = tid; c < N2 + W - 1; c += nthr) gr[c] = buf[c < N2 ? c : c - N2];
+            for (int c = tid; c < N2 + W + 1; c += nthr)
+                gr[c] = c < N2 + W - 1 ? buf[c < N2 ? c : c - N2] : mkc(T(0), T(0));
         }
     }
     if (CL > 1) tm.sync();
