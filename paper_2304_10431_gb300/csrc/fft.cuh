@@ -9,7 +9,7 @@
 // suffices.  Radices 2, 3, 4, 5, 7, 8; odd radices use the symmetric-pair
 // form y_k = x_0 + sum_q (x_q + x_{p-q}) cos(2 pi qk/p) -+ i (x_q - x_{p-q}) sin(2 pi qk/p);
 // FP32 transforms also use the composite radices 6, 9, 14 and 21 (two small
-// DFTs in registers per stage, fewer shared-memory passes).
+// DFTs in registers per stage, fewer shared-memory passes), double-float ones 6 and 9.
 //
 // DIR = -1: forward, sum x_n e^{-2 pi i nk/N};  DIR = +1: inverse (unnormalised).
 //
@@ -25,6 +25,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "dfl.cuh"
 #include "internal.h"
 
 namespace gsl {
@@ -132,7 +133,13 @@ template <typename T> struct FftConst;
     };
 GSL_FFT_CONSTS(float)
 GSL_FFT_CONSTS(double)
+GSL_FFT_CONSTS(dfl)
 #undef GSL_FFT_CONSTS
+
+// a b + c (contracted by the compiler for float and double)
+__device__ __forceinline__ float madd(float a, float b, float c) { return c + a * b; }
+__device__ __forceinline__ double madd(double a, double b, double c) { return c + a * b; }
+__device__ __forceinline__ dfl madd(dfl a, dfl b, dfl c) { return dfl_fma(a, b, c); }
 
 // multiply by -i (DIR=-1) or +i (DIR=+1)
 template <int DIR, typename C> __device__ __forceinline__ C mul_dir_i(C a)
@@ -218,13 +225,13 @@ template <int P, int DIR, typename T> struct OddDft {
         out[0] = y0;
 #pragma unroll
         for (int k = 1; k <= H; ++k) {
-            cplx<T> a = x[0], b = mkc(T(0), T(0));
+            cplx<T> a = x[0], b = mkc(T(0.0), T(0.0));
 #pragma unroll
             for (int q = 1; q <= H; ++q) {
                 const int t = (q * k) % P;
                 const T c = cs(t), sv = sn(t);
-                a.x += c * s[q - 1].x; a.y += c * s[q - 1].y;
-                b.x += sv * d[q - 1].x; b.y += sv * d[q - 1].y;
+                a.x = madd(c, s[q - 1].x, a.x); a.y = madd(c, s[q - 1].y, a.y);
+                b.x = madd(sv, d[q - 1].x, b.x); b.y = madd(sv, d[q - 1].y, b.y);
             }
             cplx<T> ib = mul_dir_i<DIR>(b);
             out[k] = cadd(a, ib);
@@ -286,7 +293,8 @@ template <int P, int Q, int DIR, typename T> struct CompositeDft {
                 if (n2 > 0 && k1 > 0) {
                     const int e = (n2 * k1) % R;
                     const T c = (T)root_cs<R>(e, false), s = (T)(DIR * root_cs<R>(e, true));
-                    t[k1] = mkc(t[k1].x * c - t[k1].y * s, t[k1].x * s + t[k1].y * c);
+                    if constexpr (std::is_same<T, dfl>::value) t[k1] = cmul(t[k1], mkc(c, s));
+                    else t[k1] = mkc(t[k1].x * c - t[k1].y * s, t[k1].x * s + t[k1].y * c);
                 }
                 y[n2][k1] = t[k1];
             }
@@ -334,7 +342,7 @@ __device__ __forceinline__ void twiddle(cplx<T> (&x)[R], const cplx<T> *__restri
     } else {
 #pragma unroll
         for (int q = 1; q < R; ++q) {
-            const cplx<T> w = __ldg(tw + e * q);
+            const cplx<T> w = ldc(tw + e * q);
             x[q] = DIR < 0 ? cmul(x[q], w) : cmulc(x[q], w);
         }
     }
@@ -401,10 +409,10 @@ __device__ void fft_smem(const B &buf, const FftDesc &d, const Team<CL> &tm)
         case 5: fft_stage<5, DIR, T>(buf, d.n, Lp, tw, tm.tid, tm.nthr); break;
         case 7: fft_stage<7, DIR, T>(buf, d.n, Lp, tw, tm.tid, tm.nthr); break;
         case 6:
-            if constexpr (std::is_same<T, float>::value) fft_stage<6, DIR, T>(buf, d.n, Lp, tw, tm.tid, tm.nthr);
+            if constexpr (!std::is_same<T, double>::value) fft_stage<6, DIR, T>(buf, d.n, Lp, tw, tm.tid, tm.nthr);
             break;
         case 9:
-            if constexpr (std::is_same<T, float>::value) fft_stage<9, DIR, T>(buf, d.n, Lp, tw, tm.tid, tm.nthr);
+            if constexpr (!std::is_same<T, double>::value) fft_stage<9, DIR, T>(buf, d.n, Lp, tw, tm.tid, tm.nthr);
             break;
         case 14:
             if constexpr (std::is_same<T, float>::value) fft_stage<14, DIR, T>(buf, d.n, Lp, tw, tm.tid, tm.nthr);
@@ -464,10 +472,10 @@ __device__ void fft_smem_dif(const B &buf, const FftDesc &d, const Team<CL> &tm)
         case 5: fft_stage_dif<5, DIR, T>(buf, d.n, Lp, tw, tm.tid, tm.nthr); break;
         case 7: fft_stage_dif<7, DIR, T>(buf, d.n, Lp, tw, tm.tid, tm.nthr); break;
         case 6:
-            if constexpr (std::is_same<T, float>::value) fft_stage_dif<6, DIR, T>(buf, d.n, Lp, tw, tm.tid, tm.nthr);
+            if constexpr (!std::is_same<T, double>::value) fft_stage_dif<6, DIR, T>(buf, d.n, Lp, tw, tm.tid, tm.nthr);
             break;
         case 9:
-            if constexpr (std::is_same<T, float>::value) fft_stage_dif<9, DIR, T>(buf, d.n, Lp, tw, tm.tid, tm.nthr);
+            if constexpr (!std::is_same<T, double>::value) fft_stage_dif<9, DIR, T>(buf, d.n, Lp, tw, tm.tid, tm.nthr);
             break;
         case 14:
             if constexpr (std::is_same<T, float>::value) fft_stage_dif<14, DIR, T>(buf, d.n, Lp, tw, tm.tid, tm.nthr);

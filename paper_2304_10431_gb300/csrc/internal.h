@@ -179,6 +179,12 @@ struct Plan {
     void *w1 = nullptr;       // [2 lmax + 1]  1/psihat(2 pi k / N1), k = -lmax..lmax
     void *w2 = nullptr;       // [ncol]        1/(M psihat(2 pi m / N2))
     FftDesc fM, fN1, fN2;
+    // FP64 plans with restart values: the synthesis transforms in double-float (dfl.cuh), with their own descriptors and
+    // deconvolution factors; ring coefficients and torus rows of a synthesis are then double-float pairs.  The adjoint's
+    // stay in FP64: deconvolution amplifies their rounding noise (5e-13 of the a_lm in double-float)
+    bool fft_dd = false;
+    FftDesc dM, dN1, dN2;
+    void *w1d = nullptr, *w2d = nullptr;
 
     // points, sorted by grid tile
     uint32_t *cell = nullptr;  // row * pitch + col of the first tap
@@ -228,11 +234,14 @@ cudaError_t launch_tab_rows(const Plan &p, const int *first, int *lstart, int *j
 cudaError_t launch_tab_fill(const Plan &p);
 // wpos multiplies the orders m > 0 (1 for the transforms themselves; the
 // gradient entry points use 1/2 forward and 2 adjoint)
-cudaError_t launch_legendre_fwd(const Plan &p, const void *alm, void *ring, cudaStream_t st, double wpos = 1.0);
+// (ring_dd: the ring coefficients as double-float pairs, for the transforms of fft_dd plans)
+cudaError_t launch_legendre_fwd(const Plan &p, const void *alm, void *ring, cudaStream_t st, double wpos = 1.0,
+                                bool ring_dd = false);
 cudaError_t launch_legendre_adj(const Plan &p, const void *ring, void *alm, cudaStream_t st, double wpos = 1.0);
 // packed kernels of the plans with restart values (legendre_pk.cuh): rpt rings per thread; src the a_lm of
 // nm maps (FP32 plans) or the prepared df32 coefficients (FP64 plans, nm = 1)
-cudaError_t launch_leg_fwd_pk(const Plan &p, int rpt, const void *src, void *ring, int nm, double wpos, cudaStream_t st);
+cudaError_t launch_leg_fwd_pk(const Plan &p, int rpt, const void *src, void *ring, int nm, double wpos, bool ring_dd,
+                              cudaStream_t st);
 cudaError_t launch_leg_adj_pk(const Plan &p, int rpt, const void *ring, void *alm, double wpos, void *fx, cudaStream_t st);
 // FP32 plans: Legendre synthesis of nm = 2 or 4 maps (a_lm consecutive) sharing
 // one recursion; ring and coef hold nm maps' ring / prepared coefficients

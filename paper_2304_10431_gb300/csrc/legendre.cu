@@ -1702,7 +1702,7 @@ bool legendre_rpt_supported(int prec, int, bool, int rpt, bool rst)
     return rpt == 1 || rpt == 2 || (rpt == 4 && prec == LENS_FP32 && rst);
 }
 
-cudaError_t launch_legendre_fwd(const Plan &p, const void *alm, void *ring, cudaStream_t st, double wpos)
+cudaError_t launch_legendre_fwd(const Plan &p, const void *alm, void *ring, cudaStream_t st, double wpos, bool ring_dd)
 {
     // entries with l < spin / columns without rings are never written by the
     // kernel: start from zero
@@ -1710,11 +1710,11 @@ cudaError_t launch_legendre_fwd(const Plan &p, const void *alm, void *ring, cuda
     cudaError_t e;
     const dim3 g(4, p.mmax + 1);
     if (p.rst) {  // packed kernels: they write every ring of every column
-        if (p.prec == LENS_FP32) return launch_leg_fwd_pk(p, p.leg_f.rpt, alm, ring, 1, wpos, st);
+        if (p.prec == LENS_FP32) return launch_leg_fwd_pk(p, p.leg_f.rpt, alm, ring, 1, wpos, false, st);
         k_coef_prep<double2, double2, float4><<<g, 256, 0, st>>>((const double2 *)alm, p.scale, p.coef, p.lmax, p.spin,
                                                                  p.nalm, 0, wpos, p.grad);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        return launch_leg_fwd_pk(p, p.leg_fd.rpt, p.coef, ring, 1, wpos, st);
+        return launch_leg_fwd_pk(p, p.leg_fd.rpt, p.coef, ring, 1, wpos, ring_dd, st);
     }
     if ((e = cudaMemsetAsync(ring, 0, eb * (size_t)p.ncol * p.ntheta, st)) != cudaSuccess) return e;
     if (p.prec == LENS_FP32) {
@@ -1755,7 +1755,7 @@ cudaError_t launch_legendre_fwd_batch(const Plan &p, const void *alm, void *ring
         for (int b = 0; b < nm; b += at) {
             const cudaError_t e2 = launch_leg_fwd_pk(p, p.leg_fb[at == 2 ? 0 : 1].rpt,
                                                      (const float2 *)alm + (size_t)b * p.alm_ncomp() * p.nalm,
-                                                     (float2 *)ring + (size_t)b * p.ncol * p.ntheta, at, wpos, st);
+                                                     (float2 *)ring + (size_t)b * p.ncol * p.ntheta, at, wpos, false, st);
             if (e2 != cudaSuccess) return e2;
         }
         return cudaSuccess;

@@ -480,7 +480,7 @@ template <class A, int MODE, bool REIN, int NR, int NM>
 __device__ __forceinline__ void fwd_pk_body(const void *__restrict__ src, const void *__restrict__ rec,
                                             const RingTab &rt, typename A::C2 *__restrict__ ring, int lmax, int mmax,
                                             int spin, int ntheta, int nnorth, int64_t nalm, int64_t ring_stride,
-                                            float wpos, const CkTab &ck, int wb, unsigned char *smem)
+                                            float wpos, bool ring_dd, const CkTab &ck, int wb, unsigned char *smem)
 {
     using V = typename A::V;
     using S = typename A::S;
@@ -598,7 +598,15 @@ __device__ __forceinline__ void fwd_pk_body(const void *__restrict__ src, const 
     // write: spin 0 column m; spin s columns mmax + m and mmax - m, with the minus sign
     const float s0 = ((lf - m) & 1) ? -1.f : 1.f, ms0 = -s0;
     auto put = [&](typename A::C2 *col, int j, S re, float sr, S im, float si) {
-        col[j] = mkc(A::out(A::ssgn(re, sr)), A::out(A::ssgn(im, si)));
+        re = A::ssgn(re, sr);
+        im = A::ssgn(im, si);
+        if constexpr (!F32) {
+            if (ring_dd) {
+                reinterpret_cast<float4 *>(col)[j] = make_float4(re.h, re.l, im.h, im.l);
+                return;
+            }
+        }
+        col[j] = mkc(A::out(re), A::out(im));
     };
 #pragma unroll
     for (int b = 0; b < NM; ++b) {
@@ -651,7 +659,7 @@ __global__ void __launch_bounds__(128) k_leg_fwd_pk(const void *__restrict__ src
                                                     const void *__restrict__ rec_a, RingTab rt,
                                                     typename A::C2 *__restrict__ ring, int lmax, int mmax, int spin,
                                                     int ntheta, int nnorth, int64_t nalm, int64_t ring_stride,
-                                                    float wpos, CkTab ck)
+                                                    float wpos, int ring_dd, CkTab ck)
 {
     extern __shared__ __align__(16) unsigned char pk_smem[];
     constexpr int RPT = MODE == kSpin0 ? 2 * NR : NR;
@@ -662,10 +670,10 @@ __global__ void __launch_bounds__(128) k_leg_fwd_pk(const void *__restrict__ src
     if constexpr (std::is_same<A, PkF>::value) {
         if (wb < ck.jb)
             return fwd_pk_body<A, MODE, true, NR, NM>(src, rec_s, rt, ring, lmax, mmax, spin, ntheta, nnorth, nalm,
-                                                      ring_stride, wpos, ck, wb, mem);
+                                                      ring_stride, wpos, false, ck, wb, mem);
     }
     fwd_pk_body<A, MODE, false, NR, NM>(src, rec_a, rt, ring, lmax, mmax, spin, ntheta, nnorth, nalm, ring_stride, wpos,
-                                        ck, wb, mem);
+                                        ring_dd != 0, ck, wb, mem);
 }
 
 // ---------------------------------------------------------------- adjoint
@@ -1032,7 +1040,7 @@ PkShape pk_shape(const Plan &p, int rpt)
 }
 
 template <class A, int MODE, int NR, int NM>
-cudaError_t fwd_pk(const Plan &p, const void *src, void *ring, double wpos, cudaStream_t st)
+cudaError_t fwd_pk(const Plan &p, const void *src, void *ring, double wpos, bool ring_dd, cudaStream_t st)
 {
     const PkShape sh = pk_shape(p, MODE == kSpin0 ? 2 * NR : NR);
     const size_t smem = sh.block.x / 32 * fwd_pk_smem<A, MODE, NM>();
@@ -1043,7 +1051,7 @@ cudaError_t fwd_pk(const Plan &p, const void *src, void *ring, double wpos, cuda
     }
     k_leg_fwd_pk<A, MODE, NR, NM><<<sh.grid, sh.block, smem, st>>>(
         src, p.rec_s, p.prec == LENS_FP32 ? p.rec_a : p.rec_a_df, p.rings, (typename A::C2 *)ring, p.lmax, p.mmax,
-        p.spin, p.ntheta, p.nnorth, p.nalm, (int64_t)p.ncol * p.ntheta, (float)wpos, p.ck);
+        p.spin, p.ntheta, p.nnorth, p.nalm, (int64_t)p.ncol * p.ntheta, (float)wpos, ring_dd ? 1 : 0, p.ck);
     return cudaGetLastError();
 }
 
@@ -1065,20 +1073,20 @@ cudaError_t adj_pk(const Plan &p, const void *ring, void *alm, double wpos, void
 }
 
 template <class A, int NM>
-cudaError_t fwd_pk_rpt(const Plan &p, int rpt, const void *src, void *ring, double wpos, cudaStream_t st)
+cudaError_t fwd_pk_rpt(const Plan &p, int rpt, const void *src, void *ring, double wpos, bool ring_dd, cudaStream_t st)
 {
-    if (!p.spin) return rpt <= 2 ? fwd_pk<A, kSpin0, 1, NM>(p, src, ring, wpos, st) : fwd_pk<A, kSpin0, 2, NM>(p, src, ring, wpos, st);
+    if (!p.spin) return rpt <= 2 ? fwd_pk<A, kSpin0, 1, NM>(p, src, ring, wpos, ring_dd, st) : fwd_pk<A, kSpin0, 2, NM>(p, src, ring, wpos, ring_dd, st);
     if constexpr (NM == 1) {
         if (p.grad) {
-            if (rpt == 1) return fwd_pk<A, kGrad, 1, 1>(p, src, ring, wpos, st);
-            return rpt == 2 ? fwd_pk<A, kGrad, 2, 1>(p, src, ring, wpos, st) : fwd_pk<A, kGrad, 4, 1>(p, src, ring, wpos, st);
+            if (rpt == 1) return fwd_pk<A, kGrad, 1, 1>(p, src, ring, wpos, ring_dd, st);
+            return rpt == 2 ? fwd_pk<A, kGrad, 2, 1>(p, src, ring, wpos, ring_dd, st) : fwd_pk<A, kGrad, 4, 1>(p, src, ring, wpos, ring_dd, st);
         }
     }
     if constexpr (NM < 4) {
-        if (rpt == 1) return fwd_pk<A, kSpinS, 1, NM>(p, src, ring, wpos, st);
-        if (rpt == 2 || NM == 2) return fwd_pk<A, kSpinS, 2, NM>(p, src, ring, wpos, st);
+        if (rpt == 1) return fwd_pk<A, kSpinS, 1, NM>(p, src, ring, wpos, ring_dd, st);
+        if (rpt == 2 || NM == 2) return fwd_pk<A, kSpinS, 2, NM>(p, src, ring, wpos, ring_dd, st);
     }
-    if constexpr (NM == 1) return fwd_pk<A, kSpinS, 4, 1>(p, src, ring, wpos, st);
+    if constexpr (NM == 1) return fwd_pk<A, kSpinS, 4, 1>(p, src, ring, wpos, ring_dd, st);
     return cudaErrorInvalidValue;
 }
 

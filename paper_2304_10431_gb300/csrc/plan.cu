@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "dfl.cuh"
 #include "internal.h"
 
 namespace gsl {
@@ -179,10 +180,9 @@ int support_for(double eps, double sigma)
     return std::max(W, 4);
 }
 
-// Radices of an FFT stage sequence.  composite (FP32): pairs of small primes
-// are fused into radices 21, 14, 9 and 6 where possible (one shared-memory
-// pass each; fft.cuh), measured on the 7-smooth lengths of lmax 4096.
-std::vector<int> factorize(int n, bool composite)
+// Radices of an FFT stage sequence.  composite: pairs of small primes are fused into radices 9 and 6 (1: double-float),
+// 21 and 14 too (2: FP32), where possible (one shared-memory pass each; fft.cuh).
+std::vector<int> factorize(int n, int composite)
 {
     std::vector<int> f;
     while (n % 8 == 0) { f.push_back(8); n /= 8; }
@@ -193,8 +193,8 @@ std::vector<int> factorize(int n, bool composite)
     while (n % 5 == 0) { ++a5; n /= 5; }
     while (n % 7 == 0) { ++a7; n /= 7; }
     if (composite) {
-        for (; a3 > 0 && a7 > 0; --a3, --a7) f.push_back(21);
-        for (; a2 > 0 && a7 > 0; --a2, --a7) f.push_back(14);
+        for (; composite == 2 && a3 > 0 && a7 > 0; --a3, --a7) f.push_back(21);
+        for (; composite == 2 && a2 > 0 && a7 > 0; --a2, --a7) f.push_back(14);
         for (; a3 > 1; a3 -= 2) f.push_back(9);
         for (; a2 > 0 && a3 > 0; --a2, --a3) f.push_back(6);
     }
@@ -225,10 +225,10 @@ struct Builder {
         if (e != cudaSuccess) return e;
         return cudaMemcpy(*ptr, v.data(), v.size() * sizeof(V), cudaMemcpyHostToDevice);
     }
-    cudaError_t fft(FftDesc &d, int n)
+    cudaError_t fft(FftDesc &d, int n, bool dd)
     {
         d.n = n;
-        std::vector<int> f = factorize(n, p.prec == LENS_FP32);
+        std::vector<int> f = factorize(n, p.prec == LENS_FP32 ? 2 : dd ? 1 : 0);
         d.nst = (int)f.size();
         for (int i = 0; i < d.nst; ++i) d.radix[i] = f[i];
         std::vector<int> perm(n);
@@ -250,6 +250,13 @@ struct Builder {
         if (p.prec == LENS_FP32) {
             std::vector<float2> t(n);
             for (int i = 0; i < n; ++i) t[i] = make_float2((float)cos(2 * kPi * i / n), (float)-sin(2 * kPi * i / n));
+            e = upload(&tw, t);
+        } else if (dd) {
+            std::vector<float4> t(n);
+            for (int i = 0; i < n; ++i) {
+                const dfl c(cos(2 * kPi * i / n)), s(-sin(2 * kPi * i / n));
+                t[i] = make_float4(c.h, c.l, s.h, s.l);
+            }
             e = upload(&tw, t);
         } else {
             std::vector<double2> t(n);
@@ -612,6 +619,7 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
             p->m_df = 0;
             p->ck_klog.resize(mmax + 1);
             for (int m = 0; m <= mmax; ++m) p->ck_klog[m] = (unsigned char)std::log2(k_of(m, K));
+            p->fft_dd = true;
         }
     }
     // ---- Legendre launch shapes: RPT rings per thread; warps per CTA chosen
@@ -839,10 +847,21 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
             if ((e = B.upload(&p->w1, w1)) != cudaSuccess) return bailc(e, "upload w1");
             if ((e = B.upload(&p->w2, w2)) != cudaSuccess) return bailc(e, "upload w2");
         }
+        if (p->fft_dd) {
+            std::vector<float2> f1(w1.size()), f2(w2.size());
+            const auto pair = [](double v) { const dfl d(v); return make_float2(d.h, d.l); };
+            std::transform(w1.begin(), w1.end(), f1.begin(), pair);
+            std::transform(w2.begin(), w2.end(), f2.begin(), pair);
+            if ((e = B.upload(&p->w1d, f1)) != cudaSuccess) return bailc(e, "upload w1");
+            if ((e = B.upload(&p->w2d, f2)) != cudaSuccess) return bailc(e, "upload w2");
+        }
     }
-    if ((e = B.fft(p->fM, p->M)) != cudaSuccess) return bailc(e, "fft tables");
-    if ((e = B.fft(p->fN1, p->N1)) != cudaSuccess) return bailc(e, "fft tables");
-    if ((e = B.fft(p->fN2, p->N2)) != cudaSuccess) return bailc(e, "fft tables");
+    if ((e = B.fft(p->fM, p->M, false)) != cudaSuccess || (e = B.fft(p->fN1, p->N1, false)) != cudaSuccess ||
+        (e = B.fft(p->fN2, p->N2, false)) != cudaSuccess)
+        return bailc(e, "fft tables");
+    if (p->fft_dd && ((e = B.fft(p->dM, p->M, true)) != cudaSuccess || (e = B.fft(p->dN1, p->N1, true)) != cudaSuccess ||
+                      (e = B.fft(p->dN2, p->N2, true)) != cudaSuccess))
+        return bailc(e, "fft tables");
 
     if ((e = launch_rec_tables(*p)) != cudaSuccess) return bailc(e, "recursion tables");
     if (p->rst) {  // (FP32: step table, then) restart values from the FP64 recursion
@@ -996,7 +1015,7 @@ struct DeviceGuard {
 int forward_one(const Plan &p, const void *alm, void *map, cudaStream_t st, double wpos = 1.0)
 {
     cudaError_t e;
-    if ((e = staged(p, 0, st, [&] { return launch_legendre_fwd(p, alm, p.ring, st, wpos); })) != cudaSuccess)
+    if ((e = staged(p, 0, st, [&] { return launch_legendre_fwd(p, alm, p.ring, st, wpos, p.fft_dd); })) != cudaSuccess)
         return cuda_fail(e, "legendre synthesis");
     if ((e = staged(p, 1, st, [&] { return launch_theta_fwd(p, p.ring, p.X, st); })) != cudaSuccess)
         return cuda_fail(e, "theta transform");

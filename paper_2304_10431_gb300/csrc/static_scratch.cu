@@ -80,7 +80,7 @@ extern "C" int lens_synthesis_static(lens_plan pl, const void *alm_d, void *map_
     void *X = b + align256(ring_b);
     void *grid = b + align256(ring_b) + align256(x_b);
     cudaStream_t st = stream ? (cudaStream_t)stream : p.stream;
-    cudaError_t e = launch_legendre_fwd(p, alm_d, ring, st);  // zeroes the ring coefficients first
+    cudaError_t e = launch_legendre_fwd(p, alm_d, ring, st, 1.0, p.fft_dd);  // writes every ring coefficient
     if (e == cudaSuccess) e = launch_theta_fwd(p, ring, X, st);
     if (e == cudaSuccess) e = launch_phi_fwd(p, X, grid, st);
     if (e == cudaSuccess) e = launch_interp(p, grid, map_d, st);

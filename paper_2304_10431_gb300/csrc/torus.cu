@@ -22,6 +22,8 @@
 // fold j and M - j with (-1)^{m+s}).
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "fft.cuh"
 #include "internal.h"
@@ -48,6 +50,9 @@ template <> __device__ __forceinline__ Buf<double2, 1> make_buf<double2, 1>(doub
 {
     return Buf<double2, 1>(l);
 }
+template <> __device__ __forceinline__ Buf<dfl2, 1> make_buf<dfl2, 1>(dfl2 *l, int) { return Buf<dfl2, 1>(l); }
+template <> __device__ __forceinline__ Buf<dfl2, 2> make_buf<dfl2, 2>(dfl2 *l, int ch) { return Buf<dfl2, 2>(l, ch); }
+template <> __device__ __forceinline__ Buf<dfl2, 4> make_buf<dfl2, 4>(dfl2 *l, int ch) { return Buf<dfl2, 4>(l, ch); }
 template <> __device__ __forceinline__ Buf<float2, 2> make_buf<float2, 2>(float2 *l, int ch)
 {
     return Buf<float2, 2>(l, ch);
@@ -87,10 +92,11 @@ template <typename T> __device__ __forceinline__ cplx<T> pack_i(cplx<T> a, cplx<
 }
 // (u + p v) / 2 and (u + q v) / 2i for q = -p: the parts of the two columns
 template <typename T>
-__device__ __forceinline__ void split_pair(cplx<T> u, cplx<T> v, T p1, cplx<T> &x1, cplx<T> &x2)
+__device__ __forceinline__ void split_pair(cplx<T> u, cplx<T> v, sgn<T> p1, cplx<T> &x1, cplx<T> &x2)
 {
-    const cplx<T> s = mkc(T(0.5) * (u.x + p1 * v.x), T(0.5) * (u.y + p1 * v.y));  // (u + p1 v) / 2
-    const cplx<T> d = mkc(T(0.5) * (u.x - p1 * v.x), T(0.5) * (u.y - p1 * v.y));  // (u + p2 v) / 2, p2 = -p1
+    constexpr sgn<T> h = sgn<T>(0.5);
+    const cplx<T> s = mkc(h * (u.x + p1 * v.x), h * (u.y + p1 * v.y));  // (u + p1 v) / 2
+    const cplx<T> d = mkc(h * (u.x - p1 * v.x), h * (u.y - p1 * v.y));  // (u + p2 v) / 2, p2 = -p1
     x1 = s;
     x2 = mkc(d.y, -d.x);  // d / i
 }
@@ -109,19 +115,19 @@ __global__ void __launch_bounds__(512, OCC) k_theta_fwd(const cplx<T> *__restric
     const int c1 = 2 * tm.vec(), c2 = c1 + 1;
     const bool has2 = c2 < ncol;
     const int mc = spin == 0 ? c1 : c1 - mmax;
-    const T p1 = ((mc + spin) & 1) ? T(-1) : T(1), p2 = -p1;
+    const sgn<T> p1 = ((mc + spin) & 1) ? sgn<T>(-1) : sgn<T>(1), p2 = -p1;
     const int M = fM.n, N1 = fN1.n, N = ntheta - 1;
     const int tid = tm.tid, nthr = tm.nthr;
     const C *F1 = ring + (int64_t)c1 * ntheta;
     const C *F2 = ring + (int64_t)c2 * ntheta;
-    const C zero = mkc(T(0), T(0));
+    const C zero = mkc(T(0.0), T(0.0));
 
     for (int i = tid; i < M; i += nthr) {
         const int j = i < ntheta ? i : M - i;
         const bool pole = j == 0 || j == N;
         C a = F1[j], b = has2 ? F2[j] : zero;
         if (i >= ntheta) { a = cscale(a, p1); b = cscale(b, p2); }
-        if (pole) { if (p1 < T(0)) a = zero; else b = zero; }
+        if (pole) { if (p1 < sgn<T>(0)) a = zero; else b = zero; }
         buf[__ldg(fM.perm + i)] = pack_i<T>(a, b);
     }
     tm.sync();
@@ -130,7 +136,7 @@ __global__ void __launch_bounds__(512, OCC) k_theta_fwd(const cplx<T> *__restric
     // split (k, -k), weight by w1(k) w2(m) per column, recombine at k and N1 - k; the
     // other positions become zero.  In one pass when the source range of the negative
     // frequencies [M - lmax, M) lies below their target [N1 - lmax, N1)
-    const T wa = w2[c1], wb = has2 ? w2[c2] : T(0);
+    const T wa = w2[c1], wb = has2 ? w2[c2] : T(0.0);
     auto pair_at = [&](int k, C zk, C zm, C &bk, C &bm) {
         C x1, x2;
         split_pair<T>(zk, zm, p1, x1, x2);
@@ -303,6 +309,16 @@ __global__ void __launch_bounds__(512, OCC) k_theta_adj(const cplx<T> *__restric
     if (CL > 1) tm.sync();
 }
 
+// Grid values: plain reals in memory (double for double-float transforms), or double-float pairs
+template <typename T> struct grid_of { using type = T; };
+template <> struct grid_of<dfl> { using type = double; };
+template <typename T> using grid_real = typename grid_of<T>::type;
+__device__ __forceinline__ float plain(float v) { return v; }
+__device__ __forceinline__ double plain(double v) { return v; }
+__device__ __forceinline__ double plain(dfl v) { return dfl_value(v); }
+__device__ __forceinline__ df32 pair_of(double v) { return df_split(v); }
+__device__ __forceinline__ df32 pair_of(dfl v) { return df_renorm(df32{v.h, v.l}); }
+
 // ------------------------------------------------------------------- phi fwd
 // spin 0: team = row pair (2b, 2b+1); spin s: team = one row.
 template <typename T, bool SPIN, int CL, int OCC = 1>
@@ -317,7 +333,7 @@ __global__ void __launch_bounds__(512, OCC) k_phi_fwd(const cplx<T> *__restrict_
     const Buf<C, CL> buf = make_buf<C, CL>(reinterpret_cast<C *>(smem_raw), chunk);
     const int N2 = fN2.n;
     const int tid = tm.tid, nthr = tm.nthr;
-    for (int i = tid; i < N2; i += nthr) buf[i] = mkc(T(0), T(0));
+    for (int i = tid; i < N2; i += nthr) buf[i] = mkc(T(0.0), T(0.0));
     tm.sync();
     if (!SPIN) {
         const int ra = 2 * tm.vec(), rb = ra + 1;
@@ -326,7 +342,7 @@ __global__ void __launch_bounds__(512, OCC) k_phi_fwd(const cplx<T> *__restrict_
         const C *xb = X + (int64_t)rb * ncol;
         for (int m = tid; m <= mmax; m += nthr) {
             C a = xa[m];
-            C b = hb ? xb[m] : mkc(T(0), T(0));
+            C b = hb ? xb[m] : mkc(T(0.0), T(0.0));
             if (m == 0) {
                 buf[__ldg(fN2.perm + 0)] = mkc(a.x, b.x);
             } else {
@@ -337,22 +353,26 @@ __global__ void __launch_bounds__(512, OCC) k_phi_fwd(const cplx<T> *__restrict_
         }
         tm.sync();
         fft_smem<+1, T, CL>(buf, fN2, tm);
-        if (sizeof(T) == 8 && dd) {  // double-float pairs for k_interp_dd
+        if constexpr (!std::is_same<T, float>::value) if (dd) {  // double-float pairs for k_interp_dd
             float2 *ga = (float2 *)grid + (int64_t)ra * pitch;
             float2 *gb = (float2 *)grid + (int64_t)rb * pitch;
             for (int c = tid; c < N2 + W - 1; c += nthr) {
-                C v = buf[c < N2 ? c : c - N2];
-                const df32 x = df_split((double)v.x), y = df_split((double)v.y);
+                const C v = buf[c < N2 ? c : c - N2];
+                const df32 x = pair_of(v.x), y = pair_of(v.y);
                 ga[c] = make_float2(x.h, x.l);
                 if (hb) gb[c] = make_float2(y.h, y.l);
             }
-        } else {
-            T *ga = (T *)grid + (int64_t)ra * pitch;
-            T *gb = (T *)grid + (int64_t)rb * pitch;
+            if (CL > 1) tm.sync();
+            return;
+        }
+        {
+            using G = grid_real<T>;
+            G *ga = (G *)grid + (int64_t)ra * pitch;
+            G *gb = (G *)grid + (int64_t)rb * pitch;
             for (int c = tid; c < N2 + W + 1; c += nthr) {  // two zeros past the wrap columns (k_interp32)
-                const C v = c < N2 + W - 1 ? buf[c < N2 ? c : c - N2] : mkc(T(0), T(0));
-                ga[c] = v.x;
-                if (hb) gb[c] = v.y;
+                const C v = c < N2 + W - 1 ? buf[c < N2 ? c : c - N2] : mkc(T(0.0), T(0.0));
+                ga[c] = plain(v.x);
+                if (hb) gb[c] = plain(v.y);
             }
         }
     } else {
@@ -364,17 +384,23 @@ __global__ void __launch_bounds__(512, OCC) k_phi_fwd(const cplx<T> *__restrict_
         }
         tm.sync();
         fft_smem<+1, T, CL>(buf, fN2, tm);
-        if (sizeof(T) == 8 && dd) {
+        if constexpr (!std::is_same<T, float>::value) if (dd) {
             float4 *gr = (float4 *)grid + (int64_t)r * pitch;
             for (int c = tid; c < N2 + W - 1; c += nthr) {
                 const C v = buf[c < N2 ? c : c - N2];
-                const df32 x = df_split((double)v.x), y = df_split((double)v.y);
+                const df32 x = pair_of(v.x), y = pair_of(v.y);
                 gr[c] = make_float4(x.h, x.l, y.h, y.l);
             }
-        } else {
-            C *gr = (C *)grid + (int64_t)r * pitch;
-            for (int c = tid; c < N2 + W + 1; c += nthr)
-                gr[c] = c < N2 + W - 1 ? buf[c < N2 ? c : c - N2] : mkc(T(0), T(0));
+            if (CL > 1) tm.sync();
+            return;
+        }
+        {
+            using G = cplx<grid_real<T>>;
+            G *gr = (G *)grid + (int64_t)r * pitch;
+            for (int c = tid; c < N2 + W + 1; c += nthr) {
+                const C v = c < N2 + W - 1 ? buf[c < N2 ? c : c - N2] : mkc(T(0.0), T(0.0));
+                gr[c] = mkc(plain(v.x), plain(v.y));
+            }
         }
     }
     if (CL > 1) tm.sync();
@@ -484,14 +510,15 @@ template <typename T>
 cudaError_t theta_fwd_t(const Plan &p, const void *ring, void *X, cudaStream_t st)
 {
     using C = cplx<T>;
+    constexpr bool DD = std::is_same<T, dfl>::value;
     const size_t sm = theta_smem_bytes(p);
     const int chunk = (int)(sm / sizeof(C));
     auto args = [&](auto kern) {
-        return launch_team(kern, p.cl_theta, (p.ncol + 1) / 2, kThetaThreads, sm, st, (const C *)ring, (C *)X, p.fM, p.fN1,
-                           (const T *)p.w1, (const T *)p.w2, p.ntheta, p.lmax, p.mmax, p.spin, p.ncol, p.r_lo, p.R,
+        return launch_team(kern, p.cl_theta, (p.ncol + 1) / 2, kThetaThreads, sm, st, (const C *)ring, (C *)X, DD ? p.dM : p.fM,
+                           DD ? p.dN1 : p.fN1, (const T *)(DD ? p.w1d : p.w1), (const T *)(DD ? p.w2d : p.w2), p.ntheta, p.lmax, p.mmax, p.spin, p.ncol, p.r_lo, p.R,
                            chunk);
     };
-    if constexpr (sizeof(T) == 4)
+    if constexpr (std::is_same<T, float>::value)
         if (p.cl_theta == 1 && sm <= kTwoCtaSmem) return args(k_theta_fwd<T, 1, 2>);
     return p.cl_theta == 4 ? args(k_theta_fwd<T, 4>) : p.cl_theta == 2 ? args(k_theta_fwd<T, 2>) : args(k_theta_fwd<T, 1>);
 }
@@ -507,7 +534,7 @@ cudaError_t theta_adj_t(const Plan &p, const void *X, void *ring, cudaStream_t s
                            (const T *)p.w1, (const T *)p.w2, p.ntheta, p.lmax, p.mmax, p.spin, p.ncol, p.r_lo, p.R,
                            chunk);
     };
-    if constexpr (sizeof(T) == 4)
+    if constexpr (std::is_same<T, float>::value)
         if (p.cl_theta == 1 && sm <= kTwoCtaSmem) return args(k_theta_adj<T, 1, 2>);
     return p.cl_theta == 4 ? args(k_theta_adj<T, 4>) : p.cl_theta == 2 ? args(k_theta_adj<T, 2>) : args(k_theta_adj<T, 1>);
 }
@@ -521,10 +548,11 @@ cudaError_t phi_fwd_t(const Plan &p, const void *X, void *grid, cudaStream_t st)
     const int nvec = SPIN ? p.R : (p.R + 1) / 2;
     auto args = [&](auto kern) {
         // FP64 plans with point weights interpolate in double-float: the grid as double-float pairs
-        return launch_team(kern, p.cl_phi, nvec, phi_threads(p), sm, st, (const C *)X, grid, p.fN2, p.mmax, p.ncol,
-                           p.R, p.pitch, p.W, chunk, (sizeof(T) == 8 && p.wts && p.wts_dd) ? 1 : 0);
+        return launch_team(kern, p.cl_phi, nvec, std::is_same<T, dfl>::value ? 512 : phi_threads(p), sm, st, (const C *)X, grid,
+                           std::is_same<T, dfl>::value ? p.dN2 : p.fN2, p.mmax, p.ncol,
+                           p.R, p.pitch, p.W, chunk, (!std::is_same<T, float>::value && p.wts && p.wts_dd) ? 1 : 0);
     };
-    if constexpr (sizeof(T) == 4)
+    if constexpr (std::is_same<T, float>::value)
         if (p.cl_phi == 1 && sm <= kTwoCtaSmem) return args(k_phi_fwd<T, SPIN, 1, 2>);
     return p.cl_phi == 4   ? args(k_phi_fwd<T, SPIN, 4>)
            : p.cl_phi == 2 ? args(k_phi_fwd<T, SPIN, 2>)
@@ -542,7 +570,7 @@ cudaError_t phi_adj_t(const Plan &p, const void *grid, void *X, cudaStream_t st)
         return launch_team(kern, p.cl_phi, nvec, phi_threads(p), sm, st, (const void *)grid, (C *)X, p.fN2, p.mmax,
                            p.ncol, p.R, p.pitch, p.W, chunk);
     };
-    if constexpr (sizeof(T) == 4)
+    if constexpr (std::is_same<T, float>::value)
         if (p.cl_phi == 1 && sm <= kTwoCtaSmem) return args(k_phi_adj<T, SPIN, 1, 2>);
     return p.cl_phi == 4   ? args(k_phi_adj<T, SPIN, 4>)
            : p.cl_phi == 2 ? args(k_phi_adj<T, SPIN, 2>)
@@ -553,6 +581,7 @@ cudaError_t phi_adj_t(const Plan &p, const void *grid, void *X, cudaStream_t st)
 
 cudaError_t launch_theta_fwd(const Plan &p, const void *ring, void *X, cudaStream_t st)
 {
+    if (p.fft_dd) return theta_fwd_t<dfl>(p, ring, X, st);
     return p.prec == LENS_FP32 ? theta_fwd_t<float>(p, ring, X, st) : theta_fwd_t<double>(p, ring, X, st);
 }
 
@@ -581,6 +610,7 @@ cudaError_t launch_theta_adj(const Plan &p, const void *X, void *ring, cudaStrea
 
 cudaError_t launch_phi_fwd(const Plan &p, const void *X, void *grid, cudaStream_t st)
 {
+    if (p.fft_dd) return p.spin ? phi_fwd_t<dfl, true>(p, X, grid, st) : phi_fwd_t<dfl, false>(p, X, grid, st);
     if (p.prec == LENS_FP32) return p.spin ? phi_fwd_t<float, true>(p, X, grid, st) : phi_fwd_t<float, false>(p, X, grid, st);
     return p.spin ? phi_fwd_t<double, true>(p, X, grid, st) : phi_fwd_t<double, false>(p, X, grid, st);
 }
