@@ -476,7 +476,15 @@ size_t phi_smem_bytes(const Plan &p)
 namespace {
 
 constexpr int kThetaThreads = 512;
-int phi_threads(const Plan &p) { return p.prec == LENS_FP32 ? 512 : 256; }
+// Threads per vector: a stage of a vector of n elements has n / radix butterflies, so short vectors keep few threads busy,
+// and several CTAs per SM cover each other's barriers and table reads (us at 512 threads / this rule; FP32 spin 0,
+// lmax 1024, n 3600: theta 55 / 42, phi 51 / 40; FP32 spin 2, lmax 512, n 1800: 44 / 29, 36 / 23; FP64 spin 2, lmax 2048, n 5760:
+// 2452 / 2264, 1678 / 1558; double-float: 697 / 589, 513 / 440).
+// Up to 1024 (FP32 theta) or 4096 elements: 128 threads. Two CTAs of 256 still fit an SM's shared memory up to about 8000 elements;
+// beyond, 256 to 512 threads measured within 2% of one another, and 512 wins for FP64 phi (5.53 ms / 5.29 at n 11520).
+int fft_threads(int n, bool short_ok) { return n <= 1024 || (short_ok && n <= 4096) ? 128 : n <= 8000 ? 256 : 512; }
+int theta_threads(const Plan &p) { return fft_threads(p.N1, p.prec == LENS_FP64); }
+int phi_threads(const Plan &p) { return fft_threads(p.N2, true); }
 // Two 512-thread CTAs per SM need at most 64 registers per thread and half the
 // SM's shared memory each; FP32 single-CTA vectors that fit then run the
 // variant compiled for two CTAs per SM (measured at lmax 4096, sigma 1.5:
@@ -514,7 +522,7 @@ cudaError_t theta_fwd_t(const Plan &p, const void *ring, void *X, cudaStream_t s
     const size_t sm = theta_smem_bytes(p);
     const int chunk = (int)(sm / sizeof(C));
     auto args = [&](auto kern) {
-        return launch_team(kern, p.cl_theta, (p.ncol + 1) / 2, kThetaThreads, sm, st, (const C *)ring, (C *)X, DD ? p.dM : p.fM,
+        return launch_team(kern, p.cl_theta, (p.ncol + 1) / 2, theta_threads(p), sm, st, (const C *)ring, (C *)X, DD ? p.dM : p.fM,
                            DD ? p.dN1 : p.fN1, (const T *)(DD ? p.w1d : p.w1), (const T *)(DD ? p.w2d : p.w2), p.ntheta, p.lmax, p.mmax, p.spin, p.ncol, p.r_lo, p.R,
                            chunk);
     };
@@ -530,7 +538,7 @@ cudaError_t theta_adj_t(const Plan &p, const void *X, void *ring, cudaStream_t s
     const size_t sm = theta_smem_bytes(p);
     const int chunk = (int)(sm / sizeof(C));
     auto args = [&](auto kern) {
-        return launch_team(kern, p.cl_theta, (p.ncol + 1) / 2, kThetaThreads, sm, st, (const C *)X, (C *)ring, p.fM, p.fN1,
+        return launch_team(kern, p.cl_theta, (p.ncol + 1) / 2, theta_threads(p), sm, st, (const C *)X, (C *)ring, p.fM, p.fN1,
                            (const T *)p.w1, (const T *)p.w2, p.ntheta, p.lmax, p.mmax, p.spin, p.ncol, p.r_lo, p.R,
                            chunk);
     };
@@ -548,7 +556,7 @@ cudaError_t phi_fwd_t(const Plan &p, const void *X, void *grid, cudaStream_t st)
     const int nvec = SPIN ? p.R : (p.R + 1) / 2;
     auto args = [&](auto kern) {
         // FP64 plans with point weights interpolate in double-float: the grid as double-float pairs
-        return launch_team(kern, p.cl_phi, nvec, std::is_same<T, dfl>::value ? 512 : phi_threads(p), sm, st, (const C *)X, grid,
+        return launch_team(kern, p.cl_phi, nvec, phi_threads(p), sm, st, (const C *)X, grid,
                            std::is_same<T, dfl>::value ? p.dN2 : p.fN2, p.mmax, p.ncol,
                            p.R, p.pitch, p.W, chunk, (!std::is_same<T, float>::value && p.wts && p.wts_dd) ? 1 : 0);
     };
