@@ -240,55 +240,96 @@ __global__ void __launch_bounds__(256) k_interp32(const float *__restrict__ grid
     }
 }
 
-// FP64 plans with point weights: the same sums in double-float arithmetic on
-// the FP32 pipe.  The grid holds double-float pairs (k_phi_fwd writes them
-// for these plans: float2 per real, spin s float4 (re h, re l, im h, im l));
-// each row sum adds the exact products of the high words with two-sum and
-// the products' error terms and cross terms in the low word, then the rows
-// are combined the same way; ~2^-46 relative per term.
+// FP64 plans with point weights: the same sums in double-float arithmetic on the FP32 pipe.  The grid holds
+// double-float pairs (k_phi_fwd writes them for these plans: float2 per real, spin s float4 (re h, im h, re l, im l)); a
+// term is one d2_fma (pk.cuh) of both components of a column, or for spin 0 of two rows; row sums are
+// normalised before the theta weights; ~2^-46 relative per term.
+// A warp brings the weights of its 32 points (contiguous in the table) through shared memory with coalesced 16-byte
+// loads, each point's row padded to an odd number of 16-byte words (conflict-free LDS.128).  Bound by the FP32
+// pipe (11 instructions a tap) and the grid loads, whose lanes cover about three rows of a tile.  Spin 2,
+// lmax 2048, 12.6M points, W = 13 (FP64 eps 1e-10): 3.09 ms with the weights read by each thread (3W loads of 32 separate
+// lines) and scalar sums, 2.87 with the weights staged, 2.05 with packed sums; spin 0: 1.45 staged, 1.38 packed.
+// Four CTAs per SM (128 registers): 2.05 ms; three 2.13, five 2.08, six 2.17.
+constexpr int kInterpDD = 128;  // threads per CTA
 template <int W, bool SPIN>
-__global__ void __launch_bounds__(256) k_interp_dd(const void *__restrict__ grid, const uint32_t *__restrict__ cell,
-                                                   const int32_t *__restrict__ perm, const double2 *__restrict__ phase,
-                                                   const double *__restrict__ wts, double *__restrict__ map,
-                                                   int64_t n, int pitch)
+__global__ void __launch_bounds__(kInterpDD, 4) k_interp_dd(const void *__restrict__ grid, const uint32_t *__restrict__ cell,
+                                                            const int32_t *__restrict__ perm,
+                                                            const double2 *__restrict__ phase,
+                                                            const double *__restrict__ wts, double *__restrict__ map,
+                                                            int64_t n, int pitch)
 {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    constexpr int NP = dd_pairs(W), Q = dd_words(W) / 4;  // 16-byte words per point: Q even, rows of Q + 1
+    __shared__ float4 sw[kInterpDD * (Q + 1)];
+    const int lane = threadIdx.x & 31;
+    const int64_t p = (int64_t)blockIdx.x * kInterpDD + threadIdx.x, p0 = p - lane;
+    float4 *wrow = sw + (threadIdx.x - lane) * (Q + 1);
+    const int words = (int)min((int64_t)32, n - p0) * Q;
+    const float4 *wg = reinterpret_cast<const float4 *>(wts) + p0 * Q;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+        const int i = k * 32 + lane;
+        if (i < words) wrow[i / Q * (Q + 1) + i % Q] = __ldg(wg + i);
+    }
+    __syncwarp();
     if (p >= n) return;
     const uint32_t c0 = cell[p];
-    const float *w = dd_weights<W>(wts, p);
-    df32 wb[W];
-#pragma unroll
-    for (int b = 0; b < W; ++b) wb[b] = dd_phi<W>(w, b);
     const int32_t dst = perm[p];
+    const float4 *w = wrow + lane * (Q + 1);
     if (!SPIN) {
-        const float2 *g = reinterpret_cast<const float2 *>(grid) + c0;
-        df32 acc = {0.f, 0.f};
+        df32 wb[2 * NP];
 #pragma unroll
-        for (int a = 0; a < W; ++a) {
-            df32 r = {0.f, 0.f};
-#pragma unroll
-            for (int b = 0; b < W; ++b) df_acc(r, df_mul(wb[b], ld_df(g + (int64_t)a * pitch + b)));
-            df_acc(acc, df_mul(dd_theta<W>(w, a), df_renorm(r)));
+        for (int i = 0; i < NP; ++i) {
+            const float4 v = w[NP + i];
+            wb[2 * i] = {v.x, v.y};
+            wb[2 * i + 1] = {v.z, v.w};
         }
-        map[dst] = df_value(acc);
-    } else {
-        const float4 *g = reinterpret_cast<const float4 *>(grid) + c0;
-        df32 ax = {0.f, 0.f}, ay = {0.f, 0.f};
+        const float2 *g = reinterpret_cast<const float2 *>(grid) + c0;
+        D2 acc = {0ull, 0ull};  // rows in pairs; an odd W's last row twice, the second time with weight zero
 #pragma unroll
-        for (int a = 0; a < W; ++a) {
-            df32 rx = {0.f, 0.f}, ry = {0.f, 0.f};
+        for (int i = 0; i < NP; ++i) {
+            const float2 *ga = g + (int64_t)(2 * i) * pitch, *gb = 2 * i + 1 < W ? ga + pitch : ga;
+            D2 r = {0ull, 0ull};
 #pragma unroll
             for (int b = 0; b < W; ++b) {
-                const float4 v = __ldg(g + (int64_t)a * pitch + b);
-                df_acc(rx, df_mul(wb[b], df32{v.x, v.y}));
-                df_acc(ry, df_mul(wb[b], df32{v.z, v.w}));
+                const float2 x = __ldg(ga + b), y = __ldg(gb + b);
+                r = d2_fma(D2{pk_make(x.x, y.x), pk_make(x.y, y.y)}, D2{pk_make(wb[b].h, wb[b].h), pk_make(wb[b].l, wb[b].l)}, r);
             }
-            const df32 wa = dd_theta<W>(w, a);
-            df_acc(ax, df_mul(wa, df_renorm(rx)));
-            df_acc(ay, df_mul(wa, df_renorm(ry)));
+            const ulonglong2 wa = reinterpret_cast<const ulonglong2 *>(w)[i];
+            acc = d2_fma(d2_norm(r), D2{wa.x, wa.y}, acc);
         }
+        const float2 sh = pk_get(acc.h), sl = pk_get(acc.l);
+        map[dst] = df_value(df32{sh.x, sl.x}) + df_value(df32{sh.y, sl.y});
+    } else {
+        // both components in one packed instruction (grid: re h, im h, re l, im l)
+        df32 wb[2 * NP];
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            const float4 v = w[NP + i];
+            wb[2 * i] = {v.x, v.y};
+            wb[2 * i + 1] = {v.z, v.w};
+        }
+        const ulonglong2 *g = reinterpret_cast<const ulonglong2 *>(grid) + c0;
+        D2 acc = {0ull, 0ull};
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            const float4 wa = w[i];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int a = 2 * i + k;
+                if (a >= W) continue;
+                D2 r = {0ull, 0ull};
+#pragma unroll
+                for (int b = 0; b < W; ++b) {
+                    const ulonglong2 v = __ldg(g + (int64_t)a * pitch + b);
+                    r = d2_fma(D2{v.x, v.y}, D2{pk_make(wb[b].h, wb[b].h), pk_make(wb[b].l, wb[b].l)}, r);
+                }
+                const df32 t = k ? df32{wa.y, wa.w} : df32{wa.x, wa.z};
+                acc = d2_fma(d2_norm(r), D2{pk_make(t.h, t.h), pk_make(t.l, t.l)}, acc);
+            }
+        }
+        const float2 sh = pk_get(acc.h), sl = pk_get(acc.l);
         const double2 ph = phase[p];
-        const double x = df_value(ax), y = df_value(ay);
+        const double x = df_value(df32{sh.x, sl.x}), y = df_value(df32{sh.y, sl.y});
         map[dst] = x * ph.x - y * ph.y;
         map[n + dst] = x * ph.y + y * ph.x;
     }
@@ -508,8 +549,8 @@ cudaError_t interp_w(const Plan &p, const void *grid, void *map, cudaStream_t st
     };
     if constexpr (std::is_same<T, double>::value) {
         if (p.wts && p.wts_dd) {  // double-float taps on the double-float grid k_phi_fwd wrote
-            k_interp_dd<W, SPIN><<<(unsigned)blocks, thr, 0, st>>>(grid, p.cell, p.perm, (const double2 *)p.phase,
-                                                                   p.wts, (double *)map, p.npts, p.pitch);
+            k_interp_dd<W, SPIN><<<(unsigned)((p.npts + kInterpDD - 1) / kInterpDD), kInterpDD, 0, st>>>(
+                grid, p.cell, p.perm, (const double2 *)p.phase, p.wts, (double *)map, p.npts, p.pitch);
             return cudaGetLastError();
         }
         if (p.wts) return run(k_interp<T, W, SPIN, 1>);

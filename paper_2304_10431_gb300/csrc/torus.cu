@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(512, OCC) k_phi_fwd(const cplx<T> *__restrict_
             for (int c = tid; c < N2 + W - 1; c += nthr) {
                 const C v = buf[c < N2 ? c : c - N2];
                 const df32 x = pair_of(v.x), y = pair_of(v.y);
-                gr[c] = make_float4(x.h, x.l, y.h, y.l);
+                gr[c] = make_float4(x.h, y.h, x.l, y.l);
             }
             if (CL > 1) tm.sync();
             return;
