@@ -16,6 +16,7 @@ constexpr int kScaleBits = 60;       // exponent step of the scaled Legendre rec
 constexpr int kLegBlock = 8;         // degrees per unrolled block of the Legendre kernels
 constexpr int kTileR = 32, kTileC = 32;  // default grid tile of the point sort (rows x columns)
 constexpr int kMaxW = 16;                 // largest kernel support
+constexpr int grid_pitch(int columns) { return (columns + 31) / 32 * 32; }  // row length of the grid
 // Double-float kernel weights of a point: the theta taps in pairs (h0, h1, l0, l1), one operand pair of a packed
 // instruction per 8 bytes, then the phi taps (h, l); both padded with zeros to an even count.
 __host__ __device__ constexpr int dd_pairs(int W) { return (W + 1) / 2; }

@@ -245,8 +245,8 @@ __global__ void __launch_bounds__(256) k_interp32(const float *__restrict__ grid
 // term is one d2_fma (pk.cuh) of both components of a column, or for spin 0 of two rows; row sums are
 // normalised before the theta weights; ~2^-46 relative per term.
 // A warp brings the weights of its 32 points (contiguous in the table) through shared memory with coalesced 16-byte
-// loads, each point's row padded to an odd number of 16-byte words (conflict-free LDS.128).  Bound by the FP32
-// pipe (11 instructions a tap) and the grid loads, whose lanes cover about three rows of a tile.  Spin 2,
+// loads, each point's row padded to an odd number of 16-byte words (conflict-free LDS.128).  Bound by the L1
+// data stage (92% busy: the grid loads, whose lanes cover about three rows of a tile); FMA pipe 58%.  Spin 2,
 // lmax 2048, 12.6M points, W = 13 (FP64 eps 1e-10): 3.09 ms with the weights read by each thread (3W loads of 32 separate
 // lines) and scalar sums, 2.87 with the weights staged, 2.05 with packed sums; spin 0: 1.45 staged, 1.38 packed.
 // Four CTAs per SM (128 registers): 2.05 ms; three 2.13, five 2.08, six 2.17.

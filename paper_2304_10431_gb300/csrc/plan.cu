@@ -532,7 +532,8 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
     }
     p->r_lo = -p->W;
     p->R = p->N1 / 2 + 2 * p->W + 1;
-    p->pitch = ((p->N2 + p->W + 1) + 31) / 32 * 32;  // W - 1 wrap columns and two zeros (k_interp32)
+    // W - 1 wrap columns; FP32 plans two zeros after them (k_interp32)
+    p->pitch = grid_pitch(p->N2 + p->W - 1 + (prec == LENS_FP32 ? 2 : 0));
 
     // ---- Legendre arithmetic: FP32 plans df32 for every m; FP64 plans native FP64
     // for m < m_df and df32 recursion + df32 accumulation for m >= m_df.  df32

@@ -29,7 +29,10 @@
 namespace {
 
 constexpr size_t kStaticScratchBytes = 64ull << 20;  // 64 MiB
-static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
+// FP32 grids may be 32 columns wider than their wrap columns need (two zeros, k_interp32): those columns do not count
+// against the limit and have room of their own, for up to 16384 rows
+constexpr size_t kStaticSlackBytes = 4ull << 20;
+static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes + kStaticSlackBytes];
 
 constexpr int kMaxDevices = 64;
 void *g_scratch_addr[kMaxDevices] = {nullptr};
@@ -47,8 +50,9 @@ extern "C" int lens_synthesis_static(lens_plan pl, const void *alm_d, void *map_
     const Plan &p = *reinterpret_cast<const Plan *>(pl);
     const ScratchSizes scr = plan_scratch_sizes(p);  // the plan builder's own workspace sizes
     const size_t ring_b = scr.ring, x_b = scr.X, grid_b = scr.grid;
-    const size_t need = align256(ring_b) + align256(x_b) + align256(grid_b);
-    if (need > kStaticScratchBytes) {
+    const size_t total = align256(ring_b) + align256(x_b) + align256(grid_b);
+    const size_t need = total - align256(grid_b) + align256(grid_b / p.pitch * grid_pitch(p.N2 + p.W - 1));
+    if (need > kStaticScratchBytes || total > kStaticScratchBytes + kStaticSlackBytes) {
         char msg[256];
         snprintf(msg, sizeof msg,
                  "lens_synthesis_static: the plan needs %zu bytes of scratch, above the fixed %zu-byte array; "

@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(512, OCC) k_phi_fwd(const cplx<T> *__restrict_
             using G = grid_real<T>;
             G *ga = (G *)grid + (int64_t)ra * pitch;
             G *gb = (G *)grid + (int64_t)rb * pitch;
-            for (int c = tid; c < N2 + W + 1; c += nthr) {  // two zeros past the wrap columns (k_interp32)
+            for (int c = tid; c < min(N2 + W + 1, pitch); c += nthr) {  // FP32: two zeros past the wrap columns (k_interp32)
                 const C v = c < N2 + W - 1 ? buf[c < N2 ? c : c - N2] : mkc(T(0.0), T(0.0));
                 ga[c] = plain(v.x);
                 if (hb) gb[c] = plain(v.y);
@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(512, OCC) k_phi_fwd(const cplx<T> *__restrict_
         {
             using G = cplx<grid_real<T>>;
             G *gr = (G *)grid + (int64_t)r * pitch;
-            for (int c = tid; c < N2 + W + 1; c += nthr) {
+            for (int c = tid; c < min(N2 + W + 1, pitch); c += nthr) {
                 const C v = c < N2 + W - 1 ? buf[c < N2 ? c : c - N2] : mkc(T(0.0), T(0.0));
                 gr[c] = mkc(plain(v.x), plain(v.y));
             }
