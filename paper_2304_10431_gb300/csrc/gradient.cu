@@ -85,8 +85,26 @@ __global__ void k_g_to_phi(const double2 *__restrict__ gg, double2 *__restrict__
     }
 }
 
+// (1 - cos a) / a^2 (k = 2) and (a - sin a) / a^3 (k = 3) for a^2 <= 1/4, from their Taylor series
+// sum_j (-1)^j a^(2j) / (2j + k)!: the first term left out is below 2^-60 of the first
+template <int K> __device__ __forceinline__ double small_angle(double a2)
+{
+    double f = 1.0;  // (2 J + K)! (all constants fold)
+#pragma unroll
+    for (int i = 2; i <= 14 + K; ++i) f *= i;
+    double r = -1.0 / f;
+#pragma unroll
+    for (int j = 6; j >= 0; --j) {
+        f /= (2 * j + K + 1) * (2 * j + K + 2);
+        r = fma(r, a2, (j & 1 ? -1.0 : 1.0) / f);
+    }
+    return r;
+}
+
 // dL/dalpha per point (FP64 arithmetic; inputs in the lensed plans' type T):
 // alpha [2][n], g / p [ncomp][n], A / B [2][n]; out [2][n] (theta, phi parts).
+// Bound by the FP64 pipe.  Deflections up to half a radian take J and the holonomy as power series in a^2, without
+// roots, divisions, sines and cosines; a gradient step of E/B at lmax 1024, 3.1M points: 6.46 -> 6.04 ms with it.
 template <typename T>
 __global__ void k_deflection_vjp(int64_t n, int spin, const double *__restrict__ alpha, const T *__restrict__ g,
                                  const T *__restrict__ p, const T *__restrict__ A, const T *__restrict__ B,
@@ -95,14 +113,27 @@ __global__ void k_deflection_vjp(int64_t n, int spin, const double *__restrict__
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double at = alpha[i], ap = alpha[n + i];
-    const double a = hypot(at, ap);
-    double hr = 1.0, hi = 0.0, k = 1.0, c = 0.0;
-    if (a > 0.0) {
-        hr = at / a;
-        hi = ap / a;
-        k = sin(a) / a;
-        const double sh = sin(0.5 * a);
-        c = 2.0 * sh * sh / a;
+    // J y = k y + w (v.y) v, holonomy term K (-v_phi, v_theta), K = -spin c Im(conj(g) P), where (v, w, c) =
+    // (alpha, (1 - k) / a^2, (1 - cos a) / a^2) or (alpha / a, 1 - k, (1 - cos a) / a), k = sin(a) / a
+    const double a2 = fma(at, at, ap * ap);
+    double vt = at, vp = ap, k, w, c;
+    if (a2 <= 0.25) {
+        c = small_angle<2>(a2);
+        w = small_angle<3>(a2);
+        k = fma(-a2, w, 1.0);
+    } else {
+        const double a = hypot(at, ap);
+        vt = 1.0;
+        vp = w = c = 0.0;
+        k = 1.0;
+        if (a > 0.0) {  // (false for NaN)
+            vt = at / a;
+            vp = ap / a;
+            k = sin(a) / a;
+            w = 1.0 - k;
+            const double sh = sin(0.5 * a);
+            c = 2.0 * sh * sh / a;
+        }
     }
     const double ar = A[i], ai = A[n + i];
     double yr, yi, K = 0.0;
@@ -114,18 +145,14 @@ __global__ void k_deflection_vjp(int64_t n, int spin, const double *__restrict__
         const double gq = g[i], gu = g[n + i];
         const double br = B[i], bi = B[n + i];
         // conj(g) A + g conj(B)
-        const double sr = (gq * ar + gu * ai) + (gq * br + gu * bi);
-        const double si = (gq * ai - gu * ar) + (gu * br - gq * bi);
-        yr = -0.5 * sr;
-        yi = -0.5 * si;
+        yr = -0.5 * (gq * (ar + br) + gu * (ai + bi));
+        yi = -0.5 * (gq * (ai - bi) + gu * (br - ar));
         const double pr = p[i], pi = p[n + i];
         K = -spin * c * (gq * pi - gu * pr);
     }
-    const double par = hr * yr + hi * yi;
-    const double jr = par * hr + k * (yr - par * hr);
-    const double ji = par * hi + k * (yi - par * hi);
-    out[i] = jr - K * hi;
-    out[n + i] = ji + K * hr;
+    const double q = w * (vt * yr + vp * yi);
+    out[i] = k * yr + q * vt - K * vp;
+    out[n + i] = k * yi + q * vp + K * vt;
 }
 
 const Plan *as_plan(lens_plan p) { return reinterpret_cast<const Plan *>(p); }
