@@ -1,4 +1,4 @@
-// Spreading of FP64 plans with double-float weights (epsilon >= 5e-11) and of FP32 plans with W >= 8 (or epsilon < 1e-5),
+// Spreading of FP64 plans with double-float weights (epsilon >= 5e-11) and of FP32 plans with W >= 8 (spin 0: W >= 10; or epsilon < 1e-5),
 // not deterministic: tiles swept row by row in registers.
 //
 // One warp owns a tile of tile_r rows x (33 - W) columns, so the W-wide windows of its points cover 32
@@ -207,11 +207,12 @@ k_spread_strip(double *__restrict__ grid, const uint32_t *__restrict__ cell, con
     while (cur < last) next_row();
 }
 
-// FP32 plans with W >= 8 (or epsilon < 1e-5): the same sweep with FP32 sums.  Each lane evaluates the 2W polynomial weights
+// FP32 plans with W >= 8 (spin 0: W >= 10; or epsilon < 1e-5): the same sweep with FP32 sums.  Each lane evaluates the 2W polynomial weights
 // of one point of a batch of 32 into shared memory (the coefficients come from the constant bank); then the warp
 // takes the points in turn.  Bound by issue: ~50 instructions per point whatever W, where the tiles of 32-bit
 // integers in shared memory (nufft.cuh) cost W^2 atomics: spin 2, lmax 4096, 50M points, W = 8: 3.07 -> 2.66 ms; W = 7: lmax 2048 0.66
-// against 0.69 ms, lmax 1024 0.17 against 0.22, so W <= 7 keeps the tiles.  Two tiles of 17 - W columns per warp, one per half,
+// against 0.69 ms, lmax 1024 0.17 against 0.22, so W <= 7 keeps the tiles; spin 0, whose tiles do half the atomics, up to W = 9
+// (lmax 4096, W = 8: tiles 1.65 ms, strips 1.85; lmax 2048, W = 10: 0.588, 0.554).  Two tiles of 17 - W columns per warp, one per half,
 // were tried for the lanes a point leaves idle: 2.83 ms, and the narrow tiles cost the interpolation 0.2-0.4 ms.
 template <int W> __host__ __device__ constexpr size_t strip32_warp_smem()
 {

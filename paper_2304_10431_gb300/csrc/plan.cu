@@ -740,9 +740,12 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
         // spreading taps in double-float on the FP32 pipe (~2^-46 relative per term; lmax 4096,
         // 50M points, W = 13: interpolation 30.1 -> 13.4 ms for spin 2); smaller epsilon keeps FP64
         const bool dd = keep && epsilon >= 5e-11;
-        // spreading by strips (nufft_strip.cuh; FP32 plans by tiles of 32-bit integers where those are faster): fewer rows
-        // per tile where the tiles would not fill the chip
-        if ((dd || (prec == LENS_FP32 && (p->W >= 8 || epsilon < 1e-5))) && !p->det) {
+        // spreading by strips (nufft_strip.cuh; FP32 plans by tiles of 32-bit integers where those are faster: a strip
+        // point costs ~50 instructions whatever W and for both components, a tile W^2 atomics for each; us at lmax
+        // 2048, 12.6M points, tiles / strips: spin 2 W 7 681 / 672, W 8 827 / 685, W 10 1177 / 810; spin 0 W 8 413 / 479, W 9
+        // 496 / 525, W 10 588 / 554, and the interpolation is 1-8% slower on the narrower tiles of strips): fewer
+        // rows per tile where the tiles would not fill the chip
+        if ((dd || (prec == LENS_FP32 && (p->W >= (spin ? 8 : 10) || epsilon < 1e-5))) && !p->det) {
             p->strip = true;
             p->tile_c = 33 - p->W;
             p->ntile_c = (p->N2 + p->tile_c - 1) / p->tile_c;
