@@ -240,22 +240,38 @@ def fp64_arithmetic(info):
     else:
         leg = ("FP64 Legendre recursion for orders m < %d, double-float (pairs of FP32) above"
                % info["legendre_df32_mmin"])
-    taps = ("double-float interpolation and spreading taps (64-bit integer spreading tiles)"
+    taps = ("double-float interpolation and spreading taps (spreading by register strips)"
             if info["epsilon"] >= 5e-11 and info["point_weight_bytes"] else "FP64 interpolation and spreading taps")
-    return leg + "; FP64 FFTs and kernel weights; " + taps
+    ffts = "double-float synthesis and FP64 adjoint FFTs" if info["legendre_restart"] else "FP64 FFTs"
+    return leg + "; " + ffts + ", FP64 kernel weights; " + taps
 
 
 def kernel_launches(info, prec):
-    """Kernels one synthesis + one adjoint launch on a (non-deterministic) plan: synthesis = coefficient
-    preparation (twice for the restarted FP32 recursion: plain and monic coefficients), Legendre, theta,
-    phi, interpolation; adjoint = the map's largest |value| (fixed-point spreading tiles: FP32 plans at
-    epsilon >= 1e-5, FP64 plans), spreading, phi, theta, Legendre; FP64 plans with FP64 low orders split
-    each Legendre step into two launches (memsets not counted)."""
+    """Most kernels one synthesis + one adjoint launch on a (non-deterministic) plan of this kind: synthesis =
+    coefficient preparation (counted twice for restarted FP32 plans), Legendre, theta, phi, interpolation;
+    adjoint = the map's largest |value| (fixed-point spreading tiles: FP32 plans at epsilon >= 1e-5, FP64 plans),
+    spreading, phi, theta, Legendre; FP64 plans with FP64 low orders split each Legendre step into two
+    launches (memsets not counted)."""
     leg = 2 if (prec == "fp64" and 0 < info["legendre_df32_mmin"] <= info["mmax"]) else 1
     prep = 2 if (prec == "fp32" and info["legendre_restart"] and not info["legendre_table_bytes"]) else 1
     det = bool(info["flags"] & 2)
     maxabs = 1 if (not det and (prec == "fp64" or info["epsilon"] >= 1e-5)) else 0
     return (prep + 3 + leg) + (maxabs + 3 + leg)
+
+
+def plan_launches(info, prec):
+    """kernel_launches less what the plan does without: restarted FP32 plans form the coefficients in the Legendre
+    kernel, and spreading by strips (FP32 plans with W >= 8, spin 0 W >= 10; FP64 plans with double-float
+    weights) needs no bound of the map."""
+    n = kernel_launches(info, prec)
+    det = bool(info["flags"] & 2)
+    if prec == "fp32":
+        if info["legendre_restart"] and not info["legendre_table_bytes"]:
+            n -= 2
+        strip = info["W"] >= (8 if info["spin"] else 10) and info["epsilon"] >= 1e-5
+    else:
+        strip = info["epsilon"] >= 5e-11 and info["point_weight_bytes"] > 0
+    return n - (1 if strip and not det else 0)
 
 
 # ------------------------------------------------------------------ ranks
@@ -457,7 +473,7 @@ def run_gpu(args):
                      "rule": "sum over stages of work / peak of the stage's bound (HBM bytes at %.1f GB/s, %s; "
                              "FP32 FMA flops at the measured %.1f TFLOP/s)" % (peaks["hbm_gbs"], peak_src,
                                                                                peaks["fp32_tflops"])}
-    gpu_launches = (kernel_launches(info_T, "fp32") + kernel_launches(info_P, "fp32")) * args.steps
+    gpu_launches = (plan_launches(info_T, "fp32") + plan_launches(info_P, "fp32")) * args.steps
 
     # ---------------- e2e through the host-buffer entry points (pinned memory)
     e2e = None

@@ -145,7 +145,9 @@ typedef struct {
                                every call; -1 = always evaluate them per call (no weight table);
                                1 = always keep them (LENS_ERR_NOMEM if they do not fit). */
     int spread_tile_rows;   /* rows of the grid tiles that sort the points and that the spreading
-                               accumulates in shared memory (32 columns): 16, 32 or 64 (0 = 32) */
+                               accumulates: 16, 32 or 64 (0 = 32; plans that spread by register
+                               strips, FP32 with W >= 8 (spin 0: 10) and FP64 with double-float weights, take
+                               8 .. 64 by the size of the grid).  32 columns; strips 33 - W */
 } lens_plan_params;
 
 typedef struct {
