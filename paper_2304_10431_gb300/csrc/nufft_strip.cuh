@@ -82,11 +82,12 @@ k_spread_strip(double *__restrict__ grid, const uint32_t *__restrict__ cell, con
     };
     fetch(0);
 
-    // the tile's largest |value| (spin s: Q^2 + U^2) as the bits of a non-negative double
+    // the tile's largest |value| (spin s: |Q| + |U|, whose exponent range is the values' own; squares would lose
+    // maps above 1e154 and below 1e-162) as the bits of a non-negative double
     unsigned long long mx = 0;
     for (uint32_t p = p0 + lane; p < p1; p += 32) {
         const int32_t src = perm[p];
-        const double q = map[src], v = SPIN ? fma(q, q, map[n + src] * map[n + src]) : fabs(q);
+        const double q = fabs(map[src]), v = SPIN ? q + fabs(map[n + src]) : q;
         const unsigned long long b = (unsigned long long)__double_as_longlong(v);
         mx = b > mx ? b : mx;  // infinities and NaNs order above the finite values
     }
@@ -95,8 +96,7 @@ k_spread_strip(double *__restrict__ grid, const uint32_t *__restrict__ cell, con
         const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, off);
         mx = o > mx ? o : mx;
     }
-    double top = __longlong_as_double((long long)mx);
-    if (SPIN) top = sqrt(top);
+    const double top = __longlong_as_double((long long)mx);
     const bool bad = !(top < 1e300);  // infinity or NaN: the tile becomes NaN
     int ex = bad || top == 0.0 ? 0 : -ilogb(top);
     ex = min(max(ex, -1000), 1000);
