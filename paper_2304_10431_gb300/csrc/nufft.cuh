@@ -407,6 +407,11 @@ __global__ void __launch_bounds__(256) k_spread_direct(void *__restrict__ grid, 
 // term is rounded once (to 2^-k; FP64: relative 2^-62 of the tile's bound);
 // the flush converts back for one global atomic per non-zero cell.  A map
 // with a non-finite value makes the whole tile NaN.
+// Where kPassFrom or more points reach one cell, the tile is spread and flushed kPassPoints points at a time: tile_kmax holds
+// at most 65535, and the unit would grow with the pile (FP32, a map of one sign, 300,000 points in one cell: 7e-5 of the
+// a_lm; with the passes 6e-7 at 150,000).  FP32: even skies reach 1024 points only above 20 per cell, where a pass's flush starts to cost.
+template <typename T> constexpr uint32_t kPassFrom = sizeof(T) == 4 ? 1024 : 65535;
+template <typename T> constexpr uint32_t kPassPoints = sizeof(T) == 4 ? 512 : 65535;
 template <typename T, bool FX, bool IT> struct SAcc { using type = typename Acc<T, FX>::type; };
 template <> struct SAcc<float, false, true> { using type = int; };
 template <> struct SAcc<double, false, true> { using type = long long; };
@@ -442,92 +447,100 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
     if (p0 == p1) return;
     T sc = FX ? (T)fxs[0] : T(1);
     bool bad = false;  // IT: non-finite map value
+    uint32_t step = p1 - p0;  // points per pass
     if constexpr (IT) {
         constexpr int kBits = sizeof(T) == 4 ? 30 : 62;  // tile sums of |terms| below 2^kBits
-        const double bound = (double)tile_kmax[t] * __longlong_as_double((long long)*maxbits);
+        const bool pile = tile_kmax[t] >= kPassFrom<T>;
+        const double bound =
+            (double)(pile ? kPassPoints<T> : tile_kmax[t]) * __longlong_as_double((long long)*maxbits);
         if (!(bound < 1e300)) bad = true;  // infinity or NaN in the map
         else if (bound > 0.0) sc = (T)ldexp(1.0, kBits - (ilogb(bound) + 1));  // bound < 2^(ilogb+1)
+        if (pile && !bad) step = kPassPoints<T>;
     }
-    for (int i = threadIdx.x; i < TR * TC * NC; i += blockDim.x) buf[i] = G(0);
-    __syncthreads();
     const int r0 = (t / ntc) * tile_r, c0 = (t % ntc) * kTileC;
-    // (points in sorted order: spin 2, lmax 2048, W = 7: 0.69 ms; a run of points per thread, for fewer of a warp's taps in
-    // one bank, 0.77, runs per group of four threads 0.78: the loads then no longer coalesce)
-    for (uint32_t p = p0 + threadIdx.x; p < (bad ? p0 : p1); p += blockDim.x) {
-        const uint32_t c = cell[p];
-        const int lr = (int)(c / (uint32_t)pitch) - r0, lc = (int)(c % (uint32_t)pitch) - c0;
-        if ((unsigned)lr >= (unsigned)tile_r || (unsigned)lc >= (unsigned)kTileC) continue;  // not this tile's
-        const int32_t src = perm[p];
-        // spin s: two planes (real parts, then imaginary parts), so that the lanes'
-        // atomics of one plane spread over all 32 banks
-        G *b0 = buf + (lr * TC + lc);
-        T wa[W], wb[W];
-        tap_weights<T, W, PRE>(wa, wb, PRE ? cplx<T>{} : frac[p], wts, p, beta, kp);
-        // IT: the power-of-two unit sc is applied to the point's value first (exact)
-        if (!SPIN) {
-            const T x = IT ? map[src] * sc : map[src];
-#pragma unroll
-            for (int a = 0; a < W; ++a) {
-                const T xa = wa[a] * x;
-#pragma unroll
-                for (int b = 0; b < W; ++b) {
-                    if constexpr (IT) tile_add(b0 + a * TC + b, tile_int(xa * wb[b]));
-                    else acc_add<T, FX>(b0 + a * TC + b, xa * wb[b], sc);
+    for (uint32_t pb = p0; pb < p1; pb += step) {
+        const uint32_t pe = min(p1, pb + step);
+        if (pb != p0) __syncthreads();  // the last pass's flush has read the tile
+        for (int i = threadIdx.x; i < TR * TC * NC; i += blockDim.x) buf[i] = G(0);
+        __syncthreads();
+        // (points in sorted order: spin 2, lmax 2048, W = 7: 0.69 ms; a run of points per thread, for fewer of a warp's taps in
+        // one bank, 0.77, runs per group of four threads 0.78: the loads then no longer coalesce)
+        for (uint32_t p = pb + threadIdx.x; p < (bad ? pb : pe); p += blockDim.x) {
+            const uint32_t c = cell[p];
+            const int lr = (int)(c / (uint32_t)pitch) - r0, lc = (int)(c % (uint32_t)pitch) - c0;
+            if ((unsigned)lr >= (unsigned)tile_r || (unsigned)lc >= (unsigned)kTileC) continue;  // not this tile's
+            const int32_t src = perm[p];
+            // spin s: two planes (real parts, then imaginary parts), so that the lanes'
+            // atomics of one plane spread over all 32 banks
+            G *b0 = buf + (lr * TC + lc);
+            T wa[W], wb[W];
+            tap_weights<T, W, PRE>(wa, wb, PRE ? cplx<T>{} : frac[p], wts, p, beta, kp);
+            // IT: the power-of-two unit sc is applied to the point's value first (exact)
+            if (!SPIN) {
+                const T x = IT ? map[src] * sc : map[src];
+    #pragma unroll
+                for (int a = 0; a < W; ++a) {
+                    const T xa = wa[a] * x;
+    #pragma unroll
+                    for (int b = 0; b < W; ++b) {
+                        if constexpr (IT) tile_add(b0 + a * TC + b, tile_int(xa * wb[b]));
+                        else acc_add<T, FX>(b0 + a * TC + b, xa * wb[b], sc);
+                    }
                 }
-            }
-        } else {
-            // e^{-i s chi} (Q + i U)
-            const cplx<T> ph = phase[p];
-            const T q = map[src], u = map[n + src];
-            T zx = ph.x * q + ph.y * u, zy = ph.x * u - ph.y * q;
-            if constexpr (IT) { zx *= sc; zy *= sc; }
-#pragma unroll
-            for (int a = 0; a < W; ++a) {
-                const T xa = wa[a] * zx, ya = wa[a] * zy;
-#pragma unroll
-                for (int b = 0; b < W; ++b) {
-                    G *q2 = b0 + (a * TC + b);
-                    if constexpr (IT) {
-                        tile_add(q2, tile_int(xa * wb[b]));
-                        tile_add(q2 + TR * TC, tile_int(ya * wb[b]));
-                    } else {
-                        acc_add<T, FX>(q2, xa * wb[b], sc);
-                        acc_add<T, FX>(q2 + TR * TC, ya * wb[b], sc);
+            } else {
+                // e^{-i s chi} (Q + i U)
+                const cplx<T> ph = phase[p];
+                const T q = map[src], u = map[n + src];
+                T zx = ph.x * q + ph.y * u, zy = ph.x * u - ph.y * q;
+                if constexpr (IT) { zx *= sc; zy *= sc; }
+    #pragma unroll
+                for (int a = 0; a < W; ++a) {
+                    const T xa = wa[a] * zx, ya = wa[a] * zy;
+    #pragma unroll
+                    for (int b = 0; b < W; ++b) {
+                        G *q2 = b0 + (a * TC + b);
+                        if constexpr (IT) {
+                            tile_add(q2, tile_int(xa * wb[b]));
+                            tile_add(q2 + TR * TC, tile_int(ya * wb[b]));
+                        } else {
+                            acc_add<T, FX>(q2, xa * wb[b], sc);
+                            acc_add<T, FX>(q2 + TR * TC, ya * wb[b], sc);
+                        }
                     }
                 }
             }
         }
-    }
-    __syncthreads();
-    if constexpr (IT) {
-        T *g = (T *)grid;
-        const T inv = bad ? T(NAN) : T(1) / sc;
-        for (int i = threadIdx.x; i < TR * TC; i += blockDim.x) {
-            const int gr = r0 + i / TC, gc = c0 + i % TC;
-            if (gr >= R || gc >= pitch) continue;
-            const int64_t o = (int64_t)gr * pitch + gc;
-            if (!SPIN) {
-                const G v = buf[i];
-                if (v != 0 || bad) atomicAdd(g + o, (T)v * inv);
-            } else {
-                const G vx = buf[i], vy = buf[TR * TC + i];
-                if (vx != 0 || bad) atomicAdd(g + 2 * o, (T)vx * inv);
-                if (vy != 0 || bad) atomicAdd(g + 2 * o + 1, (T)vy * inv);
+        __syncthreads();
+        if constexpr (IT) {
+            T *g = (T *)grid;
+            const T inv = bad ? T(NAN) : T(1) / sc;
+            for (int i = threadIdx.x; i < TR * TC; i += blockDim.x) {
+                const int gr = r0 + i / TC, gc = c0 + i % TC;
+                if (gr >= R || gc >= pitch) continue;
+                const int64_t o = (int64_t)gr * pitch + gc;
+                if (!SPIN) {
+                    const G v = buf[i];
+                    if (v != 0 || bad) atomicAdd(g + o, (T)v * inv);
+                } else {
+                    const G vx = buf[i], vy = buf[TR * TC + i];
+                    if (vx != 0 || bad) atomicAdd(g + 2 * o, (T)vx * inv);
+                    if (vy != 0 || bad) atomicAdd(g + 2 * o + 1, (T)vy * inv);
+                }
             }
-        }
-    } else {
-        G *g = (G *)grid;
-        for (int i = threadIdx.x; i < TR * TC; i += blockDim.x) {
-            const int gr = r0 + i / TC, gc = c0 + i % TC;
-            if (gr >= R || gc >= pitch) continue;
-            const int64_t o = (int64_t)gr * pitch + gc;
-            if (!SPIN) {
-                const G v = buf[i];
-                if (v != G(0)) atomicAdd(g + o, v);
-            } else {
-                const G vx = buf[i], vy = buf[TR * TC + i];
-                if (vx != G(0)) atomicAdd(g + 2 * o, vx);
-                if (vy != G(0)) atomicAdd(g + 2 * o + 1, vy);
+        } else {
+            G *g = (G *)grid;
+            for (int i = threadIdx.x; i < TR * TC; i += blockDim.x) {
+                const int gr = r0 + i / TC, gc = c0 + i % TC;
+                if (gr >= R || gc >= pitch) continue;
+                const int64_t o = (int64_t)gr * pitch + gc;
+                if (!SPIN) {
+                    const G v = buf[i];
+                    if (v != G(0)) atomicAdd(g + o, v);
+                } else {
+                    const G vx = buf[i], vy = buf[TR * TC + i];
+                    if (vx != G(0)) atomicAdd(g + 2 * o, vx);
+                    if (vy != G(0)) atomicAdd(g + 2 * o + 1, vy);
+                }
             }
         }
     }
