@@ -17,10 +17,10 @@ constexpr int kLegBlock = 8;         // degrees per unrolled block of the Legend
 constexpr int kTileR = 32, kTileC = 32;  // default grid tile of the point sort (rows x columns)
 constexpr int kMaxW = 16;                 // largest kernel support
 constexpr int grid_pitch(int columns) { return (columns + 31) / 32 * 32; }  // row length of the grid
-// Double-float kernel weights of a point: the theta taps in pairs (h0, h1, l0, l1), one operand pair of a packed
-// instruction per 8 bytes, then the phi taps (h, l); both padded with zeros to an even count.
+// Double-float kernel weights of a point, 4 W FP32 words: the theta taps in pairs (h0, h1, l0, l1), one operand pair of a
+// packed instruction per 8 bytes (an odd W's last one as (h, l)), then the phi taps (h, l).
 __host__ __device__ constexpr int dd_pairs(int W) { return (W + 1) / 2; }
-__host__ __device__ constexpr int dd_words(int W) { return 8 * dd_pairs(W); }  // FP32 words of one point
+__host__ __device__ constexpr int dd_words(int W) { return 4 * W; }
 
 // FP32 plans: the weight of kernel tap a (0 <= a < W) as a polynomial of degree W + 1 in
 // t = 2 frac - (W - 1), t in [-1, 1] (frac = u - ceil(u - W/2) in (W/2 - 1, W/2]);

@@ -125,17 +125,15 @@ __global__ void k_weights(const double2 *__restrict__ frac, int64_t n, int W, do
     const double2 f = frac[p];
     const double twoW = 2.0 / W;
     if (dd) {  // layout: dd_words
-        const int np = dd_pairs(W);
-        float4 *w = reinterpret_cast<float4 *>(reinterpret_cast<float *>(wts) + p * dd_words(W));
-        for (int i = 0; i < np; ++i) {
-            df32 x[2], y[2];
-            for (int k = 0; k < 2; ++k) {
-                const int a = 2 * i + k;
-                x[k] = df_split(a < W ? es_kernel<double>(f.x - a, twoW, beta) : 0.0);
-                y[k] = df_split(a < W ? es_kernel<double>(f.y - a, twoW, beta) : 0.0);
-            }
-            w[i] = make_float4(x[0].h, x[1].h, x[0].l, x[1].l);
-            w[np + i] = make_float4(y[0].h, y[0].l, y[1].h, y[1].l);
+        float *w = reinterpret_cast<float *>(wts) + p * dd_words(W);
+        for (int a = 0; a < W; ++a) {
+            const df32 x = df_split(es_kernel<double>(f.x - a, twoW, beta));
+            const df32 y = df_split(es_kernel<double>(f.y - a, twoW, beta));
+            const bool lone = (W & 1) && a == W - 1;
+            const int i = lone ? 2 * a : 4 * (a >> 1) + (a & 1);
+            w[i] = x.h;
+            w[i + (lone ? 1 : 2)] = x.l;
+            reinterpret_cast<float2 *>(w + 2 * W)[a] = make_float2(y.h, y.l);
         }
         return;
     }

@@ -89,12 +89,13 @@ template <int W> __device__ __forceinline__ const float *dd_weights(const double
 }
 template <int W> __device__ __forceinline__ df32 dd_theta(const float *w, int a)
 {
+    if ((W & 1) && a == W - 1) return ld_df(reinterpret_cast<const float2 *>(w + 2 * a));
     const float *q = w + 4 * (a >> 1) + (a & 1);
     return {__ldg(q), __ldg(q + 2)};
 }
 template <int W> __device__ __forceinline__ df32 dd_phi(const float *w, int b)
 {
-    return ld_df(reinterpret_cast<const float2 *>(w + 4 * dd_pairs(W)) + b);
+    return ld_df(reinterpret_cast<const float2 *>(w + 2 * W) + b);
 }
 
 // PRE: 0 evaluate the kernel, 1 read the double weights, 2 the double-float pairs
@@ -258,31 +259,35 @@ __global__ void __launch_bounds__(kInterpDD, 4) k_interp_dd(const void *__restri
                                                             const double *__restrict__ wts, double *__restrict__ map,
                                                             int64_t n, int pitch)
 {
-    constexpr int NP = dd_pairs(W), Q = dd_words(W) / 4;  // 16-byte words per point: Q even, rows of Q + 1
-    __shared__ float4 sw[kInterpDD * (Q + 1)];
+    constexpr int NP = dd_pairs(W), Q = dd_words(W) / 4, S = Q | 1;  // 16-byte words per point and per row
+    __shared__ float4 sw[kInterpDD * S];
     const int lane = threadIdx.x & 31;
     const int64_t p = (int64_t)blockIdx.x * kInterpDD + threadIdx.x, p0 = p - lane;
-    float4 *wrow = sw + (threadIdx.x - lane) * (Q + 1);
+    float4 *wrow = sw + (threadIdx.x - lane) * S;
     const int words = (int)min((int64_t)32, n - p0) * Q;
     const float4 *wg = reinterpret_cast<const float4 *>(wts) + p0 * Q;
 #pragma unroll
     for (int k = 0; k < Q; ++k) {
         const int i = k * 32 + lane;
-        if (i < words) wrow[i / Q * (Q + 1) + i % Q] = __ldg(wg + i);
+        if (i < words) wrow[i / Q * S + i % Q] = __ldg(wg + i);
     }
     __syncwarp();
     if (p >= n) return;
     const uint32_t c0 = cell[p];
     const int32_t dst = perm[p];
-    const float4 *w = wrow + lane * (Q + 1);
-    if (!SPIN) {
-        df32 wb[2 * NP];
+    const float4 *w = wrow + lane * S;
+    // phi weights; an odd W's first one shares its 16 bytes with the last theta weight
+    constexpr int O = W & 1;
+    df32 wb[W];
+    const float4 mid = w[W / 2];
+    if (O) wb[0] = {mid.z, mid.w};
 #pragma unroll
-        for (int i = 0; i < NP; ++i) {
-            const float4 v = w[NP + i];
-            wb[2 * i] = {v.x, v.y};
-            wb[2 * i + 1] = {v.z, v.w};
-        }
+    for (int i = 0; i < W / 2; ++i) {
+        const float4 v = w[W / 2 + O + i];
+        wb[2 * i + O] = {v.x, v.y};
+        wb[2 * i + O + 1] = {v.z, v.w};
+    }
+    if (!SPIN) {
         const float2 *g = reinterpret_cast<const float2 *>(grid) + c0;
         D2 acc = {0ull, 0ull};  // rows in pairs; an odd W's last row twice, the second time with weight zero
 #pragma unroll
@@ -294,20 +299,19 @@ __global__ void __launch_bounds__(kInterpDD, 4) k_interp_dd(const void *__restri
                 const float2 x = __ldg(ga + b), y = __ldg(gb + b);
                 r = d2_fma(D2{pk_make(x.x, y.x), pk_make(x.y, y.y)}, D2{pk_make(wb[b].h, wb[b].h), pk_make(wb[b].l, wb[b].l)}, r);
             }
-            const ulonglong2 wa = reinterpret_cast<const ulonglong2 *>(w)[i];
-            acc = d2_fma(d2_norm(r), D2{wa.x, wa.y}, acc);
+            D2 wa;
+            if (2 * i + 1 < W) {
+                const ulonglong2 v = reinterpret_cast<const ulonglong2 *>(w)[i];
+                wa = {v.x, v.y};
+            } else {
+                wa = {pk_make(mid.x, 0.f), pk_make(mid.y, 0.f)};
+            }
+            acc = d2_fma(d2_norm(r), wa, acc);
         }
         const float2 sh = pk_get(acc.h), sl = pk_get(acc.l);
         map[dst] = df_value(df32{sh.x, sl.x}) + df_value(df32{sh.y, sl.y});
     } else {
         // both components in one packed instruction (grid: re h, im h, re l, im l)
-        df32 wb[2 * NP];
-#pragma unroll
-        for (int i = 0; i < NP; ++i) {
-            const float4 v = w[NP + i];
-            wb[2 * i] = {v.x, v.y};
-            wb[2 * i + 1] = {v.z, v.w};
-        }
         const ulonglong2 *g = reinterpret_cast<const ulonglong2 *>(grid) + c0;
         D2 acc = {0ull, 0ull};
 #pragma unroll
@@ -323,7 +327,7 @@ __global__ void __launch_bounds__(kInterpDD, 4) k_interp_dd(const void *__restri
                     const ulonglong2 v = __ldg(g + (int64_t)a * pitch + b);
                     r = d2_fma(D2{v.x, v.y}, D2{pk_make(wb[b].h, wb[b].h), pk_make(wb[b].l, wb[b].l)}, r);
                 }
-                const df32 t = k ? df32{wa.y, wa.w} : df32{wa.x, wa.z};
+                const df32 t = 2 * i + 1 == W ? df32{wa.x, wa.y} : k ? df32{wa.y, wa.w} : df32{wa.x, wa.z};
                 acc = d2_fma(d2_norm(r), D2{pk_make(t.h, t.h), pk_make(t.l, t.l)}, acc);
             }
         }
@@ -409,7 +413,8 @@ __global__ void __launch_bounds__(256) k_spread_direct(void *__restrict__ grid, 
 // with a non-finite value makes the whole tile NaN.
 // Where kPassFrom or more points reach one cell, the tile is spread and flushed kPassPoints points at a time: tile_kmax holds
 // at most 65535, and the unit would grow with the pile (FP32, a map of one sign, 300,000 points in one cell: 7e-5 of the
-// a_lm; with the passes 6e-7 at 150,000).  FP32: even skies reach 1024 points only above 20 per cell, where a pass's flush starts to cost.
+// a_lm; with the passes 6e-7 at 150,000).  FP32: even skies reach 1024 points only above 20 per cell, where the flush of a
+// pass starts to cost.
 template <typename T> constexpr uint32_t kPassFrom = sizeof(T) == 4 ? 1024 : 65535;
 template <typename T> constexpr uint32_t kPassPoints = sizeof(T) == 4 ? 512 : 65535;
 template <typename T, bool FX, bool IT> struct SAcc { using type = typename Acc<T, FX>::type; };

@@ -169,7 +169,7 @@ k_spread_strip(double *__restrict__ grid, const uint32_t *__restrict__ cell, con
         auto column = [&](int q, int o) {
             const int b = lane - (o & 255);
             return o >= 0 && (unsigned)b < (unsigned)W
-                       ? *reinterpret_cast<const float2 *>(wbuf + q * dd_words(W) + 4 * NP + 2 * b)
+                       ? *reinterpret_cast<const float2 *>(wbuf + q * dd_words(W) + 2 * W + 2 * b)
                        : make_float2(0.f, 0.f);
         };
         float2 wb = column(0, so);
@@ -190,9 +190,16 @@ k_spread_strip(double *__restrict__ grid, const uint32_t *__restrict__ cell, con
             while (cur < row) next_row();
 #pragma unroll
             for (int i = 0; i < NP; ++i) {
-                const ulonglong2 wa = *reinterpret_cast<const ulonglong2 *>(w + 4 * i);
+                D2 wa;
+                if (2 * i + 1 < W) {
+                    const ulonglong2 u = *reinterpret_cast<const ulonglong2 *>(w + 4 * i);
+                    wa = {u.x, u.y};
+                } else {
+                    const float2 u = *reinterpret_cast<const float2 *>(w + 4 * i);
+                    wa = {pk_make(u.x, 0.f), pk_make(u.y, 0.f)};
+                }
 #pragma unroll
-                for (int c = 0; c < NC; ++c) S[c][i] = d2_fma(D2{wa.x, wa.y}, v[c], S[c][i]);
+                for (int c = 0; c < NC; ++c) S[c][i] = d2_fma(wa, v[c], S[c][i]);
             }
         }
         // keep the low words below an ulp of the sums (2,000 points in one cell, unnormalised: 2e-12 of the a_lm)

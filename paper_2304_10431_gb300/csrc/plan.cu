@@ -764,8 +764,7 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
                 (e = B.alloc((void **)&p->maxbits, sizeof(unsigned long long), true)) != cudaSuccess)
                 return bailc(e, "alloc spreading bounds");
         }
-        if (keep && (e = B.alloc((void **)&p->wts, dd ? sizeof(float) * (size_t)dd_words(p->W) * npoints : wbytes, false)) !=
-                        cudaSuccess) {
+        if (keep && (e = B.alloc((void **)&p->wts, wbytes, false)) != cudaSuccess) {
             if (e == cudaErrorMemoryAllocation) {
                 cudaGetLastError();
                 return bail(LENS_ERR_NOMEM, "point kernel weights: " + std::to_string(wbytes >> 20) + " MiB not available");
