@@ -147,8 +147,8 @@ struct Plan {
     double *scale = nullptr;
     void *coef = nullptr;     // workspace: forward coefficients c_l a_lm of one call ([ncomp][nalm], float2 /
                               // double2 / df32 float4; restarted FP32 plans form them in the kernel)
-    // FP32 plans, several maps per call: ring coefficients and prepared
-    // coefficients of up to 4 maps, allocated on the first such call
+    // FP32 plans, several maps per call: ring coefficients of up to 4 maps and (plans without restart values) their
+    // prepared coefficients, allocated on the first such call
     void *ring_batch = nullptr, *coef_batch = nullptr;
     bool group_maps = true;  // false: every map runs alone (lens_plan_set_grouping)
     bool grad = false;       // gradient-only spin s plan (C = 0): a_lm holds G alone

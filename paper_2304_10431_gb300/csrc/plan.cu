@@ -1060,9 +1060,9 @@ size_t alm_bytes(const Plan &p) { return plan_alm_bytes(p); }
 size_t map_bytes(const Plan &p) { return (size_t)p.npts * (p.spin ? 2 : 1) * (p.prec == LENS_FP32 ? 4 : 8); }
 size_t ring_bytes(const Plan &p) { return (size_t)p.ncol * p.ntheta * 8; }
 
-// Workspace of the grouped synthesis (FP32 plans): ring and prepared
-// coefficients of four maps, allocated on the first call with two or more
-// maps.  Not inside a stream capture (an allocation there would not be
+// Workspace of the grouped synthesis (FP32 plans): ring coefficients of four maps and, for plans without
+// restart values, their prepared coefficients (the packed kernels form these themselves), allocated on the first call with
+// two or more maps.  Not inside a stream capture (an allocation there would not be
 // replayed): such calls then run map by map.
 bool group_workspace(Plan &p, cudaStream_t st)
 {
@@ -1070,9 +1070,10 @@ bool group_workspace(Plan &p, cudaStream_t st)
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
     if (p.nallocs + 2 > (int)(sizeof(p.allocs) / sizeof(p.allocs[0]))) return false;
+    const size_t cbytes = p.rst ? 0 : 4 * alm_bytes(p);
     void *r = nullptr, *c = nullptr;
     if (cudaMalloc(&r, 4 * ring_bytes(p)) != cudaSuccess) { cudaGetLastError(); return false; }
-    if (cudaMalloc(&c, 4 * alm_bytes(p)) != cudaSuccess) {
+    if (cbytes && cudaMalloc(&c, cbytes) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(r);
         return false;
@@ -1080,8 +1081,8 @@ bool group_workspace(Plan &p, cudaStream_t st)
     p.ring_batch = r;
     p.coef_batch = c;
     p.allocs[p.nallocs++] = r;
-    p.allocs[p.nallocs++] = c;
-    p.work_bytes += 4 * (ring_bytes(p) + alm_bytes(p));
+    if (c) p.allocs[p.nallocs++] = c;
+    p.work_bytes += 4 * ring_bytes(p) + cbytes;
     return true;
 }
 

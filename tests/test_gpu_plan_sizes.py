@@ -19,3 +19,16 @@ def test_point_weight_bytes(w, eps):
     # per point: first cell and index (4 bytes each), offsets (two doubles), weights
     grown = [b - a for a, b in ((info[0][k], info[1][k]) for k in ("plan_bytes", "point_weight_bytes"))]
     assert grown[0] == 24 * 5000 + grown[1] and grown[1] == 16 * w * 5000
+
+
+@pytest.mark.parametrize("restart", [0, -1])
+def test_grouped_synthesis_workspace(restart):
+    """Four maps in one call: four sets of ring coefficients, and of prepared a_lm only where the kernels read them
+    (plans without restart values)."""
+    th, ph, chi = W.random_points(4001, 3)
+    plan = LensPlan(64, th, ph, chi, spin=2, epsilon=1e-5, legendre_restart=restart, device=DEV)
+    before = plan.info()
+    plan.synthesis(torch.zeros(4, 2, plan.nalm, dtype=plan.complex_dtype, device=DEV))
+    rings = 4 * 8 * (2 * 64 + 1) * before["ntheta"]
+    grown = plan.info()["workspace_bytes"] - before["workspace_bytes"]
+    assert grown == rings + (0 if restart == 0 else 4 * 8 * 2 * plan.nalm)
