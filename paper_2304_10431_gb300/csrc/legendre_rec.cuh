@@ -487,13 +487,39 @@ template <class P, int RPT, bool SPIN> struct Rings {
     }
 };
 
-// Rings of the restarted FP32 recursion, plain form: word NW receives the
+// Regime of the next block (see Rings::regime) of restarted spin-0 states
+template <int RPT> __device__ __forceinline__ int restarted_regime(const PolS::St (&sp)[RPT])
+{
+    bool all0 = true, allneg = true;
+#pragma unroll
+    for (int k = 0; k < RPT; ++k) {
+        all0 = all0 && sp[k].E == 0;
+        allneg = allneg && sp[k].E <= kSkipE;
+    }
+    if (__all_sync(0xffffffffu, all0)) return 0;
+    if (__all_sync(0xffffffffu, allneg)) return 1;
+    return 2;
+}
+// restart: state (w[0], w[1]) and exponent E from the table
+template <int RPT>
+__device__ __forceinline__ void restarted_state(PolS::St (&sp)[RPT], const CkTab &ck, int64_t row, int rp0, int nnorth)
+{
+#pragma unroll
+    for (int k = 0; k < RPT; ++k) {
+        const int rp = rp0 + k;
+        if (rp >= nnorth) continue;
+        const float2 v = __ldg((const float2 *)ck.v + row + rp);
+        sp[k].w[0] = v.x; sp[k].w[1] = v.y; sp[k].E = __ldg((const short *)ck.e + row + rp);
+    }
+}
+
+// Rings of the restarted FP32 recursion, spin 0 (the tensor-core synthesis), plain form: word NW receives the
 // newest value (as in the generic Rings), so at a block boundary w[1] holds
 // lambda_{l-1} and w[0] lambda_{l-2}.
-template <int RPT, bool SPIN> struct Rings<PolS, RPT, SPIN> {
+template <int RPT> struct Rings<PolS, RPT, false> {
     using P = PolS;
     float x[RPT];
-    P::St sp[RPT], sm[RPT];
+    P::St sp[RPT];
 
     // ring geometry only (the state comes from a restart)
     __device__ __forceinline__ void init_geom(const RingTab &rt, int rp0, int nnorth)
@@ -502,115 +528,43 @@ template <int RPT, bool SPIN> struct Rings<PolS, RPT, SPIN> {
         for (int k = 0; k < RPT; ++k) {
             x[k] = rp0 + k < nnorth ? __ldg(rt.xdf + rp0 + k).x : 0.f;
             P::zero(sp[k]);
-            P::zero(sm[k]);
         }
     }
     __device__ __forceinline__ void init(const RingTab &rt, int rp0, int nnorth, int m, int s, double lnm)
     {
+        init_geom(rt, rp0, nnorth);
 #pragma unroll
         for (int k = 0; k < RPT; ++k) {
             const int rp = rp0 + k;
-            if (rp < nnorth) {
-                x[k] = __ldg(rt.xdf + rp).x;
-                const double ls = rt.lsin2[rp], lc = rt.lcos2[rp];
-                start_value<P>(sp[k], m, s, s, lnm, ls, lc);
-                if (SPIN) start_value<P>(sm[k], m, s, -s, lnm, ls, lc);
-            } else {
-                x[k] = 0.f;
-                P::zero(sp[k]);
-                P::zero(sm[k]);
-            }
+            if (rp < nnorth) start_value<P>(sp[k], m, s, s, lnm, rt.lsin2[rp], rt.lcos2[rp]);
         }
     }
-    __device__ __forceinline__ int regime() const
+    __device__ __forceinline__ int regime() const { return restarted_regime<RPT>(sp); }
+    template <int NW, bool CHECK> __device__ __forceinline__ void advance(const float4 *reca, const float4 *, int l)
     {
-        bool all0 = true, allneg = true;
+        const float4 c = __ldg(reca + l);  // (A, B, AT, K)
 #pragma unroll
         for (int k = 0; k < RPT; ++k) {
-            all0 = all0 && sp[k].E == 0;
-            allneg = allneg && sp[k].E <= kSkipE;
-            if (SPIN) {
-                all0 = all0 && sm[k].E == 0;
-                allneg = allneg && sm[k].E <= kSkipE;
-            }
+            sp[k].w[NW] = __fmaf_rn(c.x * x[k], sp[k].w[1 - NW], -(c.y * sp[k].w[NW]));
+            if (CHECK) P::rescale(sp[k], NW);
         }
-        if (__all_sync(0xffffffffu, all0)) return 0;
-        if (__all_sync(0xffffffffu, allneg)) return 1;
-        return 2;
-    }
-    template <int NW, bool CHECK>
-    __device__ __forceinline__ void advance(const float4 *reca, const float4 *, int l)
-    {
-        advance_c<NW, CHECK>(__ldg(reca + l));
-    }
-    // one step with the step-table entry c = (A, B, AT, K) of the degree already loaded
-    template <int NW, bool CHECK> __device__ __forceinline__ void advance_c(const float4 c)
-    {
-#pragma unroll
-        for (int k = 0; k < RPT; ++k) {
-            if (!SPIN) {
-                sp[k].w[NW] = __fmaf_rn(c.x * x[k], sp[k].w[1 - NW], -(c.y * sp[k].w[NW]));
-            } else {
-                const float cp = __fmaf_rn(c.x, x[k], c.z), cm = __fmaf_rn(c.x, x[k], -c.z);
-                sp[k].w[NW] = __fmaf_rn(cp, sp[k].w[1 - NW], -(c.y * sp[k].w[NW]));
-                sm[k].w[NW] = __fmaf_rn(cm, sm[k].w[1 - NW], -(c.y * sm[k].w[NW]));
-            }
-            if (CHECK) {
-                P::rescale(sp[k], NW);
-                if (SPIN) P::rescale(sm[k], NW);
-            }
-        }
-    }
-    __device__ __forceinline__ void advance_moved(const float4 *reca, const float4 *rect, int l)
-    {
-#pragma unroll
-        for (int k = 0; k < RPT; ++k) {
-            const float a = sp[k].w[0];
-            sp[k].w[0] = sp[k].w[1];
-            sp[k].w[1] = a;
-            if (SPIN) {
-                const float b = sm[k].w[0];
-                sm[k].w[0] = sm[k].w[1];
-                sm[k].w[1] = b;
-            }
-        }
-        advance<1, true>(reca, rect, l);
     }
     template <int NW, bool SCALED> __device__ __forceinline__ float vplus(int k) const
     {
         return SCALED ? sp[k].w[NW] * P::fac(sp[k].E) : sp[k].w[NW];
     }
-    template <int NW, bool SCALED> __device__ __forceinline__ float vminus(int k) const
-    {
-        return SCALED ? sm[k].w[NW] * P::fac(sm[k].E) : sm[k].w[NW];
-    }
-    // restart: state (w[0], w[1]) and exponent E from the table
     __device__ __forceinline__ void restart(const CkTab &ck, int64_t row, int rp0, int nnorth)
     {
-#pragma unroll
-        for (int k = 0; k < RPT; ++k) {
-            const int rp = rp0 + k;
-            if (rp >= nnorth) continue;
-            if (!SPIN) {
-                const float2 v = __ldg((const float2 *)ck.v + row + rp);
-                sp[k].w[0] = v.x; sp[k].w[1] = v.y; sp[k].E = __ldg((const short *)ck.e + row + rp);
-            } else {
-                const float4 v = __ldg((const float4 *)ck.v + row + rp);
-                const short2 e = __ldg((const short2 *)ck.e + row + rp);
-                sp[k].w[0] = v.x; sp[k].w[1] = v.y; sp[k].E = e.x;
-                sm[k].w[0] = v.z; sm[k].w[1] = v.w; sm[k].E = e.y;
-            }
-        }
+        restarted_state<RPT>(sp, ck, row, rp0, nnorth);
     }
 };
 
-// Rings of the restarted FP32 recursion, Reinsch's form (PolR): w[1] holds
-// the value lambda_l, w[0] the difference D_l = lambda_l - lambda_{l-1};
-// the word index NW of the interface is not used.
-template <int RPT, bool SPIN> struct Rings<PolR, RPT, SPIN> {
+// Reinsch's form (PolR): w[1] holds the value lambda_l, w[0] the difference
+// D_l = lambda_l - lambda_{l-1}; the word index NW of the interface is not used.
+template <int RPT> struct Rings<PolR, RPT, false> {
     using P = PolS;
     float y1[RPT];  // 1 - cos theta
-    P::St sp[RPT], sm[RPT];
+    P::St sp[RPT];
 
     __device__ __forceinline__ void init_geom(const RingTab &rt, int rp0, int nnorth)
     {
@@ -618,98 +572,38 @@ template <int RPT, bool SPIN> struct Rings<PolR, RPT, SPIN> {
         for (int k = 0; k < RPT; ++k) {
             y1[k] = rp0 + k < nnorth ? __ldg(rt.y1 + rp0 + k) : 0.f;
             P::zero(sp[k]);
-            P::zero(sm[k]);
         }
     }
     __device__ __forceinline__ void init(const RingTab &rt, int rp0, int nnorth, int m, int s, double lnm)
     {
+        init_geom(rt, rp0, nnorth);
 #pragma unroll
         for (int k = 0; k < RPT; ++k) {
             const int rp = rp0 + k;
-            if (rp < nnorth) {
-                y1[k] = __ldg(rt.y1 + rp);
-                const double ls = rt.lsin2[rp], lc = rt.lcos2[rp];
-                start_value<P>(sp[k], m, s, s, lnm, ls, lc);
-                sp[k].w[0] = sp[k].w[1];  // D_{l0} = lambda_{l0} (lambda_{l0-1} = 0)
-                if (SPIN) {
-                    start_value<P>(sm[k], m, s, -s, lnm, ls, lc);
-                    sm[k].w[0] = sm[k].w[1];
-                }
-            } else {
-                y1[k] = 0.f;
-                P::zero(sp[k]);
-                P::zero(sm[k]);
-            }
+            if (rp >= nnorth) continue;
+            start_value<P>(sp[k], m, s, s, lnm, rt.lsin2[rp], rt.lcos2[rp]);
+            sp[k].w[0] = sp[k].w[1];  // D_{l0} = lambda_{l0} (lambda_{l0-1} = 0)
         }
     }
-    __device__ __forceinline__ int regime() const
+    __device__ __forceinline__ int regime() const { return restarted_regime<RPT>(sp); }
+    template <int NW, bool CHECK> __device__ __forceinline__ void advance(const float4 *reca, const float4 *, int l)
     {
-        bool all0 = true, allneg = true;
-#pragma unroll
-        for (int k = 0; k < RPT; ++k) {
-            all0 = all0 && sp[k].E == 0;
-            allneg = allneg && sp[k].E <= kSkipE;
-            if (SPIN) {
-                all0 = all0 && sm[k].E == 0;
-                allneg = allneg && sm[k].E <= kSkipE;
-            }
-        }
-        if (__all_sync(0xffffffffu, all0)) return 0;
-        if (__all_sync(0xffffffffu, allneg)) return 1;
-        return 2;
-    }
-    template <int NW, bool CHECK>
-    __device__ __forceinline__ void advance(const float4 *reca, const float4 *, int l)
-    {
-        advance_c<NW, CHECK>(__ldg(reca + l));
-    }
-    template <int NW, bool CHECK> __device__ __forceinline__ void advance_c(const float4 c)
-    {
+        const float4 c = __ldg(reca + l);  // (A, B, AT, K)
 #pragma unroll
         for (int k = 0; k < RPT; ++k) {
             const float dp = __fmaf_rn(c.x, y1[k], c.w);
             sp[k].w[0] = __fmaf_rn(c.y, sp[k].w[0], -(dp * sp[k].w[1]));
             sp[k].w[1] = __fadd_rn(sp[k].w[1], sp[k].w[0]);
-            if (SPIN) {
-                const float dm = __fmaf_rn(c.x, y1[k], __fmaf_rn(2.f, c.z, c.w));
-                sm[k].w[0] = __fmaf_rn(c.y, sm[k].w[0], -(dm * sm[k].w[1]));
-                sm[k].w[1] = __fadd_rn(sm[k].w[1], sm[k].w[0]);
-            }
-            if (CHECK) {
-                P::rescale(sp[k], 1);
-                if (SPIN) P::rescale(sm[k], 1);
-            }
+            if (CHECK) P::rescale(sp[k], 1);
         }
-    }
-    __device__ __forceinline__ void advance_moved(const float4 *reca, const float4 *rect, int l)
-    {
-        advance<1, true>(reca, rect, l);
     }
     template <int NW, bool SCALED> __device__ __forceinline__ float vplus(int k) const
     {
         return SCALED ? sp[k].w[1] * P::fac(sp[k].E) : sp[k].w[1];
     }
-    template <int NW, bool SCALED> __device__ __forceinline__ float vminus(int k) const
-    {
-        return SCALED ? sm[k].w[1] * P::fac(sm[k].E) : sm[k].w[1];
-    }
-    // restart: state (w[0], w[1]) and exponent E from the table
     __device__ __forceinline__ void restart(const CkTab &ck, int64_t row, int rp0, int nnorth)
     {
-#pragma unroll
-        for (int k = 0; k < RPT; ++k) {
-            const int rp = rp0 + k;
-            if (rp >= nnorth) continue;
-            if (!SPIN) {
-                const float2 v = __ldg((const float2 *)ck.v + row + rp);
-                sp[k].w[0] = v.x; sp[k].w[1] = v.y; sp[k].E = __ldg((const short *)ck.e + row + rp);
-            } else {
-                const float4 v = __ldg((const float4 *)ck.v + row + rp);
-                const short2 e = __ldg((const short2 *)ck.e + row + rp);
-                sp[k].w[0] = v.x; sp[k].w[1] = v.y; sp[k].E = e.x;
-                sm[k].w[0] = v.z; sm[k].w[1] = v.w; sm[k].E = e.y;
-            }
-        }
+        restarted_state<RPT>(sp, ck, row, rp0, nnorth);
     }
 };
 
