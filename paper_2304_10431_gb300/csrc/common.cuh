@@ -109,6 +109,17 @@ __device__ __forceinline__ df32 df_renorm(df32 a)
     return {h, __fadd_rn(__fsub_rn(a.h, __fsub_rn(h, bb)), __fsub_rn(a.l, bb))};
 }
 
+// a b + c: the two-sum of c and the product, whose own error joins the remainder in one fma (see d2_fma, pk.cuh)
+__device__ __forceinline__ df32 df_fma(df32 a, df32 b, df32 c)
+{
+    const float s = __fadd_rn(c.h, __fmul_rn(a.h, b.h));
+    const float bb = __fsub_rn(s, c.h);
+    const float ec = __fsub_rn(c.h, __fsub_rn(s, bb));
+    const float ep = __fmaf_rn(a.h, b.h, -bb);
+    const float lo = __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, c.l));
+    return {s, __fadd_rn(lo, __fadd_rn(ec, ep))};
+}
+
 // Fixed-point accumulation (deterministic plans): a sum whose terms are
 // bounded by `bound` in total is accumulated as integers in units of 2^-k,
 // with k the largest integer up to 122 such that bound 2^k <= 2^62 (so the

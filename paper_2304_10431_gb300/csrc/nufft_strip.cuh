@@ -53,7 +53,8 @@ k_spread_strip(double *__restrict__ grid, const uint32_t *__restrict__ cell, con
                int64_t n, int pitch, int R, int ntc, int ntiles, const uint32_t *__restrict__ tile_start, int tile_r,
                uint32_t part, unsigned *__restrict__ status)
 {
-    constexpr int NP = dd_pairs(W), NC = SPIN ? 2 : 1, TC = 33 - W;
+    constexpr int NP = W / 2, NC = SPIN ? 2 : 1, TC = 33 - W;  // row pairs; an odd W's last row by itself
+    constexpr bool ODD = W & 1;
     constexpr uint32_t WBYTES = dd_words(W) * sizeof(float);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int t = blockIdx.x * kStripWarps + wid;
@@ -104,10 +105,13 @@ k_spread_strip(double *__restrict__ grid, const uint32_t *__restrict__ cell, con
 
     const int r0 = (t / ntc) * tile_r, c0 = (t % ntc) * TC;
     D2 S[NC][NP];
+    df32 last[NC];
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
+    for (int c = 0; c < NC; ++c) {
+        last[c] = {0.f, 0.f};
 #pragma unroll
         for (int i = 0; i < NP; ++i) S[c][i] = {0ull, 0ull};
+    }
     int cur = 0;  // tile row of the window's first row
     const int gc = c0 + lane;
     auto next_row = [&]() {  // add the window's first row into the grid, move down
@@ -125,12 +129,14 @@ k_spread_strip(double *__restrict__ grid, const uint32_t *__restrict__ cell, con
             for (int c = 0; c < NC; ++c) atomicAdd(g + c, df_value(v[c]) * inv);
         }
 #pragma unroll
-        for (int c = 0; c < NC; ++c)
+        for (int c = 0; c < NC; ++c) {
 #pragma unroll
             for (int i = 0; i < NP; ++i) {
-                S[c][i].h = pk_make(pk_get(S[c][i].h).y, i + 1 < NP ? pk_get(S[c][i + 1 < NP ? i + 1 : i].h).x : 0.f);
-                S[c][i].l = pk_make(pk_get(S[c][i].l).y, i + 1 < NP ? pk_get(S[c][i + 1 < NP ? i + 1 : i].l).x : 0.f);
+                S[c][i].h = pk_make(pk_get(S[c][i].h).y, i + 1 < NP ? pk_get(S[c][i + 1 < NP ? i + 1 : i].h).x : last[c].h);
+                S[c][i].l = pk_make(pk_get(S[c][i].l).y, i + 1 < NP ? pk_get(S[c][i + 1 < NP ? i + 1 : i].l).x : last[c].l);
             }
+            last[c] = {0.f, 0.f};
+        }
         ++cur;
     };
 
@@ -178,10 +184,11 @@ k_spread_strip(double *__restrict__ grid, const uint32_t *__restrict__ cell, con
             const float *w = wbuf + q * dd_words(W);
             const int row = so >> 8;  // (-1 for a point of no tile: no row to move to, weights zero)
             D2 v[NC];
+            df32 t[NC];
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
-                const df32 t = df_mul(df32{wb.x, wb.y}, c == 0 ? df32{xv.x, xv.y} : df32{xv.z, xv.w});
-                v[c] = {pk_make(t.h, t.h), pk_make(t.l, t.l)};
+                t[c] = df_mul(df32{wb.x, wb.y}, c == 0 ? df32{xv.x, xv.y} : df32{xv.z, xv.w});
+                v[c] = {pk_make(t[c].h, t[c].h), pk_make(t[c].l, t[c].l)};
             }
             const int qn = min(q + 1, cnt - 1);
             so = soff[qn];
@@ -190,28 +197,28 @@ k_spread_strip(double *__restrict__ grid, const uint32_t *__restrict__ cell, con
             while (cur < row) next_row();
 #pragma unroll
             for (int i = 0; i < NP; ++i) {
-                D2 wa;
-                if (2 * i + 1 < W) {
-                    const ulonglong2 u = *reinterpret_cast<const ulonglong2 *>(w + 4 * i);
-                    wa = {u.x, u.y};
-                } else {
-                    const float2 u = *reinterpret_cast<const float2 *>(w + 4 * i);
-                    wa = {pk_make(u.x, 0.f), pk_make(u.y, 0.f)};
-                }
+                const ulonglong2 wa = *reinterpret_cast<const ulonglong2 *>(w + 4 * i);
 #pragma unroll
-                for (int c = 0; c < NC; ++c) S[c][i] = d2_fma(wa, v[c], S[c][i]);
+                for (int c = 0; c < NC; ++c) S[c][i] = d2_fma(D2{wa.x, wa.y}, v[c], S[c][i]);
+            }
+            if constexpr (ODD) {
+                const float2 wa = *reinterpret_cast<const float2 *>(w + 4 * NP);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) last[c] = df_fma(df32{wa.x, wa.y}, t[c], last[c]);
             }
         }
         // keep the low words below an ulp of the sums (2,000 points in one cell, unnormalised: 2e-12 of the a_lm)
 #pragma unroll
-        for (int c = 0; c < NC; ++c)
+        for (int c = 0; c < NC; ++c) {
 #pragma unroll
             for (int i = 0; i < NP; ++i) S[c][i] = d2_norm(S[c][i]);
+            if constexpr (ODD) last[c] = df_renorm(last[c]);
+        }
         __syncwarp();  // the buffers are rewritten by the next batch
     }
     if (!ok && lane == 0) atomicOr(status, FLAG_TIMEOUT);
-    const int last = min(tile_r + W - 1, bad ? 1 << 20 : cur + W);  // rows the last points reach
-    while (cur < last) next_row();
+    const int end = min(tile_r + W - 1, bad ? 1 << 20 : cur + W);  // rows the last points reach
+    while (cur < end) next_row();
 }
 
 // FP32 plans with W >= 8 (spin 0: W >= 10; or epsilon < 1e-5): the same sweep with FP32 sums.  Each lane evaluates the 2W polynomial weights
