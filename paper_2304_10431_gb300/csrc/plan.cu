@@ -225,6 +225,16 @@ struct Builder {
         if (e != cudaSuccess) return e;
         return cudaMemcpy(*ptr, v.data(), v.size() * sizeof(V), cudaMemcpyHostToDevice);
     }
+    // e^{-2 pi i k / n}, k = 0 .. n - 1; kept for the next transform of the same length
+    const std::vector<double2> &unit_roots(int n)
+    {
+        if ((int)roots.size() != n) {
+            roots.resize(n);
+            for (int k = 0; k < n; ++k) roots[k] = make_double2(cos(2 * kPi * k / n), -sin(2 * kPi * k / n));
+        }
+        return roots;
+    }
+    std::vector<double2> roots;
     cudaError_t fft(FftDesc &d, int n, bool dd)
     {
         d.n = n;
@@ -247,21 +257,20 @@ struct Builder {
         if (e != cudaSuccess) return e;
         d.perm = (const int *)dp;
         void *tw = nullptr;
+        const std::vector<double2> &r = unit_roots(n);
         if (p.prec == LENS_FP32) {
             std::vector<float2> t(n);
-            for (int i = 0; i < n; ++i) t[i] = make_float2((float)cos(2 * kPi * i / n), (float)-sin(2 * kPi * i / n));
+            for (int i = 0; i < n; ++i) t[i] = make_float2((float)r[i].x, (float)r[i].y);
             e = upload(&tw, t);
         } else if (dd) {
             std::vector<float4> t(n);
             for (int i = 0; i < n; ++i) {
-                const dfl c(cos(2 * kPi * i / n)), s(-sin(2 * kPi * i / n));
+                const dfl c(r[i].x), s(r[i].y);
                 t[i] = make_float4(c.h, c.l, s.h, s.l);
             }
             e = upload(&tw, t);
         } else {
-            std::vector<double2> t(n);
-            for (int i = 0; i < n; ++i) t[i] = make_double2(cos(2 * kPi * i / n), -sin(2 * kPi * i / n));
-            e = upload(&tw, t);
+            e = upload(&tw, r);
         }
         d.tw = tw;
         return e;
@@ -872,12 +881,10 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
             if ((e = B.upload(&p->w2d, f2)) != cudaSuccess) return bailc(e, "upload w2");
         }
     }
-    if ((e = B.fft(p->fM, p->M, false)) != cudaSuccess || (e = B.fft(p->fN1, p->N1, false)) != cudaSuccess ||
-        (e = B.fft(p->fN2, p->N2, false)) != cudaSuccess)
-        return bailc(e, "fft tables");
-    if (p->fft_dd && ((e = B.fft(p->dM, p->M, true)) != cudaSuccess || (e = B.fft(p->dN1, p->N1, true)) != cudaSuccess ||
-                      (e = B.fft(p->dN2, p->N2, true)) != cudaSuccess))
-        return bailc(e, "fft tables");
+    const struct { FftDesc &f, &d; int n; } ffts[] = {{p->fM, p->dM, p->M}, {p->fN1, p->dN1, p->N1}, {p->fN2, p->dN2, p->N2}};
+    for (const auto &t : ffts)
+        if ((e = B.fft(t.f, t.n, false)) != cudaSuccess || (p->fft_dd && (e = B.fft(t.d, t.n, true)) != cudaSuccess))
+            return bailc(e, "fft tables");
 
     if ((e = launch_rec_tables(*p)) != cudaSuccess) return bailc(e, "recursion tables");
     if (p->rst) {  // (FP32: step table, then) restart values from the FP64 recursion
