@@ -79,6 +79,8 @@ def parse():
                     help="batched T synthesis with the tensor-core Legendre step: comma list of map counts "
                          "('' to skip)")
     ap.add_argument("--no-e2e", action="store_true")
+    ap.add_argument("--details", default=None, metavar="FILE",
+                    help="also write everything measured (stage tables of every leg, arithmetic, plans) as JSON")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--cpu-seconds", type=float, default=15.0)
     ap.add_argument("--ref-seconds", type=float, default=150.0,
@@ -681,9 +683,44 @@ def run_gpu(args):
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         result["cpu_baseline"] = cpu_baseline(lmax, nside, args.cpu_seconds)
     if rank == 0:
-        print(json.dumps(result), flush=True)
+        if args.details:
+            with open(args.details, "w") as f:
+                json.dump(result, f, indent=1)
+        print(json.dumps(compact(result)), flush=True)
     if world > 1:
         dist.destroy_process_group()
+
+
+def compact(result):
+    """The printed line: the headline as it is, of the other legs their times (the whole record, about 20 kB, is longer
+    than what keeps the output of a run may hold)."""
+    def pick(d, *keys):
+        return None if d is None else {k: d[k] for k in keys if k in d}
+
+    out = {k: v for k, v in result.items() if k not in ("stages", "measured_peaks", "tables", "recursion", "tensor_cores",
+                                                        "fp64", "lmax5120", "cpu_baseline")}
+    cfg = dict(result["config"], legendre={k: pick(v, "mode", "restart_every", "bytes") if isinstance(v, dict) else v
+                                           for k, v in result["config"]["legendre"].items()})
+    for k in ("plan_T", "plan_EB"):
+        cfg[k] = pick(cfg[k], "n1", "W", "sigma")
+    out["config"] = cfg
+    out["roofline"] = pick(result["roofline"], "bound", "achieved", "peak", "unit", "frac", "traffic", "kernel",
+                           "avg_launch_ms")
+    out["step_roofline"] = pick(result["step_roofline"], "t_roof_ms", "frac")
+    out["e2e"] = pick(result["e2e"], "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step", "ms_min",
+                      "ms_max")
+    out["stages_ms_frac"] = {"%s/%d" % (r["stage"], r["spin"]): [r["ms_per_step"], r["frac"]] for r in result["stages"]}
+    leg = ("value", "epsilon", "ms_per_step", "unavailable")
+    for k in ("tables", "recursion", "fp64"):
+        if result.get(k) is not None:
+            out[k] = pick(result[k], *leg)
+    if result.get("tensor_cores"):
+        out["tensor_cores_call_ms"] = {str(r["maps"]): [r["tensor_cores"]["call_ms"], r["cuda_cores"]["call_ms"]]
+                                       for r in result["tensor_cores"]["legs"]}
+    if result.get("lmax5120"):
+        out["lmax5120_ms"] = [[r["precision"], r["epsilon"], r["ms_per_step"]] for r in result["lmax5120"]["legs"]]
+    out["cpu_baseline"] = pick(result.get("cpu_baseline"), "value", "unit", "cores", "kind", "seconds_per_step")
+    return out
 
 
 # ------------------------------------------------------------------ CPU oracle
