@@ -347,11 +347,12 @@ cudaError_t launch_prep_points(Plan &p, const double *theta, const double *phi, 
     };
     const int ntc = p.ntile_c;
     const uint64_t nkeys = (uint64_t)((p.R + p.tile_r - 1) / p.tile_r) * ntc;
-    // Sorted within a tile by row where spreading is by strips, which need it, and by row and column from 2^20 points on, for the
-    // interpolation, where the keys fit 32 bits.  Fewer points gain nothing from it (lmax 128 to 512, spin 0 and 2:
-    // interpolation within 1 us), and the longer keys cost plan creation (lmax 128: 1.28 -> 1.44 ms)
+    // Sorted within a tile by row where spreading is by strips, which need it, and by row and column for the interpolation
+    // of many points, where the keys fit 32 bits.  Fewer points gain nothing from it (W 7, spin 0 and 2, lmax 128 to 512:
+    // interpolation within 1 us; from W 8 on it shows at 786,000 points: W 9 22.9 -> 21.2 us), and the longer keys cost plan
+    // creation (lmax 128: 1.28 -> 1.44 ms)
     const bool fit = nkeys * p.tile_r * p.tile_c <= 0xffffffffull;
-    const int rows = fit && (p.strip || n >= (1 << 20)) ? 2 : p.strip ? 1 : 0;
+    const int rows = fit && (p.strip || n >= (p.W <= 7 ? 1 << 20 : 1 << 17)) ? 2 : p.strip ? 1 : 0;
     const int per = rows == 2 ? p.tile_r * p.tile_c : rows ? p.tile_r : 1;
     k_prep<<<blocks, thr, 0, st>>>(theta, phi, chi, n, p.N1, p.N2, p.W, p.r_lo, p.R, p.pitch, p.spin, scale_of(p.N1),
                                    scale_of(p.N2), p.tile_r, p.tile_c, rows, key, idx, cell_u, frac_u, phase_u, p.flags);
