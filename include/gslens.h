@@ -168,7 +168,7 @@ typedef struct {
     size_t legendre_table_bytes; /* Legendre tables held by the plan (0: recursion) */
     int legendre_restart;        /* recursion restarted every this many degrees (FP32 plans: FP32
                                     recursion, FP64 plans: double-float; 0: no restarts, or tables) */
-    size_t restart_bytes;        /* restart values held by the plan */
+    size_t restart_bytes;        /* restart values held by the plan (without the start values, one row per order) */
     int legendre_df32_mmin;      /* FP64 plans: first order run in double-float (mmax + 1: none) */
     int64_t legendre_triples;    /* restarted recursions: (ring pair, l, m) triples from the first
                                     degree at which |lambda| reaches 2^-40 (FP64 plans: 2^-64) on each

@@ -1,7 +1,8 @@
 // Double-float real numbers with operators, and complex numbers of them: the synthesis transforms of fft.cuh and
 // torus.cu run with T = dfl in FP64 plans with restart values, where FP64 butterflies waited for GB300's FP64 pipe
-// (1/60 of the FP32 rate).  lmax 2048, spin 2: theta 2.68 -> 0.74 ms, phi 2.45 -> 0.66 ms; the error of a synthesis against
-// 64-bit sums is unchanged (4.3e-12 at epsilon 6e-11, lmax 256).  Operations are those of common.cuh's df32 (sums by
+// (1/60 of the FP32 rate), as long as the plan's truncation error hides their rounding (plan.cu: not with W = 16 on small
+// grids).  lmax 2048, spin 2: theta 2.68 -> 0.65 ms, phi 2.45 -> 0.60 ms; the error of a synthesis against
+// 64-bit sums is unchanged (epsilon 1e-10, lmax 512 to 4096: within 0.05%).  Operations are those of common.cuh's df32 (sums by
 // two-sum, ~2^-46 relative; not renormalised); factors of +-1 and 1/2 are plain floats.  Not for the adjoint: there the
 // deconvolution comes last and amplifies the transforms' rounding noise (5e-13 of the a_lm).
 #pragma once

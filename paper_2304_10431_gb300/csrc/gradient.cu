@@ -104,7 +104,8 @@ template <int K> __device__ __forceinline__ double small_angle(double a2)
 // dL/dalpha per point (FP64 arithmetic; inputs in the lensed plans' type T):
 // alpha [2][n], g / p [ncomp][n], A / B [2][n]; out [2][n] (theta, phi parts).
 // Bound by the FP64 pipe.  Deflections up to half a radian take J and the holonomy as power series in a^2, without
-// roots, divisions, sines and cosines; a gradient step of E/B at lmax 1024, 3.1M points: 6.46 -> 6.04 ms with it.
+// roots, divisions, sines and cosines; map and both gradients of E/B at lmax 1024, 3.1M points, on a model that has its
+// potential: 6.46 -> 6.04 ms with it (a new potential also sorts its points and builds its plans: 59 ms).
 template <typename T>
 __global__ void k_deflection_vjp(int64_t n, int spin, const double *__restrict__ alpha, const T *__restrict__ g,
                                  const T *__restrict__ p, const T *__restrict__ A, const T *__restrict__ B,

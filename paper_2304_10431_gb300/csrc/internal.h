@@ -180,8 +180,8 @@ struct Plan {
     void *w1 = nullptr;       // [2 lmax + 1]  1/psihat(2 pi k / N1), k = -lmax..lmax
     void *w2 = nullptr;       // [ncol]        1/(M psihat(2 pi m / N2))
     FftDesc fM, fN1, fN2;
-    // FP64 plans with restart values: the synthesis transforms in double-float (dfl.cuh), with their own descriptors and
-    // deconvolution factors; ring coefficients and torus rows of a synthesis are then double-float pairs.  The adjoint's
+    // FP64 plans with restart values and a truncation error that hides the rounding: the synthesis transforms in double-float
+    // (dfl.cuh), with their own descriptors and deconvolution factors; ring coefficients and torus rows of a synthesis are then double-float pairs.  The adjoint's
     // stay in FP64: deconvolution amplifies their rounding noise (5e-13 of the a_lm in double-float)
     bool fft_dd = false;
     FftDesc dM, dN1, dN2;
@@ -200,7 +200,7 @@ struct Plan {
     uint32_t strip_part = 0;         // points of a tile that one warp sweeps, and the most such parts of a tile
     int strip_parts = 1;
     double *wts = nullptr;     // FP64 plans: [npts][2W] kernel weights (theta taps, then phi taps)
-    bool wts_dd = false;       // weights as double-float pairs (layout: dd_words, nufft.cuh); double-float
+    bool wts_dd = false;       // weights as double-float pairs (layout: dd_words); double-float
                                // interpolation and spreading taps (FP64 plans with epsilon >= 5e-11)
 
     // per-call workspace

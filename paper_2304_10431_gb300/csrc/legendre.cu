@@ -1578,7 +1578,7 @@ Plan::LegShape legendre_shape(const Plan &p, bool adjoint, bool dd, int rpt, int
                                            : kernel_of<PolF64>(p.spin != 0, p.grad, rpt, adjoint);
     const int nw = (p.nnorth + 32 * rpt - 1) / (32 * rpt);
     Plan::LegShape best;
-    if (p.rst && (p.prec == LENS_FP32 || dd)) {  // legendre_pk.cu packs its own CTAs
+    if (p.rst && (p.prec == LENS_FP32 || dd)) {  // legendre_pk.cuh packs its own CTAs
         best.rpt = rpt;
         return best;
     }

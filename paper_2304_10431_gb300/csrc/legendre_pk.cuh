@@ -28,8 +28,8 @@
 // which rescales every four degrees (four steps grow a value by at most 2^34).
 //
 // Time per launch at lmax 4096, before (scalar instructions, coefficient pass, rings per thread adjacent) and
-// after, ms: FP32 spin 0 synthesis 4.35 -> 3.0, adjoint 5.26 -> 4.8; spin 2 11.4 -> 7.5, 13.6 -> 9.8; FP64 spin 0
-// 19.2 -> 16.5, 27.0 -> 22.1; spin 2 63.6 -> 51.3, 100.7 -> 70.4.  The loops are bound by register operands
+// after, ms: FP32 spin 0 synthesis 4.35 -> 3.0, adjoint 5.26 -> 4.6; spin 2 11.4 -> 7.6, 13.6 -> 10.1; FP64 spin 0
+// 19.2 -> 16.3, 27.0 -> 21.8; spin 2 63.6 -> 51.3, 100.7 -> 70.4.  The loops are bound by register operands
 // (FP32: the FMA pipe is busy 63% of the cycles against 67% with three operand reads each) and, in double-float, by the
 // FMA pipe.  Tried and not kept: skipping the 32-ring groups of a warp that are still evanescent
 // (8-16% fewer ring-degrees, but a second copy of the block: spin 2 7.5 -> 7.9 ms).

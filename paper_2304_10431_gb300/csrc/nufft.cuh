@@ -12,15 +12,15 @@
 // Points are prepared once per plan (Sect. 4: the geometry is reused): cell
 // offset into the row-padded grid, fractional offsets (u - i0, v - j0) from
 // FP64 coordinates, the spin phase e^{i s chi}, a permutation that sorts
-// points by grid tile (of the first tap), within a tile by cell row and column, so that neighbouring
-// threads share grid rows and cells, and the first sorted point of every tile.
+// points by grid tile (of the first tap), within a tile by cell row and column where that pays (launch_prep_points), so that
+// neighbouring threads share grid rows and cells, and the first sorted point of every tile.
 // Interpolation runs one thread per sorted point and reads its taps
 // through L1: sorted neighbours share rows, so the tile stays cached (staging
 // the tile and its halo in shared memory first measured 1.36x slower for
 // spin 0 at lmax 4096).  Sorted by row and column, and by aligned pairs (k_interp32): lmax 4096, 50M points, FP32, spin 0
 // 1.17 -> 0.77 ms, spin 2 2.08 -> 1.56 ms.
-// Spreading: FP64 plans with double-float weights and FP32 plans with W >= 8 by strips in registers (nufft_strip.cuh); the
-// others one CTA per 32 x 32 tile: its points add their W x W taps into the tile and its halo, (32 + W - 1) x (32 + W - 1)
+// Spreading: FP64 plans with double-float weights and FP32 plans with W >= 8 (spin 0: W >= 10) or epsilon < 1e-5 by strips in
+// registers (nufft_strip.cuh); the others one CTA per 32 x 32 tile: its points add their W x W taps into the tile and its halo, (32 + W - 1) x (32 + W - 1)
 // integers held in shared memory, and the CTA then adds the non-zero cells into the grid with one global atomic each.
 //
 // Deterministic plans (LENS_DETERMINISTIC) spread in 64-bit fixed point: every

@@ -6,9 +6,9 @@
 // (f32x2 instructions).  The points are sorted by cell row (plan creation); after the points of a
 // row, its grid row receives nothing more from this tile: the lane adds it into the grid with one atomic and
 // the window moves down a row.  No shared-memory accumulation: the tiles of 64-bit integers that this replaces
-// were bound by shared-memory atomics (1.1 taps per clock and SM; 24.2 ms for spin 0 and 42 ms for spin 2
-// at lmax 4096, 50M points, W = 13).  A point costs the whole warp W/2 multiply-adds of a pair, whatever part
-// of the 32 columns it covers (W = 13: 41%).
+// were bound by shared-memory atomics (1.1 taps per clock and SM; lmax 4096, 50M points, W = 13: spin 0 24.2 ms, spin 2
+// 45.7, now 9.6 and 17.0).  A point costs the whole warp W/2 multiply-adds of a pair (an odd W's last row is scalar: half
+// of one), whatever part of the 32 columns it covers (W = 13: 41%).
 //
 // Sums are double-float (d2_fma, ~2^-47 of the partial sums), of values scaled by the power of two that brings the
 // tile's largest one near 1.  Tried and not kept: high words offset by a bound of the cell's sum, where a term takes 6
@@ -223,10 +223,11 @@ k_spread_strip(double *__restrict__ grid, const uint32_t *__restrict__ cell, con
 
 // FP32 plans with W >= 8 (spin 0: W >= 10; or epsilon < 1e-5): the same sweep with FP32 sums.  Each lane evaluates the 2W polynomial weights
 // of one point of a batch of 32 into shared memory (the coefficients come from the constant bank); then the warp
-// takes the points in turn.  Bound by issue: ~50 instructions per point whatever W, where the tiles of 32-bit
-// integers in shared memory (nufft.cuh) cost W^2 atomics: spin 2, lmax 4096, 50M points, W = 8: 3.07 -> 2.66 ms; W = 7: lmax 2048 0.66
-// against 0.69 ms, lmax 1024 0.17 against 0.22, so W <= 7 keeps the tiles; spin 0, whose tiles do half the atomics, up to W = 9
-// (lmax 4096, W = 8: tiles 1.65 ms, strips 1.85; lmax 2048, W = 10: 0.588, 0.554).  Two tiles of 17 - W columns per warp, one per half,
+// takes the points in turn.  Bound by issue: for both components of spin s about 50 instructions a point at W = 8 and 60 at
+// W = 10, where the tiles of 32-bit integers in shared memory (nufft.cuh) cost 2 W^2 atomics.  The rule stands in plan.cu
+// with both sides measured (spin 2, lmax 4096, 50M points, W = 8: tiles 3.34 ms, strips 2.66).  Sums of up to 4096 points of a
+// warp (more in piles above 262,144 points) are plain FP32: 1e-6 of the a_lm for 300,000 points in one cell (integer tiles
+// in one pass: 5e-5 to 4e-4).  Two tiles of 17 - W columns per warp, one per half,
 // were tried for the lanes a point leaves idle: 2.83 ms, and the narrow tiles cost the interpolation 0.2-0.4 ms.
 template <int W> __host__ __device__ constexpr size_t strip32_warp_smem()
 {

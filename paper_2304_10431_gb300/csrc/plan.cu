@@ -478,6 +478,9 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
         sizes_for(lmax, mmax, p->M, sg, W, N1, N2);
         const size_t lim = force_cl ? force_cl * fft_one : fft_max;
         if ((size_t)N1 > lim || (size_t)N2 > lim) continue;
+        // The weights below are those of the kernels of their measurements: one thread per point with float tiles (FP32,
+        // epsilon < 1e-5) or 32-bit tiles, native FP64 FFTs.  They have not been refitted to strips (a point costs W/2 steps),
+        // double-float synthesis transforms (3.5 times cheaper a cell) and interpolation by pairs.
         // per-point taps (+ kernel evaluations in FP32 plans; FP64 plans keep the
         // weights) against grid passes (FFTs).  Grid weight per cell, in taps, from
         // the stage times at lmax 4096: ~12 in FP32, ~60 in FP64 (FP64 butterflies
@@ -749,11 +752,19 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
         // spreading taps in double-float on the FP32 pipe (~2^-46 relative per term; lmax 4096,
         // 50M points, W = 13: interpolation 30.1 -> 13.4 ms for spin 2); smaller epsilon keeps FP64
         const bool dd = keep && epsilon >= 5e-11;
-        // spreading by strips (nufft_strip.cuh; FP32 plans by tiles of 32-bit integers where those are faster: a strip
-        // point costs ~50 instructions whatever W and for both components, a tile W^2 atomics for each; us at lmax
-        // 2048, 12.6M points, tiles / strips: spin 2 W 7 681 / 672, W 8 827 / 685, W 10 1177 / 810; spin 0 W 8 413 / 479, W 9
-        // 496 / 525, W 10 588 / 554, and the interpolation is 1-8% slower on the narrower tiles of strips): fewer
-        // rows per tile where the tiles would not fill the chip
+        // Spreading by strips (nufft_strip.cuh), except FP32 plans at epsilon >= 1e-5 with few taps, which keep tiles of 32-bit
+        // integers: a strip point costs the warp about 50 instructions at W 8 and 60 at W 10 (both components of spin s), a tile
+        // point W^2 shared atomics a component, and the interpolation is 0-8% slower on the narrower tiles of strips.  us of
+        // spreading and interpolation together, tiles / strips, at 1.2 points per cell:
+        //   lmax   spin 0: W 7         W 8          W 9          W 10         spin 2: W 7         W 8
+        //    256     44.6 / 32.5    47.8 / 36.4   52.9 / 38.9   57.5 / 40.2    54.4 / 39.2    64.2 / 45.3
+        //    512     60.9 / 63.0    66.6 / 62.6   74.2 / 68.2   84.8 / 74.4    88.8 / 87.4   103.7 / 89.7
+        //   1024      141 / 207      165 / 193     192 / 212     225 / 236      264 / 302      309 / 296
+        //   2048      511 / 645      597 / 679     734 / 775     867 / 853      998 / 1005    1182 / 1085
+        //   4096     2014 / 2491    2368 / 2609   2931 / 2998   3487 / 3296    4003 / 3909    4772 / 4218
+        // The line suits these to within 5% from lmax 1024 on (lmax 4096 takes W 8, smaller ones W 7).  On smaller grids, and
+        // with a quarter of the points, strips win at W 7 too (spin 2 at lmax 2048 436 / 385): the rule does not look at the
+        // number of points.  Fewer rows per tile where the tiles would not fill the chip
         if ((dd || (prec == LENS_FP32 && (p->W >= (spin ? 8 : 10) || epsilon < 1e-5))) && !p->det) {
             p->strip = true;
             p->tile_c = 33 - p->W;
