@@ -878,8 +878,8 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
         // 1.051e-9 / 1.068e-9; W 16, sigma 1.41 6.52e-12 / 6.71e-12), and such plans, small grids with few points,
         // keep the FP64 transforms
         const auto growth = [](const std::vector<double> &w) {
-            const auto r = std::minmax_element(w.begin(), w.end());
-            return *r.second / *r.first;
+            const auto r = std::minmax_element(w.begin(), w.end(), [](double a, double b) { return fabs(a) < fabs(b); });
+            return fabs(*r.second / *r.first);
         };
         if (p->fft_dd)
             p->fft_dd = 0x1p-41 + growth(w1) * growth(w2) * 0x1p-55 <= 0.25 * exp(-kPi * p->W * sqrt(1.0 - 1.0 / p->sigma));
