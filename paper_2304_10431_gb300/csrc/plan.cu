@@ -872,7 +872,7 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
         }
         // Double-float synthesis transforms only where their rounding stays out of sight of the plan's truncation error
         // (3 exp(-pi W sqrt(1 - 1/sigma)), see support_for).  The deconvolution factors grow from the lowest to the highest mode
-        // by `amp` over both axes; the noise of a synthesis is about 2^-41 + amp 2^-55 of the map.  Up to a twelfth
+        // by `amp` over both axes; the noise of a synthesis is about 2^-41 + amp 2^-55 of the map.  Up to a 24th
         // of the truncation error it does not show (errors with FP64 / double-float transforms at lmax 2048: W 13, sigma 1.64
         // 3.538e-11 / 3.537e-11; W 15, sigma 1.31 2.664e-10 / 2.665e-10); above that it does (W 16, sigma 1.22
         // 1.051e-9 / 1.068e-9; W 16, sigma 1.41 6.52e-12 / 6.71e-12), and such plans, small grids with few points,
@@ -882,7 +882,7 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
             return fabs(*r.second / *r.first);
         };
         if (p->fft_dd)
-            p->fft_dd = 0x1p-41 + growth(w1) * growth(w2) * 0x1p-55 <= 0.25 * exp(-kPi * p->W * sqrt(1.0 - 1.0 / p->sigma));
+            p->fft_dd = 0x1p-41 + growth(w1) * growth(w2) * 0x1p-55 <= 0.125 * exp(-kPi * p->W * sqrt(1.0 - 1.0 / p->sigma));
         if (p->fft_dd) {
             std::vector<float2> f1(w1.size()), f2(w2.size());
             const auto pair = [](double v) { const dfl d(v); return make_float2(d.h, d.l); };
