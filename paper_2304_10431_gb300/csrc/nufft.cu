@@ -347,12 +347,19 @@ cudaError_t launch_prep_points(Plan &p, const double *theta, const double *phi, 
     };
     const int ntc = p.ntile_c;
     const uint64_t nkeys = (uint64_t)((p.R + p.tile_r - 1) / p.tile_r) * ntc;
-    // Sorted within a tile by row where spreading is by strips, which need it, and by row and column for the interpolation
-    // of many points, where the keys fit 32 bits.  Fewer points gain nothing from it (W 7, spin 0 and 2, lmax 128 to 512:
-    // interpolation within 1 us; from W 8 on it shows at 786,000 points: W 9 22.9 -> 21.2 us), and the longer keys cost plan
-    // creation (lmax 128: 1.28 -> 1.44 ms)
+    // Order within a tile, where the keys fit 32 bits.  Strips need rows.  The interpolation gains from rows and columns from 2^17
+    // points on (fewer: within 1 us, and the longer keys cost plan creation, lmax 128 1.28 -> 1.44 ms).  Integer tiles pay for
+    // columns with conflicts of their shared atomics, the more the more points share a cell, so from 3/4 points per cell on
+    // they take rows alone.  us of spreading and interpolation, rows and columns / rows, FP32, spin 2:
+    //   0.5 points per cell (lmax 2048, Nside 1024, W 7)    687 + 314 / 656 + 367
+    //   0.8 (lmax 2048, Nside 1280, W 7)                   1036 + 451 / 963 + 529
+    //   1.1 (lmax 2048, Nside 2048, W 6)                   2210 + 1022 / 1961 + 1170
+    //   4.6 (lmax 1024, Nside 2048, W 6)                   3554 + 952 / 1792 + 995
+    //   18 (lmax 512, Nside 2048, W 6)                     8035 + 927 / 2273 + 917
     const bool fit = nkeys * p.tile_r * p.tile_c <= 0xffffffffull;
-    const int rows = fit && (p.strip || n >= (p.W <= 7 ? 1 << 20 : 1 << 17)) ? 2 : p.strip ? 1 : 0;
+    const bool dense = 4.0 * (double)n >= 3.0 * (0.5 * p.N1) * p.N2;
+    const bool tiles64 = p.prec == LENS_FP64 && p.tile_kmax;  // FP64 interpolation without strips: nothing to gain
+    const int rows = p.strip ? (fit ? 2 : 1) : n >= (1 << 17) && fit && !tiles64 ? (dense ? 1 : 2) : 0;
     const int per = rows == 2 ? p.tile_r * p.tile_c : rows ? p.tile_r : 1;
     k_prep<<<blocks, thr, 0, st>>>(theta, phi, chi, n, p.N1, p.N2, p.W, p.r_lo, p.R, p.pitch, p.spin, scale_of(p.N1),
                                    scale_of(p.N2), p.tile_r, p.tile_c, rows, key, idx, cell_u, frac_u, phase_u, p.flags);
