@@ -17,6 +17,8 @@ constexpr int kLegBlock = 8;         // degrees per unrolled block of the Legend
 constexpr int kTileR = 32, kTileC = 32;  // default grid tile of the point sort (rows x columns)
 constexpr int kMaxW = 16;                 // largest kernel support
 constexpr int grid_pitch(int columns) { return (columns + 31) / 32 * 32; }  // row length of the grid
+// FP32 plans at epsilon >= 1e-5 spread by strips from this W on (plan.cu)
+constexpr int strip_support(bool spin) { return spin ? 8 : 10; }
 // Double-float kernel weights of a point, 4 W FP32 words: the theta taps in pairs (h0, h1, l0, l1), one operand pair of a
 // packed instruction per 8 bytes (an odd W's last one as (h, l)), then the phi taps (h, l).
 __host__ __device__ constexpr int dd_pairs(int W) { return (W + 1) / 2; }
@@ -197,8 +199,10 @@ struct Plan {
     void *phase = nullptr;     // float2 / double2 e^{i s chi}, spin != 0 only
     int tile_c = kTileC;             // columns of a tile: 32; plans that spread by strips 33 - W
     bool strip = false;              // spreading by strips (nufft_strip.cuh)
-    uint32_t strip_part = 0;         // points of a tile that one warp sweeps, and the most such parts of a tile
-    int strip_parts = 1;
+    bool sorted = false;             // points sorted by row within a tile
+    uint32_t strip_part = 0;         // strips: points of a tile that one warp sweeps
+    int parts = 1;                   // the most warps (strips) or CTAs (integer tiles) that share a tile
+    bool piles = false;              // integer tiles: some tile is spread in passes (kPassFrom, nufft.cuh)
     double *wts = nullptr;     // FP64 plans: [npts][2W] kernel weights (theta taps, then phi taps)
     bool wts_dd = false;       // weights as double-float pairs (layout: dd_words); double-float
                                // interpolation and spreading taps (FP64 plans with epsilon >= 5e-11)

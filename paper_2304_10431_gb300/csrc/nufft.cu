@@ -104,12 +104,17 @@ __global__ void k_tile_bounds(const uint32_t *__restrict__ skey, int64_t n, int 
     for (int64_t t = lo + 1; t <= hi; ++t) start[t] = (uint32_t)p;
 }
 
-__global__ void k_tile_most(const uint32_t *__restrict__ start, int ntiles, unsigned *__restrict__ most)
+// most[0]: points of the fullest tile; most[1]: the largest kmax (integer tiles)
+__global__ void k_tile_most(const uint32_t *__restrict__ start, const unsigned short *__restrict__ kmax, int ntiles,
+                            unsigned *__restrict__ most)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned c = t < ntiles ? start[t + 1] - start[t] : 0u;
-    c = __reduce_max_sync(0xffffffffu, c);
-    if ((threadIdx.x & 31) == 0) atomicMax(most, c);
+    const unsigned c = __reduce_max_sync(0xffffffffu, t < ntiles ? start[t + 1] - start[t] : 0u);
+    const unsigned k = __reduce_max_sync(0xffffffffu, t < ntiles && kmax ? (unsigned)kmax[t] : 0u);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(most, c);
+        atomicMax(most + 1, k);
+    }
 }
 
 // FP64 plans' 2W kernel weights of every (sorted) point, computed once, evaluated in FP64 and kept as
@@ -360,6 +365,7 @@ cudaError_t launch_prep_points(Plan &p, const double *theta, const double *phi, 
     const bool dense = 4.0 * (double)n >= 3.0 * (0.5 * p.N1) * p.N2;
     const bool tiles64 = p.prec == LENS_FP64 && p.tile_kmax;  // FP64 interpolation without strips: nothing to gain
     const int rows = p.strip ? (fit ? 2 : 1) : n >= (1 << 17) && fit && !tiles64 ? (dense ? 1 : 2) : 0;
+    p.sorted = rows > 0;
     const int per = rows == 2 ? p.tile_r * p.tile_c : rows ? p.tile_r : 1;
     k_prep<<<blocks, thr, 0, st>>>(theta, phi, chi, n, p.N1, p.N2, p.W, p.r_lo, p.R, p.pitch, p.spin, scale_of(p.N1),
                                    scale_of(p.N2), p.tile_r, p.tile_c, rows, key, idx, cell_u, frac_u, phase_u, p.flags);
@@ -406,21 +412,32 @@ cudaError_t launch_prep_points(Plan &p, const double *theta, const double *phi, 
         k_weights<<<blocks, thr, 0, st>>>((const double2 *)p.frac, n, p.W, p.beta, p.wts, p.wts_dd ? 1 : 0);
         GSL_TRY(cudaGetLastError());
     }
-    if (p.strip) {  // most points of a tile
-        GSL_TRY(cudaMemsetAsync(p.flags + 2, 0, sizeof(unsigned), st));
-        k_tile_most<<<(unsigned)((p.ntiles + thr - 1) / thr), thr, 0, st>>>(p.tile_start, p.ntiles, p.flags + 2);
+    if (!p.det) {
+        GSL_TRY(cudaMemsetAsync(p.flags + 2, 0, 2 * sizeof(unsigned), st));
+        k_tile_most<<<(unsigned)((p.ntiles + thr - 1) / thr), thr, 0, st>>>(p.tile_start, p.tile_kmax, p.ntiles, p.flags + 2);
         GSL_TRY(cudaGetLastError());
     }
-    unsigned hf[3] = {0, 0, 0};
+    unsigned hf[4] = {0, 0, 0, 0};
     GSL_TRY(cudaMemcpyAsync(hf, p.flags, sizeof(hf), cudaMemcpyDeviceToHost, st));
     GSL_TRY(cudaStreamSynchronize(st));
-    const unsigned hflags = hf[0];
-    if (p.strip) {
-        // A warp sweeps at most 4096 points (uniform skies have ~1000 per tile; a tile into which a survey patch
-        // piles its points is shared by up to 64 warps)
+    const unsigned hflags = hf[0], most = p.det ? 0 : hf[2];
+    // Tiles with many points are shared by up to 64 warps or CTAs, more where the grid has few tiles
+    const unsigned share = (unsigned)std::min(std::max((1 << 16) / p.ntiles, 64), 1024);
+    p.parts = 1;
+    if (p.strip && most > 0) {
+        // A warp sweeps at most 4096 points (uniform skies have ~1000 per tile; a survey patch may pile its points into one
+        // tile); fewer, down to one batch of 32, where the points lie in so few tiles that their warps would not fill the chip:
+        // us with parts of 4096 / as now, FP64 W 13 at lmax 128, 49,152 points, spin 0 56 / 36, spin 2 72 / 51; FP32 W 12,
+        // lmax 82, 13,584 points, spin 0 26 / 13
         p.strip_part = 4096;
-        while ((uint64_t)p.strip_part * 64 < hf[2]) p.strip_part *= 2;
-        p.strip_parts = hf[2] ? (int)((hf[2] - 1) / p.strip_part + 1) : 1;
+        if ((uint64_t)most * 152 * 8 > (uint64_t)n)
+            while (p.strip_part > 32 && (uint64_t)p.strip_part * 152 * 16 > 2 * (uint64_t)n) p.strip_part /= 2;
+        while ((uint64_t)p.strip_part * share < most) p.strip_part *= 2;
+        p.parts = (int)((most - 1) / p.strip_part + 1);
+    } else if (p.tile_kmax && hf[3] >= (p.prec == LENS_FP32 ? kPassFrom<float> : kPassFrom<double>)) {
+        const unsigned pass = p.prec == LENS_FP32 ? kPassPoints<float> : kPassPoints<double>;
+        p.piles = true;
+        p.parts = (int)std::min((most - 1) / pass + 1, share);
     }
 #undef GSL_TRY
     cleanup();

@@ -411,8 +411,8 @@ __global__ void __launch_bounds__(256) k_spread_direct(void *__restrict__ grid, 
 // term is rounded once (to 2^-k; FP64: relative 2^-62 of the tile's bound);
 // the flush converts back for one global atomic per non-zero cell.  A map
 // with a non-finite value makes the whole tile NaN.
-// Where kPassFrom or more points reach one cell, the tile is spread and flushed kPassPoints points at a time: tile_kmax holds
-// at most 65535, and the unit would grow with the pile (FP32, a map of one sign, 300,000 points in one cell: 7e-5 of the
+// Where kPassFrom or more points reach one cell, the tile is spread and flushed kPassPoints points at a time, by
+// gridDim.y CTAs in turn: tile_kmax holds at most 65535, and the unit would grow with the pile (FP32, a map of one sign, 300,000 points in one cell: 7e-5 of the
 // a_lm; with the passes 6e-7 at 150,000).  FP32: even skies reach 1024 points only above 20 per cell, where the flush of a
 // pass starts to cost.
 template <typename T> constexpr uint32_t kPassFrom = sizeof(T) == 4 ? 1024 : 65535;
@@ -428,7 +428,9 @@ __device__ __forceinline__ void tile_add(long long *dst, long long v)
     atomicAdd(reinterpret_cast<unsigned long long *>(dst), (unsigned long long)v);  // two's complement sum
 }
 
-template <typename T, int W, bool SPIN, int PRE, bool FX, bool IT = false>
+// PILE: some tile has kPassFrom or more points in a cell (FP32 plans run the variant without passes otherwise: with their loop
+// spin 0, lmax 512, W = 9 took 56.5 us for 53.4).
+template <typename T, int W, bool SPIN, int PRE, bool FX, bool IT = false, bool PILE = sizeof(T) == 8>
 __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThreads) k_spread(void *__restrict__ grid, const uint32_t *__restrict__ cell,
                                                            const cplx<T> *__restrict__ frac,
                                                            const int32_t *__restrict__ perm,
@@ -437,7 +439,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
                                                            int64_t n, int pitch, int R, int ntc,
                                                            const uint32_t *__restrict__ tile_start, T beta,
                                                            const double *__restrict__ fxs,
-                                                           int tile_r, const unsigned short *__restrict__ tile_kmax,
+                                                           int tile_r, int sorted, const unsigned short *__restrict__ tile_kmax,
                                                            const unsigned long long *__restrict__ maxbits,
                                                            const __grid_constant__ KerPoly kp)
 {
@@ -452,21 +454,31 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
     if (p0 == p1) return;
     T sc = FX ? (T)fxs[0] : T(1);
     bool bad = false;  // IT: non-finite map value
-    uint32_t step = p1 - p0;  // points per pass
+    bool pile = false;
     if constexpr (IT) {
         constexpr int kBits = sizeof(T) == 4 ? 30 : 62;  // tile sums of |terms| below 2^kBits
-        const bool pile = tile_kmax[t] >= kPassFrom<T>;
+        pile = PILE && tile_kmax[t] >= kPassFrom<T>;
         const double bound =
             (double)(pile ? kPassPoints<T> : tile_kmax[t]) * __longlong_as_double((long long)*maxbits);
         if (!(bound < 1e300)) bad = true;  // infinity or NaN in the map
         else if (bound > 0.0) sc = (T)ldexp(1.0, kBits - (ilogb(bound) + 1));  // bound < 2^(ilogb+1)
-        if (pile && !bad) step = kPassPoints<T>;
+        pile = pile && !bad;
     }
+    if (PILE && blockIdx.y > 0 && !pile) return;
+    const uint32_t step = pile ? kPassPoints<T> : p1 - p0, stride = pile ? gridDim.y * step : step;  // points per pass
     const int r0 = (t / ntc) * tile_r, c0 = (t % ntc) * kTileC;
-    for (uint32_t pb = p0; pb < p1; pb += step) {
-        const uint32_t pe = min(p1, pb + step);
-        if (pb != p0) __syncthreads();  // the last pass's flush has read the tile
-        for (int i = threadIdx.x; i < TR * TC * NC; i += blockDim.x) buf[i] = G(0);
+    for (uint32_t pb = PILE ? p0 + blockIdx.y * step : p0; pb < p1; pb += stride) {
+        const uint32_t pe = PILE ? min(p1, pb + step) : p1;
+        int lo = 0, hi = TR;  // tile rows to clear and flush: those that the points of this pass reach, if sorted by row
+        if (pile && sorted) {
+            lo = max((int)(cell[pb] / (uint32_t)pitch) - r0, 0);
+            hi = min((int)(cell[pe - 1] / (uint32_t)pitch) - r0 + W, TR);
+        }
+        if (PILE && pb >= p0 + stride) __syncthreads();  // the last pass's flush has read the tile
+        for (int i = lo * TC + threadIdx.x; i < hi * TC; i += blockDim.x) {
+            buf[i] = G(0);
+            if (SPIN) buf[TR * TC + i] = G(0);
+        }
         __syncthreads();
         // (points in sorted order: spin 2, lmax 2048, W = 7: 0.69 ms; a run of points per thread, for fewer of a warp's taps in
         // one bank, 0.77, runs per group of four threads 0.78: the loads then no longer coalesce)
@@ -483,10 +495,10 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
             // IT: the power-of-two unit sc is applied to the point's value first (exact)
             if (!SPIN) {
                 const T x = IT ? map[src] * sc : map[src];
-    #pragma unroll
+#pragma unroll
                 for (int a = 0; a < W; ++a) {
                     const T xa = wa[a] * x;
-    #pragma unroll
+#pragma unroll
                     for (int b = 0; b < W; ++b) {
                         if constexpr (IT) tile_add(b0 + a * TC + b, tile_int(xa * wb[b]));
                         else acc_add<T, FX>(b0 + a * TC + b, xa * wb[b], sc);
@@ -498,10 +510,10 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
                 const T q = map[src], u = map[n + src];
                 T zx = ph.x * q + ph.y * u, zy = ph.x * u - ph.y * q;
                 if constexpr (IT) { zx *= sc; zy *= sc; }
-    #pragma unroll
+#pragma unroll
                 for (int a = 0; a < W; ++a) {
                     const T xa = wa[a] * zx, ya = wa[a] * zy;
-    #pragma unroll
+#pragma unroll
                     for (int b = 0; b < W; ++b) {
                         G *q2 = b0 + (a * TC + b);
                         if constexpr (IT) {
@@ -519,7 +531,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
         if constexpr (IT) {
             T *g = (T *)grid;
             const T inv = bad ? T(NAN) : T(1) / sc;
-            for (int i = threadIdx.x; i < TR * TC; i += blockDim.x) {
+            for (int i = lo * TC + threadIdx.x; i < hi * TC; i += blockDim.x) {
                 const int gr = r0 + i / TC, gc = c0 + i % TC;
                 if (gr >= R || gc >= pitch) continue;
                 const int64_t o = (int64_t)gr * pitch + gc;
@@ -534,7 +546,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
             }
         } else {
             G *g = (G *)grid;
-            for (int i = threadIdx.x; i < TR * TC; i += blockDim.x) {
+            for (int i = lo * TC + threadIdx.x; i < hi * TC; i += blockDim.x) {
                 const int gr = r0 + i / TC, gc = c0 + i % TC;
                 if (gr >= R || gc >= pitch) continue;
                 const int64_t o = (int64_t)gr * pitch + gc;
@@ -580,6 +592,8 @@ cudaError_t interp_w(const Plan &p, const void *grid, void *map, cudaStream_t st
     }
 }
 
+template <bool SPIN> constexpr int kStripW = strip_support(SPIN);
+
 template <typename T, bool SPIN, int W>
 cudaError_t spread_w(const Plan &p, const void *map, void *grid, cudaStream_t st)
 {
@@ -590,9 +604,9 @@ cudaError_t spread_w(const Plan &p, const void *map, void *grid, cudaStream_t st
         const size_t sm = cells * esz;
         cudaError_t e2 = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e2 != cudaSuccess) return e2;
-        kern<<<(unsigned)p.ntiles, sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThreads, sm, st>>>(
+        kern<<<dim3((unsigned)p.ntiles, (unsigned)p.parts), sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThreads, sm, st>>>(
             grid, p.cell, (const cplx<T> *)p.frac, p.perm, (const cplx<T> *)p.phase, p.wts, (const T *)map, p.npts,
-            p.pitch, p.R, p.ntile_c, p.tile_start, (T)p.beta, fxs, p.tile_r, p.tile_kmax, p.maxbits, p.kpoly);
+            p.pitch, p.R, p.ntile_c, p.tile_start, (T)p.beta, fxs, p.tile_r, p.sorted ? 1 : 0, p.tile_kmax, p.maxbits, p.kpoly);
         return cudaGetLastError();
     };
     if constexpr (std::is_same<T, double>::value) {
@@ -613,8 +627,10 @@ cudaError_t spread_w(const Plan &p, const void *map, void *grid, cudaStream_t st
         return direct(k_spread_direct<T, W, SPIN, 0>);
     } else {
         if (p.det) return run(k_spread<T, W, SPIN, 0, true>, 8);
-        if (!p.strip) return run(k_spread<T, W, SPIN, 0, false, true>, 4);
-        return spread_strip32<W, SPIN>(p, map, grid, st);
+        if (p.strip) return spread_strip32<W, SPIN>(p, map, grid, st);
+        if constexpr (W < kStripW<SPIN>)
+            return p.piles ? run(k_spread<T, W, SPIN, 0, false, true, true>, 4) : run(k_spread<T, W, SPIN, 0, false, true, false>, 4);
+        else return cudaErrorInvalidValue;  // such plans spread by strips
     }
 }
 

@@ -355,7 +355,7 @@ k_spread_strip32(float *__restrict__ grid, const uint32_t *__restrict__ cell, co
 
 inline dim3 strip_grid(const Plan &p)
 {
-    return dim3((unsigned)((p.ntiles + kStripWarps - 1) / kStripWarps), (unsigned)p.strip_parts);
+    return dim3((unsigned)((p.ntiles + kStripWarps - 1) / kStripWarps), (unsigned)p.parts);
 }
 
 template <int W, bool SPIN> cudaError_t spread_strip(const Plan &p, const void *map, void *grid, cudaStream_t st)

@@ -765,7 +765,7 @@ int lens_plan_create_ex(lens_plan *out, int lmax, int mmax, int spin, int64_t np
         // The line suits these to within 5% from lmax 1024 on (lmax 4096 takes W 8, smaller ones W 7).  On smaller grids, and
         // with a quarter of the points, strips win at W 7 too (spin 2 at lmax 2048 436 / 385): the rule does not look at the
         // number of points.  Fewer rows per tile where the tiles would not fill the chip
-        if ((dd || (prec == LENS_FP32 && (p->W >= (spin ? 8 : 10) || epsilon < 1e-5))) && !p->det) {
+        if ((dd || (prec == LENS_FP32 && (p->W >= strip_support(spin != 0) || epsilon < 1e-5))) && !p->det) {
             p->strip = true;
             p->tile_c = 33 - p->W;
             p->ntile_c = (p->N2 + p->tile_c - 1) / p->tile_c;

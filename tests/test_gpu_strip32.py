@@ -1,9 +1,9 @@
 """FP32 spreading by strips (csrc/nufft_strip.cuh, k_spread_strip32) at every kernel support, and tiles that several warps
-share (more than 4096 points) in both precisions.
+share in both precisions.
 
 The deterministic plan of the same geometry, kernel and later stages adds the same FP32 taps as 64-bit integers, so the two
 adjoints differ by the strips' running FP32 sums alone: about sqrt(n / 3) 2^-25 of a sum of n terms of one sign, 1.6e-6 for
-the 8192 points that a warp sweeps at most here, below the plans' epsilon of 5e-6.  FP64: the 2e-12 of
+8192 points of a warp, more than any sweeps here, below the plans' epsilon of 5e-6.  FP64: the 2e-12 of
 tests/test_gpu_strip.py.  Below epsilon 1e-5 every W spreads by strips; at 1e-5 W >= 10 does for every spin.
 """
 import numpy as np
@@ -44,7 +44,7 @@ def test_adjoint_equals_deterministic(w, spin, n):
 @pytest.mark.parametrize("precision,w,eps,tol", [("fp32", 5, 5e-6, 5e-6), ("fp32", 8, 5e-6, 5e-6), ("fp32", 13, 1e-5, 5e-6),
                                                  ("fp64", 8, 1e-6, 2e-12), ("fp64", 13, 1e-6, 2e-12)])
 @pytest.mark.parametrize("spin", [0, 2])
-@pytest.mark.parametrize("n", [4095, 4097, 5003, 300007])  # parts of 4096 points, of 8192 from 262145 on
+@pytest.mark.parametrize("n", [4095, 4097, 5003, 300007])  # few parts, and more points than the parts of 128 hold
 @pytest.mark.parametrize("spread", [1e-4, 0.05])  # one cell; rows and columns of a tile
 def test_tiles_shared_by_warps(precision, w, eps, tol, spin, n, spread):
     th, ph, _ = W.random_points(n, 7)
