@@ -36,7 +36,16 @@ __device__ __forceinline__ dfl operator*(dfl a, dfl b) { return to_dfl(df_mul(to
 __device__ __forceinline__ dfl operator*(float f, dfl a) { return {f * a.h, f * a.l}; }  // f a power of two, +-
 __device__ __forceinline__ dfl operator*(dfl a, float f) { return f * a; }
 __device__ __forceinline__ dfl operator*(int f, dfl a) { return (float)f * a; }
-__device__ __forceinline__ dfl dfl_fma(dfl a, dfl b, dfl c) { return to_dfl(df_fma(to_df(a), to_df(b), to_df(c))); }
+// a b + c, as df_fma of common.cuh
+__device__ __forceinline__ dfl dfl_fma(dfl a, dfl b, dfl c)
+{
+    const float s = __fadd_rn(c.h, __fmul_rn(a.h, b.h));
+    const float bb = __fsub_rn(s, c.h);
+    const float ec = __fsub_rn(c.h, __fsub_rn(s, bb));
+    const float ep = __fmaf_rn(a.h, b.h, -bb);
+    const float lo = __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, c.l));
+    return {s, __fadd_rn(lo, __fadd_rn(ec, ep))};
+}
 __device__ __forceinline__ dfl2 mkc(dfl r, dfl i) { return {r, i}; }
 __device__ __forceinline__ dfl2 cadd(dfl2 a, dfl2 b) { return {a.x + b.x, a.y + b.y}; }
 __device__ __forceinline__ dfl2 csub(dfl2 a, dfl2 b) { return {a.x - b.x, a.y - b.y}; }

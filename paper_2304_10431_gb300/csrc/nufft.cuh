@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kInterpDD, 4) k_interp_dd(const void *__restri
     // phi weights; an odd W's first one shares its 16 bytes with the last theta weight
     constexpr int O = W & 1;
     df32 wb[W];
-    const float4 mid = w[W / 2];
+    const float4 mid = O ? w[W / 2] : make_float4(0.f, 0.f, 0.f, 0.f);
     if (O) wb[0] = {mid.z, mid.w};
 #pragma unroll
     for (int i = 0; i < W / 2; ++i) {
@@ -428,8 +428,8 @@ __device__ __forceinline__ void tile_add(long long *dst, long long v)
     atomicAdd(reinterpret_cast<unsigned long long *>(dst), (unsigned long long)v);  // two's complement sum
 }
 
-// PILE: some tile has kPassFrom or more points in a cell (FP32 plans run the variant without passes otherwise: with their loop
-// spin 0, lmax 512, W = 9 took 56.5 us for 53.4).
+// PILE: some tile has kPassFrom or more points in a cell (FP32 plans run the variant without passes otherwise: with a loop of
+// passes around the body spin 0, lmax 512, W = 9 took 56.5 us for 53.4).
 template <typename T, int W, bool SPIN, int PRE, bool FX, bool IT = false, bool PILE = sizeof(T) == 8>
 __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThreads) k_spread(void *__restrict__ grid, const uint32_t *__restrict__ cell,
                                                            const cplx<T> *__restrict__ frac,
@@ -465,16 +465,9 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
         pile = pile && !bad;
     }
     if (PILE && blockIdx.y > 0 && !pile) return;
-    const uint32_t step = pile ? kPassPoints<T> : p1 - p0, stride = pile ? gridDim.y * step : step;  // points per pass
     const int r0 = (t / ntc) * tile_r, c0 = (t % ntc) * kTileC;
-    for (uint32_t pb = PILE ? p0 + blockIdx.y * step : p0; pb < p1; pb += stride) {
-        const uint32_t pe = PILE ? min(p1, pb + step) : p1;
-        int lo = 0, hi = TR;  // tile rows to clear and flush: those that the points of this pass reach, if sorted by row
-        if (pile && sorted) {
-            lo = max((int)(cell[pb] / (uint32_t)pitch) - r0, 0);
-            hi = min((int)(cell[pe - 1] / (uint32_t)pitch) - r0 + W, TR);
-        }
-        if (PILE && pb >= p0 + stride) __syncthreads();  // the last pass's flush has read the tile
+    // points pb .. pe - 1, which reach the tile rows lo .. hi - 1
+    const auto pass = [&](uint32_t pb, uint32_t pe, int lo, int hi) {
         for (int i = lo * TC + threadIdx.x; i < hi * TC; i += blockDim.x) {
             buf[i] = G(0);
             if (SPIN) buf[TR * TC + i] = G(0);
@@ -560,6 +553,21 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kSpreadThreads64 : kSpreadThr
                 }
             }
         }
+    };
+    if (!PILE || !pile) {
+        pass(p0, p1, 0, TR);
+        return;
+    }
+    constexpr uint32_t step = kPassPoints<T>;
+    for (uint32_t pb = p0 + blockIdx.y * step; pb < p1; pb += gridDim.y * step) {
+        const uint32_t pe = min(p1, pb + step);
+        int lo = 0, hi = TR;
+        if (sorted) {
+            lo = max((int)(cell[pb] / (uint32_t)pitch) - r0, 0);
+            hi = min((int)(cell[pe - 1] / (uint32_t)pitch) - r0 + W, TR);
+        }
+        pass(pb, pe, lo, hi);
+        __syncthreads();  // the next pass clears the tile
     }
 }
 
